@@ -436,7 +436,7 @@ lhe_status lhe_lbm_create(const lhe_lbm_params *p, lhe_lbm **out) {
     }
   }
   l->red_blocks = 152 * 4;
-  cudaError_t e = cudaMalloc(&l->red_partials, sizeof(double) * 4 * (size_t)l->red_blocks + sizeof(double) * 4);
+  cudaError_t e = cudaMalloc(&l->red_partials, sizeof(double) * (4 * (size_t)l->red_blocks + 5));
   if (e != cudaSuccess) return bail(cuda_fail(l, e, "cudaMalloc(reduction scratch)"));
   l->red_out = l->red_partials + 4 * (size_t)l->red_blocks;
   if (p->bc != LHE_BC_PERIODIC) {
@@ -1214,16 +1214,22 @@ lhe_status lhe_lbm_diagnostics(lhe_lbm *l, double *out_host) {
   if (!out_host) return fail(l, LHE_ERR_ARG, "out_host is NULL");
   if (!l->initialised) return fail(l, LHE_ERR_STATE, "lhe_lbm_diagnostics before lhe_lbm_init");
   if (lhe_status st = unscale(l, 0)) return st;
+  if (!l->red_done) {  // the block counter, zeroed once on the stream of the first call (every call drains its stream)
+    unsigned *done = reinterpret_cast<unsigned *>(l->red_out + 4);
+    LHE_CK(l, cudaMemsetAsync(done, 0, sizeof(unsigned), l->stream));
+    l->red_done = done;
+  }
   ReduceArgs a{};
   a.g = l->g;
   a.pop = l->pop[l->cur];
   a.phi = l->phi[l->cur];
   a.Rfield = l->Rfield;
-  for (int k = 0; k < l->Q; ++k) a.omega[k] = l->omega[k];
+  a.c = diag_coef(l->Q, l->omega, l->s);
   a.s = l->s;
   a.dt = l->dt;
   a.dtR = l->dt * l->R;
   a.partials = l->red_partials;
+  a.done = l->red_done;
   a.out = l->red_out;
   LHE_CK(l, launch_reduce(l->p.d, l->p.precision == LHE_FP32_DEV, a, l->red_blocks, l->stream));
   LHE_CK(l, cudaMemcpyAsync(out_host, l->red_out, sizeof(double) * 4, cudaMemcpyDeviceToHost, l->stream));

@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "lhe_device.cuh"
+#include "lhe_diag.cuh"
 #include "lhe_lbm.h"
 
 namespace lhe {
@@ -165,9 +166,10 @@ struct ReduceArgs {
   const void *pop;
   const float2 *phi;       // FP32_DEV
   const double *Rfield;
-  double omega[kMaxQ];
+  DiagCoef c;
   double s, dt, dtR;
   double *partials;        // gridDim.x * 4
+  unsigned *done;          // blocks that have written their partials (0 between launches)
   double *out;             // 4 (device)
 };
 
@@ -312,6 +314,7 @@ struct lhe_lbm {
   // diagnostics
   double *red_partials = nullptr;
   double *red_out = nullptr;
+  unsigned *red_done = nullptr;
   int red_blocks = 0;
   std::string err;
 };

@@ -1,5 +1,7 @@
 // lhe_misc.cu -- initialisation, finite-difference gradient, diagnostics reduction and the
 // adjoint seed / gradient kernels.
+#include <algorithm>
+
 #include "lhe_diag.cuh"
 #include "lhe_internal.h"
 #include "lhe_sites.cuh"
@@ -129,58 +131,61 @@ cudaError_t launch_fd_grad_transpose_add(int d, const Geom &g, double dx, const 
 // Per site: phi (from the post-collision state: sum_k f*_k - dt R), the pre-collision populations
 // recovered from f* = (1-s) f + omega (s phi + dt R) (s != 1; for s = 1 the post-collision values
 // are used), the kinetic entropy sum_k f_k^2 / (2 omega_k) (Eq. (skfk)), |phi| and non-finite
-// values. Block partials go to a scratch array; a second single-block pass adds them in a fixed
+// values. Block partials go to a scratch array; the block that finishes last adds them in block
 // order, so the result does not depend on scheduling.
 template <int D, bool DEV>
-__global__ void __launch_bounds__(256) k_reduce_partials(const ReduceArgs a) {
+__global__ void __launch_bounds__(256) k_reduce(const ReduceArgs a) {
   constexpr int Q = Lattice<D>::Q;
   __shared__ double sh[8 * 4];
+  __shared__ bool last;
   const int64_t S = a.g.S;
   double v[4] = {0.0, 0.0, 0.0, 0.0};
-  const bool recover = a.s != 1.0;
   for (int64_t site = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; site < S;
        site += (int64_t)gridDim.x * blockDim.x) {
     const double dtR = a.Rfield ? a.dt * a.Rfield[site] : a.dtR;
     if (DEV) {
-      double phi, ent = 0.0, bad = 0.0;
-      const float *g = static_cast<const float *>(a.pop);
-      phi = df_value(a.phi[site]);
-      if (!isfinite(phi)) bad += 1.0;
-      ent = 0.5 * phi * phi;  // sum_k f_k^2/(2 w_k) = phi^2/2 + sum_k g_k^2/(2 w_k) since sum_k g_k = 0
+      // sum_k f_k^2/(2 w_k) = phi^2/2 + sum_k g_k^2/(2 w_k) since sum_k g_k = 0
+      const float *__restrict__ g = static_cast<const float *>(a.pop);
+      const double phi = df_value(a.phi[site]);
+      const double rdtR = a.s != 1.0 ? dtR : 0.0;
+      int bad = nonfinite_bits(phi) ? 1 : 0;
+      double ent = 0.0;
+#pragma unroll
       for (int k = 0; k < Q; ++k) {
-        const double gs = (double)g[k * S + site];
-        if (!isfinite(gs)) bad += 1.0;
-        const double gk = recover ? (gs - a.omega[k] * dtR) / (1.0 - a.s) : gs;
-        ent += gk * gk / (2.0 * a.omega[k]);
+        const double gs = (double)__ldg(g + k * S + site);
+        bad += nonfinite_bits(gs) ? 1 : 0;
+        const double d = fma(-a.c.omega[k], rdtR, gs);
+        ent = fma(d * d, a.c.iw[k], ent);
       }
       v[0] += phi;
-      v[1] += ent;
+      v[1] += fma(ent, a.c.inv2, 0.5 * phi * phi);
       v[2] = fmax(v[2], fabs(phi));
-      v[3] += bad;
+      v[3] += (double)bad;
     } else {
-      diag_site_fp64(static_cast<const double *>(a.pop), S, site, Q, a.omega, a.s, recover, dtR, v);
+      diag_site_fp64<Q>(static_cast<const double *>(a.pop), S, site, a.c, a.s, dtR, v);
     }
   }
   block_reduce4(v, sh);
-  if (threadIdx.x == 0)
+  if (threadIdx.x == 0) {
     for (int j = 0; j < 4; ++j) a.partials[blockIdx.x * 4 + j] = v[j];
-}
-
-__global__ void __launch_bounds__(256) k_reduce_final(const double *__restrict__ partials, int nblocks,
-                                                      double *__restrict__ out) {
-  __shared__ double sh[8 * 4];
-  reduce_partials_final(partials, nblocks, out, sh);
+    __threadfence();
+    last = atomicInc(a.done, gridDim.x - 1) == gridDim.x - 1;  // wraps to 0 for the next launch
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  reduce_partials_final(a.partials, (int)gridDim.x, a.out, sh);
 }
 
 template <int D>
 static cudaError_t reduce_d(bool dev, const ReduceArgs &a, int nblocks, cudaStream_t st) {
-  if (dev) k_reduce_partials<D, true><<<nblocks, 256, 0, st>>>(a);
-  else k_reduce_partials<D, false><<<nblocks, 256, 0, st>>>(a);
-  k_reduce_final<<<1, 256, 0, st>>>(a.partials, nblocks, a.out);
+  if (dev) k_reduce<D, true><<<nblocks, 256, 0, st>>>(a);
+  else k_reduce<D, false><<<nblocks, 256, 0, st>>>(a);
   return cudaGetLastError();
 }
 
 cudaError_t launch_reduce(int d, bool dev, const ReduceArgs &a, int nblocks, cudaStream_t st) {
+  nblocks = (int)std::min<int64_t>(nblocks, (a.g.S + 255) / 256);
   switch (d) {
     case 1: return reduce_d<1>(dev, a, nblocks, st);
     case 2: return reduce_d<2>(dev, a, nblocks, st);

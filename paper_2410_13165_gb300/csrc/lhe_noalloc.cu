@@ -31,23 +31,22 @@ constexpr int64_t kNoAllocMaxSites = int64_t(1) << 28;  // 268,435,456 nodes: th
 
 struct NoAllocArgs {
   int64_t S;
-  int32_t Q;
   const double *pop;
   const double *Rfield;
-  double omega[kMaxQ];
+  DiagCoef c;
   double s, dt, dtR;
 };
 
 // Grid-stride over the nodes; block b overwrites its own four partials, so nothing in the scratch
 // array has to be cleared first. The per-node formula is diag_site_fp64, as in the handle's kernel.
+template <int D>
 __global__ void __launch_bounds__(kNoAllocThreads) k_noalloc_partials(const NoAllocArgs a, double *partials) {
   __shared__ double sh[(kNoAllocThreads / 32) * 4];
-  const bool recover = a.s != 1.0;
   double v[4] = {0.0, 0.0, 0.0, 0.0};
   for (int64_t site = (int64_t)blockIdx.x * kNoAllocThreads + threadIdx.x; site < a.S;
        site += (int64_t)gridDim.x * kNoAllocThreads) {
     const double dtR = a.Rfield ? a.dt * a.Rfield[site] : a.dtR;
-    diag_site_fp64(a.pop, a.S, site, a.Q, a.omega, a.s, recover, dtR, v);
+    diag_site_fp64<Lattice<D>::Q>(a.pop, a.S, site, a.c, a.s, dtR, v);
   }
   block_reduce4(v, sh);
   if (threadIdx.x == 0)
@@ -155,11 +154,10 @@ extern "C" LHE_API lhe_status lhe_lbm_diagnostics_noalloc(const lhe_lbm_params *
                                           cudaGetErrorString(se));
   NoAllocArgs a{};
   a.S = S;
-  a.Q = Q;
   a.pop = pop_dev;
   a.Rfield = R_dev;
-  for (int k = 0; k < Q; ++k) a.omega[k] = omega[k];
   a.s = 1.0 / p->tau;
+  a.c = diag_coef(Q, omega, a.s);
   // dt = dx / c with dx from the first dimension (lhe_lbm_model has checked that dx agrees in all).
   const double span = (p->bc == LHE_BC_FULLWAY) ? (double)(p->n[0] - 1) : (double)p->n[0];
   a.dt = (p->hi[0] - p->lo[0]) / span / p->c;
@@ -169,7 +167,13 @@ extern "C" LHE_API lhe_status lhe_lbm_diagnostics_noalloc(const lhe_lbm_params *
   nb = std::max<int64_t>(1, std::min<int64_t>(nb, kNoAllocMaxBlocks));
   const int nblocks = (int)nb;
   cudaStream_t stream = static_cast<cudaStream_t>(p->stream);
-  k_noalloc_partials<<<nblocks, kNoAllocThreads, 0, stream>>>(a, scratch);
+  switch (p->d) {
+    case 1: k_noalloc_partials<1><<<nblocks, kNoAllocThreads, 0, stream>>>(a, scratch); break;
+    case 2: k_noalloc_partials<2><<<nblocks, kNoAllocThreads, 0, stream>>>(a, scratch); break;
+    case 3: k_noalloc_partials<3><<<nblocks, kNoAllocThreads, 0, stream>>>(a, scratch); break;
+    case 4: k_noalloc_partials<4><<<nblocks, kNoAllocThreads, 0, stream>>>(a, scratch); break;
+    default: k_noalloc_partials<5><<<nblocks, kNoAllocThreads, 0, stream>>>(a, scratch); break;
+  }
   k_noalloc_final<<<1, kNoAllocThreads, 0, stream>>>(scratch, nblocks, out_dev);
   const cudaError_t le = cudaGetLastError();
   if (le != cudaSuccess) return record_error(LHE_ERR_CUDA, std::string("diagnostics launch: ") + cudaGetErrorString(le));
