@@ -702,32 +702,41 @@ lhe_status lhe_lbm_init(lhe_lbm *l, const double *phi0, const double *grad, cons
     LHE_CK(l, cudaFree(l->Rfield));
     l->Rfield = nullptr;
   }
-  const double *gptr = grad;
-  l->grad_was_fd = false;
-  if (!grad && l->p.init_order == 3) {
-    if (!l->fdgrad) LHE_CK(l, cudaMalloc(&l->fdgrad, sizeof(double) * S * d));
-    LHE_CK(l, launch_fd_grad(d, l->g, l->dx, phi0, l->fdgrad, l->stream));
-    gptr = l->fdgrad;
-    l->grad_was_fd = true;
-  }
+  l->grad_was_fd = !grad && l->p.init_order == 3;
   InitArgs a{};
   a.g = l->g;
   a.phi0 = phi0;
-  a.grad = gptr;
+  a.grad = grad;
   a.Rfield = l->Rfield;
   a.dst = l->pop[0];
   a.phi_dst = l->phi[0];
+  const auto pair = [](double v) {
+    const float h = (float)v;
+    return make_float2(h, (float)(v - (double)h));
+  };
+  const double w = (1.0 - l->s) * 0.5 * l->dt / (l->grad_was_fd ? 12.0 * l->dx : 1.0);
+  a.wc = w * l->p.c;
+  a.wc_f = pair(a.wc);
+  const auto in_range = [](double v) { return v == 0.0 || (std::fabs(v) >= 0x1p-40 && std::fabs(v) <= 0x1p20); };
+  a.pairs = in_range(a.wc);
+  for (int i = 0; i < d; ++i) {
+    a.wu[i] = w * l->p.u[i];
+    a.pairs = a.pairs && in_range(a.wu[i]);
+    a.wu_f[i] = pair(a.wu[i]);
+    a.werr += (float)std::fabs(a.wu[i]);
+    a.u[i] = l->p.u[i];
+  }
+  a.werr += (float)std::fabs(a.wc);
   for (int k = 0; k < l->Q; ++k) {
     a.omega[k] = l->omega[k];
+    a.omega_f[k] = pair(l->omega[k]);
     a.c1[k] = (1.0 - l->s) * 0.5 * l->dt * l->omega[k];
     a.c2[k] = l->p.c * a.c1[k];
+    for (int i = 0; i < d; ++i) a.e[k][i] = (int8_t)l->e[k * d + i];
   }
-  a.s = l->s;
-  a.oms = 1.0 - l->s;
+  a.inv12dx = 1.0 / (12.0 * l->dx);
   a.dt = l->dt;
   a.dtR = l->dt * l->R;
-  a.c = l->p.c;
-  for (int i = 0; i < d; ++i) a.u[i] = l->p.u[i];
   a.order = l->p.init_order;
   l->init_order_used = l->p.init_order;
   LHE_CK(l, launch_init(d, l->p.precision == LHE_FP32_DEV, a, l->stream));

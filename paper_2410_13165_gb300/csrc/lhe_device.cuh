@@ -99,32 +99,40 @@ __host__ __device__ constexpr int ceil_log2(int q) {
 // the Q-1 additions of the moment sum (and the conversion) off the FP64 pipe.
 // Subnormal terms are placed as if their exponent were 0 instead of 1 (an error below 2^-1022 in
 // absolute value); any NaN or infinite term makes the result NaN.
-template <int Q, int P2, class Get>
-__device__ __forceinline__ double fixed_moment_sum_impl(Get f) {
-  constexpr int G = 10 - ceil_log2(Q);
-  static_assert(G >= 3, "too many terms for a 64-bit accumulator");
-  unsigned emf = 0u;  // largest exponent field, in place (bits 20..30 of the high word)
-#pragma unroll
-  for (int k = 0; k < Q; ++k) emf = max(emf, (unsigned)__double2hiint(f(k)) & 0x7FF00000u);
-  if (emf == 0x7FF00000u) return __longlong_as_double(0x7FF8000000000000ll);
-  emf = max(emf, 0x00100000u);
-  long long acc = 0;
-#pragma unroll
-  for (int k = 0; k < Q; ++k) {
-    const double fk = f(k);
-    const unsigned hi = (unsigned)__double2hiint(fk);
-    const unsigned lo = (unsigned)__double2loint(fk);
-    const unsigned ef = hi & 0x7FF00000u;
-    const unsigned mh = (hi & 0x000FFFFFu) | min(ef, 0x00100000u);  // implicit bit unless zero/subnormal
-    const unsigned sh = (emf - max(ef, 0x00100000u)) >> 20;
-    const unsigned long long m = ((((unsigned long long)mh) << 32) | lo) << G;  // < 2^(53+G)
-    unsigned long long v;
-    if (sh < 32u) v = (m + ((1ull << sh) >> 1)) >> sh;
-    else if (sh < 64u) v = (m + (1ull << (sh - 1))) >> sh;
-    else v = 0ull;
-    const long long sg = (long long)((int)hi >> 31);  // 0 or -1
-    acc += ((long long)v ^ sg) - sg;
-  }
+constexpr unsigned kExpField = 0x7FF00000u;  // exponent field in the high word of a double
+
+// One term in the frame of the largest exponent field emf (in place, at least 0x00100000) with G guard bits.
+template <int G>
+__device__ __forceinline__ long long fixed_align(double f, unsigned emf) {
+  const unsigned hi = (unsigned)__double2hiint(f);
+  const unsigned lo = (unsigned)__double2loint(f);
+  const unsigned ef = hi & kExpField;
+  const unsigned mh = (hi & 0x000FFFFFu) | min(ef, 0x00100000u);  // implicit bit unless zero/subnormal
+  const unsigned sh = (emf - max(ef, 0x00100000u)) >> 20;
+  const unsigned long long m = ((((unsigned long long)mh) << 32) | lo) << G;  // < 2^(53+G)
+  unsigned long long v;
+  if (sh < 32u) v = (m + ((1ull << sh) >> 1)) >> sh;
+  else if (sh < 64u) v = (m + (1ull << (sh - 1))) >> sh;
+  else v = 0ull;
+  const long long sg = (long long)((int)hi >> 31);  // 0 or -1
+  return ((long long)v ^ sg) - sg;
+}
+
+// fixed_align of the double of a float; emaxf: largest exponent field of the floats (0 .. 254; the frame of the
+// doubles is emf = (max(emaxf, 1) + 896) << 20). Truncates toward zero below the frame (2^-(53+G) of the largest).
+template <int G>
+__device__ __forceinline__ long long fixed_align(float f, unsigned emaxf) {
+  const unsigned b = (unsigned)__float_as_int(f), e = (b >> 23) & 0xFFu;
+  const unsigned m = (b & 0x007FFFFFu) | (e ? 0x00800000u : 0u);
+  const unsigned sh = max(emaxf, 1u) - max(e, 1u);
+  const unsigned long long v = sh < 64u ? ((unsigned long long)m << (29 + G)) >> sh : 0ull;
+  const long long sg = (long long)((int)b >> 31);
+  return ((long long)v ^ sg) - sg;
+}
+
+// The value of a total acc in that frame, correctly rounded (ties to even), times 2^P2.
+template <int G, int P2>
+__device__ __forceinline__ double fixed_value(long long acc, unsigned emf) {
   if (acc == 0) return 0.0;
   const unsigned long long sbit = acc < 0 ? 0x8000000000000000ull : 0ull;
   unsigned long long a = acc < 0 ? (unsigned long long)(-acc) : (unsigned long long)acc;
@@ -144,6 +152,21 @@ __device__ __forceinline__ double fixed_moment_sum_impl(Get f) {
     return __ll2double_rn(acc) * pow2_bits(p1) * pow2_bits(p - p1);
   }
   return __longlong_as_double((long long)(sbit | ((unsigned long long)ex << 52) | (mant & 0xFFFFFFFFFFFFFull)));
+}
+
+template <int Q, int P2, class Get>
+__device__ __forceinline__ double fixed_moment_sum_impl(Get f) {
+  constexpr int G = 10 - ceil_log2(Q);
+  static_assert(G >= 3, "too many terms for a 64-bit accumulator");
+  unsigned emf = 0u;  // largest exponent field, in place (bits 20..30 of the high word)
+#pragma unroll
+  for (int k = 0; k < Q; ++k) emf = max(emf, (unsigned)__double2hiint(f(k)) & kExpField);
+  if (emf == kExpField) return __longlong_as_double(0x7FF8000000000000ll);
+  emf = max(emf, 0x00100000u);
+  long long acc = 0;
+#pragma unroll
+  for (int k = 0; k < Q; ++k) acc += fixed_align<G>(f(k), emf);
+  return fixed_value<G, P2>(acc, emf);
 }
 
 template <int Q, int P2>
@@ -194,6 +217,57 @@ __device__ __forceinline__ float2 df_add(float h, float t) {
   const bool away = (s > 0.0f && e < 0.0f) || (s < 0.0f && e > 0.0f);
   const float hn = away ? __int_as_float(__float_as_int(s) - 1) : s;
   return make_float2(hn, __fadd_rn(__fsub_rn(s, hn), e));
+}
+
+// The double of a float, by its bits (FP32 -> FP64 conversions retire at the FP64 pipe's ~2 per clock per SM);
+// subnormals are scaled by 2^64 first. Branch-free: a branch to the conversion would be predicated, and a
+// predicated conversion costs as much as one that runs.
+__device__ __forceinline__ double float_to_double(float f) {
+  const bool tiny = ((unsigned)__float_as_int(f) & 0x7F800000u) == 0u;
+  const unsigned b = (unsigned)__float_as_int(tiny ? __fmul_rn(f, 0x1p64f) : f), mag = b & 0x7FFFFFFFu;
+  const unsigned bias = tiny ? 0x34000000u : (mag >= 0x7F800000u ? 0x70000000u : 0x38000000u);
+  const unsigned hi = mag == 0u ? 0u : (mag >> 3) + bias;
+  return __hiloint2double((int)((b & 0x80000000u) | hi), (int)(b << 29));
+}
+
+// Arithmetic on unevaluated pairs h + l of floats (Dekker, "A floating-point technique for extending the
+// available precision", Numer. Math. 18, 1971; Knuth's TwoSum): ~2^-46 of the operands, on the FP32
+// pipe, which runs 64 times the FP64 pipe's rate here. The intrinsics keep the compiler from contracting.
+__device__ __forceinline__ float2 ff_quick(float a, float b) {  // |a| >= |b| or a = 0
+  const float s = __fadd_rn(a, b);
+  return make_float2(s, __fsub_rn(b, __fsub_rn(s, a)));
+}
+
+__device__ __forceinline__ float2 ff_add(float2 a, float2 b) {
+  const float s = __fadd_rn(a.x, b.x);
+  const float bp = __fsub_rn(s, a.x);
+  const float e = __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, bp)), __fsub_rn(b.x, bp));
+  return ff_quick(s, __fadd_rn(e, __fadd_rn(a.y, b.y)));
+}
+
+__device__ __forceinline__ float2 ff_neg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 ff_sub(float2 a, float2 b) { return ff_add(a, ff_neg(b)); }
+
+__device__ __forceinline__ float2 ff_mul(float2 a, float2 b) {
+  const float p = __fmul_rn(a.x, b.x);
+  const float e = __fmaf_rn(a.x, b.x, -p);
+  return ff_quick(p, __fmaf_rn(a.x, b.y, __fmaf_rn(a.y, b.x, e)));
+}
+
+// Exponent of a double: 2^E <= |x| < 2^(E+1); -1023 for zero and subnormals, 1024 for infinities and NaN.
+__device__ __forceinline__ int double_exponent(double x) { return (int)(((unsigned)__double2hiint(x) & kExpField) >> 20) - 1023; }
+
+// df_split by integer operations, for E = double_exponent(x) <= 126: h the value truncated to 24 bits, l the rest
+// rounded to nearest. Below 2^-70 the low part and below 2^-126 the whole value is taken as zero.
+__device__ __forceinline__ float2 ff_split(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int E = (int)((hi & kExpField) >> 20) - 1023;
+  if (E < -126) return make_float2(0.0f, 0.0f);
+  const unsigned sign = hi & 0x80000000u;
+  const float h = __int_as_float((int)(sign | ((unsigned)(E + 127) << 23) | ((hi & 0x000FFFFFu) << 3) | (lo >> 29)));
+  const float r = (float)(lo & 0x1FFFFFFFu);
+  const float sc = E >= -70 ? __int_as_float((int)(sign | ((unsigned)(E - 52 + 127) << 23))) : 0.0f;
+  return make_float2(h, __fmul_rn(r, sc));
 }
 
 // Stores of the new state with the default cache policy. The evict-first hint (st.global.cs) was

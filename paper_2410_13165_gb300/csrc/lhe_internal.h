@@ -149,15 +149,25 @@ struct BoundaryArgs {
 struct InitArgs {
   Geom g;
   const double *phi0;
-  const double *grad;      // d*S (may be the library's FD buffer)
+  const double *grad;      // d*S, or nullptr: finite differences of phi0 (order 3)
   const double *Rfield;
   void *dst;
   float2 *phi_dst;
   double omega[kMaxQ];
+  float2 omega_f[kMaxQ];   // FP32_DEV: the same as float pairs
+  // weights of the gradient in B and h (lhe_misc.cu): (1 - s)(dt/2) u_i and (1 - s)(dt/2) c, over 12 dx
+  // when the kernel forms the differences itself (grad == nullptr)
+  double wu[kMaxD], wc;
+  float2 wu_f[kMaxD], wc_f;
+  float werr;              // |wc| + sum_i |wu_i|
+  int32_t pairs;           // the weights lie well inside the range of float pairs
+  // the FP64 form of one population (lhe_misc.cu deviation_fp64)
   double c1[kMaxQ];        // (1 - s)(dt/2) omega_k
   double c2[kMaxQ];        // c (1 - s)(dt/2) omega_k
-  double s, oms, dt, dtR, c;
   double u[kMaxD];
+  double inv12dx;
+  int8_t e[kMaxQ][kMaxD];
+  double dt, dtR;
   int32_t order;
 };
 
@@ -217,7 +227,6 @@ cudaError_t launch_stability(int d, const double *omega_dev, int64_t npoints, in
                              unsigned long long *rho_bits_dev, cudaStream_t st);
 cudaError_t launch_init(int d, bool dev, const InitArgs &a, cudaStream_t st);
 cudaError_t launch_macro_fp64(int d, const StepArgs &a, double *phi_out, cudaStream_t st);
-cudaError_t launch_fd_grad(int d, const Geom &g, double dx, const double *phi, double *grad, cudaStream_t st);
 cudaError_t launch_fd_grad_transpose_add(int d, const Geom &g, double dx, const double *G, double *out,
                                          cudaStream_t st);
 cudaError_t launch_reduce(int d, bool dev, const ReduceArgs &a, int nblocks, cudaStream_t st);

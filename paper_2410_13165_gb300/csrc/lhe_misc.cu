@@ -1,6 +1,7 @@
 // lhe_misc.cu -- initialisation, finite-difference gradient, diagnostics reduction and the
 // adjoint seed / gradient kernels.
 #include <algorithm>
+#include <type_traits>
 
 #include "lhe_diag.cuh"
 #include "lhe_internal.h"
@@ -8,52 +9,222 @@
 
 namespace lhe {
 
-// ------------------------------------------------------------------------------ initialisation
-// Eq. (ini-simp): f_k(x,0) = omega_k [phi0 + (dt/2)(u - c e_k) . grad phi0] (order 3) or
-// omega_k phi0 (order 1); the stored state is post-collision. With A = phi0 + dt R(x) and the first
-// moment of the correction vanishing (sum_k omega_k (u - c e_k) = 0), the collision
-// f*_k = (1 - s) f_k + omega_k (s phi0 + dt R) is
-//   f*_k = omega_k A + (1 - s)(dt/2) omega_k [u . grad phi0 - c e_k . grad phi0]     (FP64)
-//   g*_k = f*_k - omega_k phi0 = omega_k dt R + (same correction),  phi = phi0      (FP32_DEV)
-// three FP64 operations per population (c1_k = (1 - s)(dt/2) omega_k, c2_k = c c1_k on the host).
-template <int D, bool DEV>
-__global__ void __launch_bounds__(256) k_init(const InitArgs a) {
-  constexpr Lattice<D> L{};
-  constexpr int Q = Lattice<D>::Q;
-  const int64_t site = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t S = a.g.S;
-  if (site >= S) return;
-  const double phi0 = a.phi0[site];
-  const double dtR = a.Rfield ? a.dt * a.Rfield[site] : a.dtR;
-  double gr[D];
-  double ug = 0.0;
+// ------------------------------------------------------------------------------ FD gradient
+// Periodic fourth-order central difference: d_i phi ~ (-phi(x+2e_i) + 8 phi(x+e_i) - 8 phi(x-e_i)
+// + phi(x-2e_i)) / (12 dx).
+__device__ __forceinline__ int32_t wrap_off(int xi, int o, int32_t n, int32_t stride) {
+  int y = xi + o;
+  if (y < 0) y += n;
+  if (y >= n) y -= n;
+  return (y - xi) * stride;
+}
+
+// phi(x + e_i) - phi(x - e_i) and phi(x + 2e_i) - phi(x - 2e_i); `near`: the largest high word of their magnitudes.
+__device__ __forceinline__ void fd_differences(const double *__restrict__ v, int32_t site, int xi, int32_t n,
+                                               int32_t stride, double &d1, double &d2, unsigned &near) {
+  const double p1 = __ldg(v + site + wrap_off(xi, 1, n, stride)), m1 = __ldg(v + site + wrap_off(xi, -1, n, stride));
+  const double p2 = __ldg(v + site + wrap_off(xi, 2, n, stride)), m2 = __ldg(v + site + wrap_off(xi, -2, n, stride));
+  d1 = p1 - m1;
+  d2 = p2 - m2;
+  const unsigned a = max((unsigned)__double2hiint(p1) & 0x7FFFFFFFu, (unsigned)__double2hiint(m1) & 0x7FFFFFFFu);
+  const unsigned b = max((unsigned)__double2hiint(p2) & 0x7FFFFFFFu, (unsigned)__double2hiint(m2) & 0x7FFFFFFFu);
+  near = max(near, max(a, b));
+}
+
+// Adds D_i^T G_i = -D_i G_i to `out` (the transpose of the difference).
+template <int D>
+__global__ void __launch_bounds__(256) k_fd_transpose(const Geom g, double inv12dx, const double *__restrict__ in,
+                                                      double *__restrict__ out) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= g.S) return;
+  int x[D];
+  const int32_t site = decode_site<D, false>(g, t, x);
+  double acc = out[site];
 #pragma unroll
   for (int i = 0; i < D; ++i) {
-    gr[i] = (a.order == 3) ? a.grad[i * S + site] : 0.0;
-    ug = fma(a.u[i], gr[i], ug);
+    const double *v = in + (int64_t)i * g.S;
+    const double p2 = v[site + wrap_off(x[i], 2, g.n[i], g.stride[i])];
+    const double p1 = v[site + wrap_off(x[i], 1, g.n[i], g.stride[i])];
+    const double m1 = v[site + wrap_off(x[i], -1, g.n[i], g.stride[i])];
+    const double m2 = v[site + wrap_off(x[i], -2, g.n[i], g.stride[i])];
+    acc -= (-p2 + 8.0 * p1 - 8.0 * m1 + m2) * inv12dx;
   }
-  const double A = DEV ? dtR : phi0 + dtR;
+  out[site] = acc;
+}
+
+cudaError_t launch_fd_grad_transpose_add(int d, const Geom &g, double dx, const double *G, double *out,
+                                         cudaStream_t st) {
+  const unsigned blocks = (unsigned)((g.S + 255) / 256);
+  const double w = 1.0 / (12.0 * dx);
+  switch (d) {
+    case 1: k_fd_transpose<1><<<blocks, 256, 0, st>>>(g, w, G, out); break;
+    case 2: k_fd_transpose<2><<<blocks, 256, 0, st>>>(g, w, G, out); break;
+    case 3: k_fd_transpose<3><<<blocks, 256, 0, st>>>(g, w, G, out); break;
+    case 4: k_fd_transpose<4><<<blocks, 256, 0, st>>>(g, w, G, out); break;
+    case 5: k_fd_transpose<5><<<blocks, 256, 0, st>>>(g, w, G, out); break;
+    default: return cudaErrorInvalidValue;
+  }
+  return cudaGetLastError();
+}
+
+// ------------------------------------------------------------------------------ initialisation
+// Eq. (ini-simp): f_k(x,0) = omega_k [phi0 + (dt/2)(u - c e_k) . grad phi0] (order 3) or
+// omega_k phi0 (order 1); the stored state is post-collision. The first moment of the correction
+// vanishes (sum_k omega_k (u - c e_k) = 0), so the collision f*_k = (1 - s) f_k + omega_k (s phi0 + dt R) is
+//   f*_k = omega_k (B - sum_i e_ki h_i),  h_i = (1 - s)(dt/2) c d_i phi0,
+//   B = phi0 + dt R + (1 - s)(dt/2) u . grad phi0                                    (FP64)
+//   g*_k = f*_k - omega_k phi0: the same with B = dt R + (1 - s)(dt/2) u . grad phi0,  phi = phi0   (FP32_DEV)
+// The gradient is read (kGradGiven) or formed here from phi0 (kGradFD), which saves its trip through memory.
+// Bound by the FP64 pipe (~2 operations per clock per SM), not by memory, unless operations are spared:
+// two per population here (the four values B -+ (h_i +- h_j) of a pair share their sums), against five
+// before (D3Q19 256^3, gradient formed: 3.03 -> 1.89 ms; the memory floor is 0.42).
+// FP32_DEV results are rounded to float, so the sums and products run on float pairs (48 bits) on the FP32
+// pipe and only the differences of phi0 in FP64. A result whose rounding the pairs' error could change
+// (Ziv's rounding test, "Fast evaluation of elementary mathematical functions with correctly rounded last
+// bit", TOMS 1991), and every one outside the pairs' range (largest term outside 2^-60 .. 2^100, infinities, NaN),
+// is formed in FP64 instead, so the stored floats are those of the FP64 form at every node. D3Q19 128^3
+// 451 -> 80 us (memory floor 36), D5Q51 24^5 4.24 -> 0.89 ms (floor 0.26).
+constexpr int kGradNone = 0, kGradGiven = 1, kGradFD = 2;
+
+// v_k = omega_k (B - sum_i e_ki h_i) for every k, with the arithmetic of T (double or float pairs).
+template <int D, class T, class Add, class Sub, class Out>
+__device__ __forceinline__ void init_populations(T B, const T (&h)[D], Add add, Sub sub, Out out) {
+  out(0, B);
 #pragma unroll
-  for (int k = 0; k < Q; ++k) {
-    double eg = 0.0;  // e_k . grad phi0 (components are 0 or +-1)
+  for (int i = 0; i < D; ++i) {
+    out(1 + i, sub(B, h[i]));
+    out(1 + D + i, add(B, h[i]));
+  }
+  int k = 2 * D + 1;
+#pragma unroll
+  for (int i = 0; i < D; ++i)
+#pragma unroll
+    for (int j = i + 1; j < D; ++j) {  // components (1, 1), (-1, 1), (-1, -1), (1, -1)
+      const T p = add(h[i], h[j]), q = sub(h[i], h[j]);
+      out(k, sub(B, p));
+      out(k + 1, add(B, q));
+      out(k + 2, add(B, p));
+      out(k + 3, sub(B, q));
+      k += 4;
+    }
+}
+
+// g*_k of one node and population in FP64, rounded to float.
+template <int D, int GRAD>
+__device__ __noinline__ float deviation_fp64(const InitArgs &a, int32_t site, int k) {
+  const double dtR = a.Rfield ? a.dt * __ldg(a.Rfield + site) : a.dtR;
+  int x[D];
+  decode_site<D, false>(a.g, site, x);
+  double ug = 0.0, eg = 0.0;
+  for (int i = 0; i < D; ++i) {
+    double gr = 0.0;
+    if (GRAD == kGradGiven) gr = __ldg(a.grad + i * a.g.S + site);
+    if (GRAD == kGradFD) {
+      const double p2 = __ldg(a.phi0 + site + wrap_off(x[i], 2, a.g.n[i], a.g.stride[i]));
+      const double p1 = __ldg(a.phi0 + site + wrap_off(x[i], 1, a.g.n[i], a.g.stride[i]));
+      const double m1 = __ldg(a.phi0 + site + wrap_off(x[i], -1, a.g.n[i], a.g.stride[i]));
+      const double m2 = __ldg(a.phi0 + site + wrap_off(x[i], -2, a.g.n[i], a.g.stride[i]));
+      gr = (fma(-8.0, m1, fma(8.0, p1, -p2)) + m2) * a.inv12dx;
+    }
+    ug = fma(a.u[i], gr, ug);
+    if (a.e[k][i] == 1) eg += gr;
+    if (a.e[k][i] == -1) eg -= gr;
+  }
+  return (float)fma(a.omega[k], dtR, fma(-a.c2[k], eg, a.c1[k] * ug));
+}
+
+template <int D, bool DEV, int GRAD>
+__global__ void __launch_bounds__(256) k_init(const __grid_constant__ InitArgs a) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t S = a.g.S;
+  if (t >= S) return;
+  const int32_t site = (int32_t)t;
+  const double phi0 = __ldg(a.phi0 + site);
+  const double dtR = a.Rfield ? a.dt * __ldg(a.Rfield + site) : a.dtR;
+  // g1: the gradient, or phi(x+e_i) - phi(x-e_i), and g2 = phi(x+2e_i) - phi(x-2e_i)
+  double g1[D], g2[D];
+  unsigned near = 0u;  // high word of the largest |phi0| that the differences were formed from
+  if (GRAD == kGradFD) {
+    int x[D];
+    decode_site<D, false>(a.g, t, x);
+#pragma unroll
+    for (int i = 0; i < D; ++i) fd_differences(a.phi0, site, x[i], a.g.n[i], a.g.stride[i], g1[i], g2[i], near);
+  } else {
 #pragma unroll
     for (int i = 0; i < D; ++i) {
-      if (L.e[k][i] == 1) eg += gr[i];
-      if (L.e[k][i] == -1) eg -= gr[i];
+      g1[i] = GRAD == kGradGiven ? __ldg(a.grad + i * S + site) : 0.0;
+      g2[i] = 0.0;
     }
-    const double v = fma(a.omega[k], A, fma(-a.c2[k], eg, a.c1[k] * ug));
-    if (DEV) static_cast<float *>(a.dst)[k * S + site] = (float)v;
-    else static_cast<double *>(a.dst)[k * S + site] = v;
   }
-  if (DEV) a.phi_dst[site] = df_split(phi0);
+  if (DEV) {
+    float *__restrict__ dst = static_cast<float *>(a.dst);
+    int top = double_exponent(dtR);
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      top = max(top, double_exponent(g1[i]));
+      if (GRAD == kGradFD) top = max(top, double_exponent(g2[i]));
+    }
+    const int ep = double_exponent(phi0), en = (int)(near >> 20) - 1023;
+    a.phi_dst[site] = (ep >= -60 && ep <= 100) ? ff_split(phi0) : df_split(phi0);
+    if (a.pairs && en <= 100 && ((top >= -60 && top <= 100) || top == -1023)) {
+      float2 h[D], B = ff_split(dtR);
+      float err = fabsf(B.x);  // sum of the magnitudes of the terms
+#pragma unroll
+      for (int i = 0; i < D; ++i) {
+        float2 g = ff_split(g1[i]);
+        float m = fabsf(g.x);
+        if (GRAD == kGradFD) {
+          const float2 w = ff_split(g2[i]);
+          g = ff_sub(make_float2(8.0f * g.x, 8.0f * g.y), w);
+          m = fmaf(8.0f, m, fabsf(w.x));
+        }
+        if (GRAD != kGradNone) B = ff_add(B, ff_mul(a.wu_f[i], g));
+        h[i] = ff_mul(a.wc_f, g);
+        err = fmaf(a.werr, m, err);
+      }
+      // bound of the difference to the FP64 form: 2^-43 of the terms (an operation on pairs is within ~2^-45
+      // of its operands) and the rounding of the FP64 differences, 2^-48 of the values that enter them
+      err *= 0x1p-43f;
+      if (GRAD == kGradFD) err = fmaf(a.werr * 0x1p-48f, ff_split(__hiloint2double((int)near, 0)).x, err);
+      init_populations<D>(
+          B, h, [](float2 p, float2 q) { return ff_add(p, q); }, [](float2 p, float2 q) { return ff_sub(p, q); },
+          [&](int k, float2 v) {
+            const float2 w = a.omega_f[k];
+            const float p = __fmul_rn(w.x, v.x);
+            const float e = __fmaf_rn(w.x, v.y, __fmaf_rn(w.y, v.x, __fmaf_rn(w.x, v.x, -p)));
+            float r = __fadd_rn(p, __fmaf_rn(w.x, err, e));
+            if (r != __fadd_rn(p, __fmaf_rn(-w.x, err, e))) r = deviation_fp64<D, GRAD>(a, site, k);
+            dst[k * S + site] = r;
+          });
+      return;
+    }
+    for (int k = 0; k < Lattice<D>::Q; ++k) dst[k * S + site] = deviation_fp64<D, GRAD>(a, site, k);
+    return;
+  }
+  double h[D], B = phi0 + dtR;
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    const double g = GRAD == kGradFD ? fma(8.0, g1[i], -g2[i]) : g1[i];
+    if (GRAD != kGradNone) B = fma(a.wu[i], g, B);
+    h[i] = a.wc * g;
+  }
+  double *__restrict__ dst = static_cast<double *>(a.dst);
+  init_populations<D>(B, h, [](double p, double q) { return p + q; }, [](double p, double q) { return p - q; },
+                      [&](int k, double v) { dst[k * S + site] = a.omega[k] * v; });
+}
+
+template <int D, int GRAD>
+static cudaError_t init_dg(bool dev, const InitArgs &a, cudaStream_t st) {
+  const unsigned blocks = (unsigned)((a.g.S + 255) / 256);
+  if (dev) k_init<D, true, GRAD><<<blocks, 256, 0, st>>>(a);
+  else k_init<D, false, GRAD><<<blocks, 256, 0, st>>>(a);
+  return cudaGetLastError();
 }
 
 template <int D>
 static cudaError_t init_d(bool dev, const InitArgs &a, cudaStream_t st) {
-  const unsigned blocks = (unsigned)((a.g.S + 255) / 256);
-  if (dev) k_init<D, true><<<blocks, 256, 0, st>>>(a);
-  else k_init<D, false><<<blocks, 256, 0, st>>>(a);
-  return cudaGetLastError();
+  if (a.order != 3) return init_dg<D, kGradNone>(dev, a, st);
+  return a.grad ? init_dg<D, kGradGiven>(dev, a, st) : init_dg<D, kGradFD>(dev, a, st);
 }
 
 cudaError_t launch_init(int d, bool dev, const InitArgs &a, cudaStream_t st) {
@@ -65,66 +236,6 @@ cudaError_t launch_init(int d, bool dev, const InitArgs &a, cudaStream_t st) {
     case 5: return init_d<5>(dev, a, st);
     default: return cudaErrorInvalidValue;
   }
-}
-
-// ------------------------------------------------------------------------------ FD gradient
-// Periodic fourth-order central difference: d_i phi ~ (-phi(x+2e_i) + 8 phi(x+e_i) - 8 phi(x-e_i)
-// + phi(x-2e_i)) / (12 dx). TRANSPOSE adds D_i^T G_i = -D_i G_i to `out` instead.
-__device__ __forceinline__ int32_t wrap_off(int xi, int o, int32_t n, int32_t stride) {
-  int y = xi + o;
-  if (y < 0) y += n;
-  if (y >= n) y -= n;
-  return (y - xi) * stride;
-}
-
-template <int D, bool TRANSPOSE>
-__global__ void __launch_bounds__(256) k_fd(const Geom g, double inv12dx, const double *__restrict__ in,
-                                            double *__restrict__ out) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= g.S) return;
-  int x[D];
-  const int32_t site = decode_site<D, false>(g, t, x);
-  double acc = TRANSPOSE ? out[site] : 0.0;
-#pragma unroll
-  for (int i = 0; i < D; ++i) {
-    const double *v = in + (TRANSPOSE ? (int64_t)i * g.S : 0);
-    const double p2 = v[site + wrap_off(x[i], 2, g.n[i], g.stride[i])];
-    const double p1 = v[site + wrap_off(x[i], 1, g.n[i], g.stride[i])];
-    const double m1 = v[site + wrap_off(x[i], -1, g.n[i], g.stride[i])];
-    const double m2 = v[site + wrap_off(x[i], -2, g.n[i], g.stride[i])];
-    const double di = (-p2 + 8.0 * p1 - 8.0 * m1 + m2) * inv12dx;
-    if (TRANSPOSE) acc -= di;
-    else out[(int64_t)i * g.S + site] = di;
-  }
-  if (TRANSPOSE) out[site] = acc;
-}
-
-template <int D, bool T>
-static cudaError_t fd_d(const Geom &g, double dx, const double *in, double *out, cudaStream_t st) {
-  const unsigned blocks = (unsigned)((g.S + 255) / 256);
-  k_fd<D, T><<<blocks, 256, 0, st>>>(g, 1.0 / (12.0 * dx), in, out);
-  return cudaGetLastError();
-}
-
-template <bool T>
-static cudaError_t fd_dispatch(int d, const Geom &g, double dx, const double *in, double *out, cudaStream_t st) {
-  switch (d) {
-    case 1: return fd_d<1, T>(g, dx, in, out, st);
-    case 2: return fd_d<2, T>(g, dx, in, out, st);
-    case 3: return fd_d<3, T>(g, dx, in, out, st);
-    case 4: return fd_d<4, T>(g, dx, in, out, st);
-    case 5: return fd_d<5, T>(g, dx, in, out, st);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-cudaError_t launch_fd_grad(int d, const Geom &g, double dx, const double *phi, double *grad, cudaStream_t st) {
-  return fd_dispatch<false>(d, g, dx, phi, grad, st);
-}
-
-cudaError_t launch_fd_grad_transpose_add(int d, const Geom &g, double dx, const double *G, double *out,
-                                         cudaStream_t st) {
-  return fd_dispatch<true>(d, g, dx, G, out, st);
 }
 
 // ------------------------------------------------------------------------------ diagnostics
