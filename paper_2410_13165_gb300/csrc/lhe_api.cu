@@ -1362,7 +1362,9 @@ lhe_status lhe_lbm_stability_map(const lhe_lbm_params *p, const double *sigma, i
   int32_t e[kMaxQ * kMaxD];
   const int Q = lattice_vectors(d, e);
   const int npairs = d * (d - 1) / 2;
-  std::vector<double> om((size_t)npoints * Q);
+  // one device buffer: the radii (as the bits of doubles, from 0) and the weights
+  std::vector<double> buf((size_t)npoints * (Q + 1), 0.0);
+  double *om = buf.data() + npoints;
   for (int64_t q = 0; q < npoints; ++q) {
     double sig[kMaxD], m4[10] = {};
     for (int i = 0; i < d; ++i) {
@@ -1376,24 +1378,17 @@ lhe_status lhe_lbm_stability_map(const lhe_lbm_params *p, const double *sigma, i
     omega_min[q] = mn;
   }
   cudaStream_t st = static_cast<cudaStream_t>(p->stream);
-  double *dom = nullptr;
-  unsigned long long *drho = nullptr;
-  auto release = [&]() {
-    cudaFree(dom);
-    cudaFree(drho);
-  };
-  cudaError_t e1 = cudaMalloc(&dom, sizeof(double) * om.size());
-  if (e1 == cudaSuccess) e1 = cudaMalloc(&drho, sizeof(unsigned long long) * (size_t)npoints);
-  if (e1 == cudaSuccess) e1 = cudaMemcpyAsync(dom, om.data(), sizeof(double) * om.size(), cudaMemcpyHostToDevice, st);
-  if (e1 == cudaSuccess) e1 = cudaMemsetAsync(drho, 0, sizeof(unsigned long long) * (size_t)npoints, st);
-  if (e1 == cudaSuccess) e1 = launch_stability(d, dom, npoints, nxi, 1.0 / p->tau, drho, st);
-  std::vector<unsigned long long> bits((size_t)npoints);
+  double *dev = nullptr;
+  cudaError_t e1 = cudaMalloc(&dev, sizeof(double) * buf.size());
+  if (e1 == cudaSuccess) e1 = cudaMemcpyAsync(dev, buf.data(), sizeof(double) * buf.size(), cudaMemcpyHostToDevice, st);
   if (e1 == cudaSuccess)
-    e1 = cudaMemcpyAsync(bits.data(), drho, sizeof(unsigned long long) * bits.size(), cudaMemcpyDeviceToHost, st);
+    e1 = launch_stability(d, dev + npoints, npoints, nxi, 1.0 / p->tau, reinterpret_cast<unsigned long long *>(dev), st);
+  if (e1 == cudaSuccess)
+    e1 = cudaMemcpyAsync(buf.data(), dev, sizeof(double) * (size_t)npoints, cudaMemcpyDeviceToHost, st);
   if (e1 == cudaSuccess) e1 = cudaStreamSynchronize(st);
-  release();
+  cudaFree(dev);
   if (e1 != cudaSuccess) return cuda_fail(nullptr, e1, "stability map");
-  for (int64_t q = 0; q < npoints; ++q) std::memcpy(&rho_max[q], &bits[(size_t)q], sizeof(double));
+  std::memcpy(rho_max, buf.data(), sizeof(double) * (size_t)npoints);
   return LHE_OK;
 }
 

@@ -4,12 +4,16 @@
 // is the same matrix in moment space, G_moment = M G M^{-1}). The von Neumann (L2) condition is
 // rho(G(xi)) <= 1 for every xi; Proposition 1's microscopic entropy condition is min_k omega_k > 0.
 //
-// One thread per (sigma, xi): the Q x Q complex matrix is reduced to upper Hessenberg form by
-// Householder reflections, then its eigenvalues are found by the shifted QR iteration (Givens
-// rotations, Wilkinson shifts, deflation on negligible subdiagonals), all in FP64. The QR route
-// is backward stable, so the (Q-1)-fold eigenvalue 1 - s of G(0) comes out to rounding, where the
-// roots of the characteristic polynomial would spread by eps^(1/(Q-1)). The radius per sigma is the
-// maximum over its xi, reduced with an integer atomic max on the (non-negative) double bits.
+// The matrix is a diagonal plus a rank-one matrix: its eigenvalues are found from the secular equation
+// (k_stability), with repeated phases deflated, so that the (Q-1)-fold eigenvalue 1 - s of G(0) comes out to
+// rounding, where the roots of the characteristic polynomial would spread by eps^(1/(Q-1)). A matrix whose roots
+// do not pass the trace checks takes the backward-stable QR route (radius_qr): the Q x Q complex matrix is reduced
+// to upper Hessenberg form by Householder reflections, then its eigenvalues are found by the shifted
+// QR iteration (Givens rotations, Wilkinson shifts, deflation on negligible subdiagonals), all in FP64.
+// The radius per sigma is the maximum over its xi, reduced with an integer atomic max on the (non-negative)
+// double bits.
+#include <algorithm>
+
 #include "lhe_internal.h"
 
 namespace lhe {
@@ -154,21 +158,13 @@ __device__ double spectral_radius(cd (&A)[N][N]) {
   return rho;
 }
 
+// The radius of one matrix by the QR route, from the population-space matrix itself.
 template <int D>
-__global__ void __launch_bounds__(128) k_stability(const double *__restrict__ omega, int64_t npoints, int32_t nxi,
-                                                   int64_t nper, double s, unsigned long long *__restrict__ rho_bits) {
+__device__ __noinline__ double radius_qr(const double *__restrict__ omega, const int (&j)[D], int32_t nxi, double s) {
   constexpr Lattice<D> L{};
   constexpr int Q = Lattice<D>::Q;
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= npoints * nper) return;
-  const int64_t p = t / nper;
-  int64_t r = t - p * nper;
   double xi[D];
-  for (int i = 0; i < D; ++i) {
-    const int64_t j = r % nxi;
-    r /= nxi;
-    xi[i] = -kPi + 2.0 * kPi * (double)j / (double)nxi;
-  }
+  for (int i = 0; i < D; ++i) xi[i] = -kPi + 2.0 * kPi * (double)j[i] / (double)nxi;
   cd A[Q][Q];
   for (int k = 0; k < Q; ++k) {
     double ph = 0.0;
@@ -176,32 +172,325 @@ __global__ void __launch_bounds__(128) k_stability(const double *__restrict__ om
     double sn, cs;
     sincos(ph, &sn, &cs);
     const cd tk = mk(cs, sn);  // exp(-i e_k . xi)
-    const double wk = s * omega[p * Q + k];
-    for (int j = 0; j < Q; ++j) A[k][j] = (wk + (j == k ? 1.0 - s : 0.0)) * tk;
+    const double wk = s * omega[k];
+    for (int q = 0; q < Q; ++q) A[k][q] = (wk + (q == k ? 1.0 - s : 0.0)) * tk;
   }
-  double rho = spectral_radius<Q>(A);
-  if (rho != rho) rho = __longlong_as_double(0x7FF0000000000000ll);  // not converged: report +inf
-  atomicMax(rho_bits + p, (unsigned long long)__double_as_longlong(rho));
+  const double rho = spectral_radius<Q>(A);
+  return rho == rho ? rho : __longlong_as_double(0x7FF0000000000000ll);  // not converged: report +inf
+}
+
+struct StabilityArgs {
+  const double *omega;  // Q per velocity
+  unsigned long long *rho_bits;
+  int64_t npoints, nper;  // velocities; Fourier variables per velocity that are visited
+  int32_t nxi;
+  double s;
+  int8_t e[33][4];
+};
+
+struct cf {
+  float re, im;
+};
+__device__ __forceinline__ cf operator+(cf a, cf b) { return cf{a.re + b.re, a.im + b.im}; }
+__device__ __forceinline__ cf operator-(cf a, cf b) { return cf{a.re - b.re, a.im - b.im}; }
+__device__ __forceinline__ cf operator*(cf a, cf b) { return cf{a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re}; }
+__device__ __forceinline__ float ab2(cf a) { return fmaf(a.re, a.re, a.im * a.im); }
+__device__ __forceinline__ cf rcp(cf a) {
+  const float n = __fdividef(1.0f, ab2(a));
+  return cf{a.re * n, -a.im * n};
+}
+// 1/n by one third-order Newton step, x (1 + e + e^2) with e = 1 - n x, from a seed of ~22 bits: three FP64
+// operations (a division takes several times that), within one unit in the last place. For 2^-126 < n < 2^126.
+__device__ __forceinline__ cd rcp(cd a) {
+  const double n = ab2(a);
+  const double x = float_to_double(__fdividef(1.0f, ff_split(n).x));
+  const double e = fma(-n, x, 1.0);
+  const double y = fma(x, fma(e, e, e), x);
+  return cd{a.re * y, -a.im * y};
+}
+
+// G(xi) is a diagonal plus a rank-one matrix, T((1 - s) I + s omega 1^T), so its eigenvalues need no O(Q^3)
+// reduction. Links with the same phase share a pole tau_p (the phases are multiples of pi / nxi: exact integers),
+// whose weights add up to W_p; all but one of a shared pole's links, and poles of weight zero, have the eigenvalue
+// (1 - s) tau_p. The others are (1 - s) z with z a root of the secular equation (Golub, "Some modified
+// matrix eigenvalue problems", SIAM Review 15, 1973)
+//   1 + kappa sum_p tau_p W_p / (tau_p - z) = 0,  kappa = s / (1 - s).
+// All P <= Q roots are found together by the Ehrlich-Aberth iteration (Aberth, "Iteration methods for finding all
+// zeros of a polynomial simultaneously", Math. Comp. 27, 1973) on the polynomial of which they are the
+// zeros, each as an offset d from a pole b, z = tau_b + d, which keeps roots next to poles of small weight
+// exact: with c_p = kappa tau_p W_p, S = 1 + sum_{p != b} c_p / (tau_p - z) and g = d S - c_b,
+//   d -= g / (S + d S' + g (sum_{p != b} 1 / (z - tau_p) - sum_{other roots} 1 / (z - z_j))).
+// FP32 iterations (the FP32 pipe runs 64 times the FP64 pipe's rate) bring the offsets to ~1e-6; then S and g
+// in FP64, with the denominator still in FP32, until a step is below 2e-9 (the step's relative error
+// is ~1e-6, so the next one would be below rounding): two as a rule. The roots are accepted if their sum and sum
+// of squares match the matrix's traces; else, and without convergence, the matrix takes the QR route.
+// A group of G lanes holds a matrix, a lane a root (two for the 33rd pole of D = 4); G is the smallest of 8, 16
+// and 32 that holds the poles, of which there are at most nxi (nxi even) or 2 nxi. G(-xi) is the conjugate of G(xi), so half
+// of the last axis is visited. Bound by the FP64 pipe (~70 % busy: S in the last two iterations, the poles' sines). Against roots
+// refined in 80 bits (600 random D3Q19 matrices) the radius is within 6e-15, LAPACK's QR within 3e-14. 24 velocities of D3Q19, 12^3 Fourier variables: 29.2 ms by QR (one thread
+// per matrix, in local memory) -> 0.53 ms.
+template <int D, int G>
+__global__ void __launch_bounds__(128) k_stability(const __grid_constant__ StabilityArgs a) {
+  constexpr int Q = 2 * D * D + 1;
+  constexpr int R = (Q + G - 1) / G;  // roots per lane at most
+  constexpr int kGroups = 128 / G;
+  __shared__ cd tau64[kGroups][Q], c64[kGroups][Q];  // poles and kappa tau_p W_p
+  __shared__ float4 tauf[kGroups][Q];                // poles as float pairs (re, im, low parts)
+  __shared__ cf cfl[kGroups][Q], off[kGroups][Q];    // the weights in FP32; offsets of the roots from their own poles
+  __shared__ int ang[kGroups][Q];
+  const int grp = threadIdx.x / G, lane = threadIdx.x % G, nxi = a.nxi;
+  const unsigned shift = (threadIdx.x & 31u) / G * G, gmask = G == 32 ? 0xffffffffu : ((1u << (G & 31)) - 1u) << shift;
+  const int64_t total = a.npoints * a.nper;
+  for (int64_t t0 = blockIdx.x * (int64_t)kGroups; t0 < total; t0 += (int64_t)gridDim.x * kGroups) {
+    int64_t t = t0 + grp;
+    const bool idle = t >= total;  // surplus groups repeat the last matrix and write nothing
+    if (idle) t = total - 1;
+    __syncwarp();  // the last matrix's tables are read out
+    const int64_t pt = t / a.nper;
+    const double *__restrict__ omega = a.omega + pt * Q;
+    int j[D];
+    {
+      int64_t r = t - pt * a.nper;
+#pragma unroll
+      for (int i = 0; i < D; ++i) {
+        j[i] = (int)(i == D - 1 ? r : r % nxi);
+        r /= nxi;
+      }
+    }
+    // phases of the links, -e_k . xi = (pi / nxi) (nxi sum_i e_ki - 2 sum_i e_ki j_i)
+    for (int k = lane; k < Q; k += G) {
+      int v = 0;
+#pragma unroll
+      for (int i = 0; i < D; ++i) v += a.e[k][i] * (nxi - 2 * j[i]);
+      v %= 2 * nxi;
+      ang[grp][k] = v < 0 ? v + 2 * nxi : v;
+    }
+    __syncwarp();
+    const double r1 = 1.0 - a.s, kappa = a.s / r1;
+    int P = 0;
+    bool deflated = false;
+    cd trace = mk(0.0, 0.0);  // sum over the links of tau W
+    for (int k0 = 0; k0 < Q; k0 += G) {
+      const int k = k0 + lane;
+      bool first = k < Q;
+      double W = 0.0;
+      if (k < Q)
+        for (int q = 0; q < Q; ++q)
+          if (ang[grp][q] == ang[grp][k]) {
+            if (q < k) first = false;
+            W += omega[q];
+          }
+      const bool keep = first && fabs(W) > 1e-15;
+      const unsigned kept = __ballot_sync(0xffffffffu, keep) & gmask;
+      if (__ballot_sync(0xffffffffu, k < Q && !keep) & gmask) deflated = true;
+      if (keep) {
+        const int p = P + __popc(kept & ((1u << (threadIdx.x & 31u)) - 1u));
+        double sn, cs;
+        sincospi((double)ang[grp][k] / (double)nxi, &sn, &cs);
+        const cd c = (kappa * W) * mk(cs, sn);
+        tau64[grp][p] = mk(cs, sn);
+        c64[grp][p] = a.s == 1.0 ? W * mk(cs, sn) : c;
+        cfl[grp][p] = cf{(float)c.re, (float)c.im};
+        const float2 x = df_split(cs), y = df_split(sn);
+        tauf[grp][p] = make_float4(x.x, y.x, x.y, y.y);
+      }
+      P += __popc(kept);
+    }
+    __syncwarp();
+    for (int p = 0; p < P; ++p) trace = trace + c64[grp][p];  // kappa sum tau W
+    if (a.s == 1.0) {  // the matrix has rank one: its only eigenvalue besides 0 is sum tau W
+      if (lane == 0 && !idle) atomicMax(a.rho_bits + pt, (unsigned long long)__double_as_longlong(ab(trace)));
+      continue;
+    }
+    // pole i minus pole q in FP32
+    auto pole_diff = [&](float4 ti, int q) {
+      const float4 tq = tauf[grp][q];
+      return cf{(ti.x - tq.x) + (ti.z - tq.z), (ti.y - tq.y) + (ti.w - tq.w)};
+    };
+    // first offsets: the other poles seen from the pole
+    cf d[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int i = lane + r * G;
+      d[r] = cf{0.0f, 0.0f};
+      if (i >= P) continue;
+      const float4 ti = tauf[grp][i];
+      cf S{1.0f, 0.0f};
+      for (int q = 0; q < P; ++q)
+        if (q != i) S = S - cfl[grp][q] * rcp(pole_diff(ti, q));
+      if (!(ab2(S) >= 0.0625f)) S = cf{0.25f, 0.0f};
+      // a little off the symmetric starts from which the iteration cannot part two roots
+      d[r] = cfl[grp][i] * rcp(S) * cf{1.0f + 0.02f * (float)((i * 5) % 7 - 3) * 0.33f, 0.02f * (float)((i * 3) % 5 - 2) * 0.5f};
+      off[grp][i] = d[r];
+    }
+    __syncwarp();
+    const float reach = fmaxf(0.5f, 0.5f * fabsf((float)kappa));
+    for (int it = 0; it < 20; ++it) {
+      float worst = 0.0f;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int i = lane + r * G;
+        if (i >= P) continue;
+        const float4 ti = tauf[grp][i];
+        cf S{1.0f, 0.0f}, Sp{0.0f, 0.0f}, sum{0.0f, 0.0f};
+        for (int q = 0; q < P; ++q) {
+          if (q == i) continue;
+          const cf z = pole_diff(ti, q) + d[r];
+          const cf A = rcp(z), T = cfl[grp][q] * A;
+          S = S - T;
+          Sp = Sp + T * A;
+          sum = sum + A - rcp(z - off[grp][q]);
+        }
+        const cf g = d[r] * S - cfl[grp][i];
+        cf st = g * rcp(S + d[r] * Sp + g * sum);
+        const float m = sqrtf(ab2(st)), lim = fmaxf(reach, sqrtf(ab2(d[r])));
+        if (!(m < 1e30f)) st = cf{0.01f, 0.0f};
+        else if (m > lim) st = cf{st.re * (lim / m), st.im * (lim / m)};
+        worst = fmaxf(worst, m < 1e30f ? m / fmaxf(1.0f, sqrtf(ab2(d[r]))) : 1.0f);
+        d[r] = d[r] - st;
+      }
+      __syncwarp();
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        if (lane + r * G < P) off[grp][lane + r * G] = d[r];
+      __syncwarp();
+      if (!__any_sync(0xffffffffu, worst > 4e-6f)) break;
+    }
+    // FP64: the offset from the nearest pole
+    int b[R];
+    cd d64[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int i = lane + r * G;
+      b[r] = 0;
+      d64[r] = mk(0.0, 0.0);
+      if (i >= P) continue;
+      const float4 ti = tauf[grp][i];
+      float best = ab2(d[r]);
+      b[r] = i;
+      for (int q = 0; q < P; ++q) {
+        const float m = ab2(pole_diff(ti, q) + d[r]);
+        if (q != i && m < best) {
+          best = m;
+          b[r] = q;
+        }
+      }
+      d64[r] = (tau64[grp][i] - tau64[grp][b[r]]) + mk((double)d[r].re, (double)d[r].im);
+    }
+    bool converged = false;
+    for (int it = 0; it < 12; ++it) {
+      bool small = true;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int i = lane + r * G;
+        if (i >= P) continue;
+        const float4 ti = tauf[grp][i];
+        const cd tb = tau64[grp][b[r]];
+        cd S = mk(1.0, 0.0);
+        cf Sp{0.0f, 0.0f}, sum{0.0f, 0.0f};
+        for (int q = 0; q < P; ++q) {
+          const cf z = pole_diff(ti, q) + off[grp][i];
+          if (q != i) sum = sum - rcp(z - off[grp][q]);
+          if (q == b[r]) continue;
+          S = S - c64[grp][q] * rcp((tb - tau64[grp][q]) + d64[r]);
+          const cf A = rcp(z);
+          Sp = Sp + cfl[grp][q] * A * A;
+          sum = sum + A;
+        }
+        const cd g = d64[r] * S - c64[grp][b[r]];
+        const cf gf{(float)g.re, (float)g.im}, df{(float)d64[r].re, (float)d64[r].im};
+        const cf inv = rcp(cf{(float)S.re, (float)S.im} + df * Sp + gf * sum);
+        const cd st = g * mk((double)inv.re, (double)inv.im);
+        d64[r] = d64[r] - st;
+        if (!(ab2(st) <= 4e-18 * fmax(1.0, ab2(d64[r])))) small = false;
+      }
+      __syncwarp();
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int i = lane + r * G;
+        if (i >= P) continue;
+        const cd o = (tau64[grp][b[r]] - tau64[grp][i]) + d64[r];
+        off[grp][i] = cf{(float)o.re, (float)o.im};
+      }
+      __syncwarp();
+      converged = (__ballot_sync(0xffffffffu, !small) & gmask) == 0u;
+      if (__all_sync(0xffffffffu, converged)) break;
+    }
+    // traces: sum z = sum tau + kappa sum tau W; sum z^2 = sum tau^2 (1 + 2 kappa W) + (kappa sum tau W)^2
+    cd s1 = mk(0.0, 0.0), s2 = mk(0.0, 0.0);
+    double top = 0.0;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int i = lane + r * G;
+      if (i >= P) continue;
+      const cd ti = tau64[grp][i], z = tau64[grp][b[r]] + d64[r], c = c64[grp][i];
+      s1 = s1 + z - ti - c;
+      s2 = s2 + z * z - ti * ti - 2.0 * (ti * c);
+      top = fmax(top, ab2(z));
+    }
+    for (int o = G / 2; o > 0; o >>= 1) {
+      s1 = s1 + mk(__shfl_xor_sync(0xffffffffu, s1.re, o), __shfl_xor_sync(0xffffffffu, s1.im, o));
+      s2 = s2 + mk(__shfl_xor_sync(0xffffffffu, s2.re, o), __shfl_xor_sync(0xffffffffu, s2.im, o));
+      top = fmax(top, __shfl_xor_sync(0xffffffffu, top, o));
+    }
+    s2 = s2 - trace * trace;
+    const double tol = 1e-10 * P * fmax(1.0, kappa * kappa);
+    const bool good = converged && ab1(s1) < tol && ab1(s2) < tol;
+    if (lane == 0 && !idle) {
+      double rho = fabs(r1) * sqrt(top);
+      if (deflated) rho = fmax(rho, fabs(r1));
+      if (!good) rho = radius_qr<D>(omega, j, nxi, a.s);
+      // the bits of non-negative doubles order as integers; most matrices do not raise the maximum
+      unsigned long long *out = a.rho_bits + pt;
+      const unsigned long long bits = (unsigned long long)__double_as_longlong(rho);
+      if (*(volatile unsigned long long *)out < bits) atomicMax(out, bits);
+    }
+  }
+}
+
+template <int D, int G>
+cudaError_t stability_dg(const StabilityArgs &a, cudaStream_t st) {
+  const int64_t groups = a.npoints * a.nper;
+  const int64_t blocks = std::min<int64_t>((groups + 128 / G - 1) / (128 / G), 1 << 20);
+  k_stability<D, G><<<(unsigned)blocks, 128, 0, st>>>(a);
+  return cudaGetLastError();
+}
+
+template <int D>
+cudaError_t stability_d(StabilityArgs &a, cudaStream_t st) {
+  constexpr Lattice<D> L{};
+  constexpr int Q = Lattice<D>::Q;
+  for (int k = 0; k < Q; ++k)
+    for (int i = 0; i < D; ++i) a.e[k][i] = (int8_t)L.e[k][i];
+  a.nper = a.nxi / 2 + 1;  // G(-xi) = conj G(xi): j_d <= nxi / 2 (and its partner nxi - j_d)
+  if (a.nper > a.nxi) a.nper = a.nxi;
+  for (int i = 0; i < D - 1; ++i) a.nper *= a.nxi;
+  const int poles = std::min(Q, a.nxi % 2 ? 2 * a.nxi : a.nxi);
+  if constexpr (Q > 16)
+    if (poles > 16) return stability_dg<D, 32>(a, st);
+  if constexpr (Q > 8)
+    if (poles > 8) return stability_dg<D, 16>(a, st);
+  return stability_dg<D, 8>(a, st);
 }
 
 }  // namespace
 
 cudaError_t launch_stability(int d, const double *omega_dev, int64_t npoints, int32_t nxi, double s,
                              unsigned long long *rho_bits_dev, cudaStream_t st) {
-  int64_t nper = 1;
-  for (int i = 0; i < d; ++i) nper *= nxi;
-  const int64_t total = npoints * nper;
-  if (total <= 0) return cudaSuccess;
-  const unsigned blocks = (unsigned)((total + 127) / 128);
+  if (npoints <= 0) return cudaSuccess;
+  StabilityArgs a{};
+  a.omega = omega_dev;
+  a.rho_bits = rho_bits_dev;
+  a.npoints = npoints;
+  a.nxi = nxi;
+  a.s = s;
   switch (d) {
-    case 1: k_stability<1><<<blocks, 128, 0, st>>>(omega_dev, npoints, nxi, nper, s, rho_bits_dev); break;
-    case 2: k_stability<2><<<blocks, 128, 0, st>>>(omega_dev, npoints, nxi, nper, s, rho_bits_dev); break;
-    case 3: k_stability<3><<<blocks, 128, 0, st>>>(omega_dev, npoints, nxi, nper, s, rho_bits_dev); break;
-    case 4: k_stability<4><<<blocks, 128, 0, st>>>(omega_dev, npoints, nxi, nper, s, rho_bits_dev); break;
-    case 5: k_stability<5><<<blocks, 128, 0, st>>>(omega_dev, npoints, nxi, nper, s, rho_bits_dev); break;
+    case 1: return stability_d<1>(a, st);
+    case 2: return stability_d<2>(a, st);
+    case 3: return stability_d<3>(a, st);
+    case 4: return stability_d<4>(a, st);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 }  // namespace lhe
