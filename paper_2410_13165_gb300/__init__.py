@@ -178,7 +178,7 @@ class LBM:
     def set_boundary_jet(self, jet):
         """Jets of phi at boundary_points() for the next step: a float64 tensor of P * jet_len(d)
         values (every derivative of order 0..3 in (t, x_1..x_d), in the order of jet_index(d))."""
-        P = len(self.boundary_points()[0])
+        P = _abi.lhe_lbm_boundary_count(self.h)
         self._stream()
         _abi.lhe_lbm_set_boundary_jet(self.h, self._ptr(jet, P * jet_len(self.d), "jet"))
 
@@ -231,7 +231,7 @@ class LBM:
     def adjoint_jet_grad(self, out=None):
         """dL/d(jet) of the Dirichlet data of the step that the next adjoint_step(1) reverses, as a
         (P, jet_len(d)) float64 tensor at boundary_points() (lhe_lbm_adjoint_jet_grad)."""
-        P = len(self.boundary_points()[0])
+        P = _abi.lhe_lbm_boundary_count(self.h)
         JL = jet_len(self.d)
         if out is None:
             out = self._torch.empty((P, JL), dtype=self._torch.float64, device=self.device)

@@ -197,6 +197,13 @@ def lhe_lbm_set_boundary_sine_product(h, sp: lhe_sine_product) -> None:
     check(load().lhe_lbm_set_boundary_sine_product(h, ctypes.byref(sp)), h)
 
 
+def lhe_lbm_boundary_count(h) -> int:
+    """Number of points of lhe_lbm_boundary_points."""
+    P = ctypes.c_int64(0)
+    check(load().lhe_lbm_boundary_points(h, None, ctypes.byref(P), None), h)
+    return P.value
+
+
 def lhe_lbm_boundary_points(h, d: int):
     """(points[P][d], t_offset): where the Dirichlet jets of the next step are needed and the time of
     the data relative to the current step's time."""

@@ -334,18 +334,6 @@ void forget_steps_of(const lhe_lbm *l) {
   if (g_last_steps_handle == l) g_last_steps_handle = nullptr;
 }
 
-// The link k-bar with e_kbar = -e_k.
-int opposite_link(const lhe_lbm *l, int k) {
-  const int d = l->p.d;
-  for (int j = 0; j < l->Q; ++j) {
-    bool opp = true;
-    for (int i = 0; i < d; ++i)
-      if (l->e[j * d + i] != -l->e[k * d + i]) opp = false;
-    if (opp) return j;
-  }
-  return -1;
-}
-
 lhe_status check_handle(lhe_lbm *l) {
   if (!l) return fail(nullptr, LHE_ERR_ARG, "handle is NULL");
   return LHE_OK;
@@ -418,6 +406,13 @@ lhe_status lhe_lbm_create(const lhe_lbm_params *p, lhe_lbm **out) {
   std::memcpy(l->omega, m.omega, sizeof(m.omega));
   std::memcpy(l->m4, m.m4, sizeof(m.m4));
   std::memcpy(l->e, m.e, sizeof(m.e));
+  for (int k = 0; k < m.Q; ++k)
+    for (int j = 0; j < m.Q; ++j) {
+      bool opp = true;
+      for (int i = 0; i < p->d; ++i)
+        if (m.e[j * p->d + i] != -m.e[k * p->d + i]) opp = false;
+      if (opp) l->kbar[k] = (int8_t)j;
+    }
   std::memcpy(l->x0, m.x0, sizeof(m.x0));
   l->g = make_geom(p->d, p->n);
   l->stream = static_cast<cudaStream_t>(p->stream);
@@ -610,6 +605,8 @@ lhe_status lhe_lbm_destroy(lhe_lbm *l) {
   cudaFree(l->fdgrad);
   cudaFree(l->bsites);
   cudaFree(l->broff);
+  cudaFree(l->blinks);
+  cudaFree(l->bjetw);
   cudaFree(l->brec);
   cudaFree(l->sp_R0);
   cudaFree(l->sp_rec0);
@@ -766,13 +763,7 @@ lhe_status lhe_lbm_set_boundary_wave(lhe_lbm *l, const lhe_wave *w) {
   double gu = 0.0;
   for (int i = 0; i < d; ++i) gu += w->g[i] * l->p.u[i];
   for (int k = 0; k < Q; ++k) {
-    int kb = -1;
-    for (int j = 0; j < Q; ++j) {
-      bool opp = true;
-      for (int i = 0; i < d; ++i)
-        if (l->e[j * d + i] != -l->e[k * d + i]) opp = false;
-      if (opp) kb = j;
-    }
+    const int kb = l->kbar[k];
     double ge = 0.0;  // g . e_k
     for (int i = 0; i < d; ++i) ge += w->g[i] * l->e[k * d + i];
     const double wp = l->omega[k] + l->omega[kb], wm = l->omega[k] - l->omega[kb];
@@ -868,15 +859,8 @@ static BoundaryArgs boundary_args(const lhe_lbm *l) {
   b.axis_len = off;
   for (int k = 0; k < l->Q; ++k) {
     b.omega[k] = l->omega[k];
-    for (int j = 0; j < l->Q; ++j) {
-      bool opp = true;
-      for (int i = 0; i < l->p.d; ++i)
-        if (l->e[j * l->p.d + i] != -l->e[k * l->p.d + i]) opp = false;
-      if (opp) {
-        b.wratio[k] = l->omega[k] / l->omega[j];
-        b.kbar[k] = (int8_t)j;
-      }
-    }
+    b.wratio[k] = l->omega[k] / l->omega[l->kbar[k]];
+    b.kbar[k] = l->kbar[k];
   }
   b.nrow_ent = l->nrow_ent;
   b.s = l->s;
@@ -964,10 +948,73 @@ static std::vector<int16_t> jet_index_table(int d) {
   return jidx;
 }
 
-// The per-node offsets of the unknown populations (device) and the record buffer, on first use.
+// Weights of the derivatives of a jet in the record of each link (Eq. (bun1) / Eq. (bun2) as in k_jet_records), over
+// omega_k: what its cotangent rho_k is spread by.
+static std::vector<double> jet_weights(const lhe_lbm *l, const int16_t *jidx) {
+  const int d = l->p.d, P = l->p.bc_order;
+  const int JL = LHE_JET_LEN(d);
+  const double dt = l->dt;
+  std::vector<double> out((size_t)l->Q * JL, 0.0);
+  for (int k = 0; k < l->Q; ++k) {
+    double *g = &out[(size_t)k * JL];
+    double w[kMaxD + 1] = {1.0};
+    for (int i = 0; i < d; ++i) w[i + 1] = l->p.c * l->e[k * d + i];
+    const auto i2 = [&](int a, int b) { return jidx[216 + a * 6 + b]; };
+    const auto i3 = [&](int a, int b, int c) { return jidx[a * 36 + b * 6 + c]; };
+    if (l->p.bc == LHE_BC_FULLWAY) {
+      g[0] = 1.0;
+      for (int a = 0; a <= d; ++a) {
+        if (P >= 3) g[1 + a] -= 0.5 * dt * w[a];
+        for (int b = 0; b <= d; ++b)
+          for (int c = 0; c <= d; ++c)
+            if (P >= 4) g[i3(a, b, c)] += dt * dt * dt / 24.0 * w[a] * w[b] * w[c];
+      }
+      continue;
+    }
+    const double ratio = l->omega[l->kbar[k]] / l->omega[k], wp = 1.0 + ratio, wm = 1.0 - ratio;
+    g[0] = wp;
+    if (P >= 2) g[1] += 0.5 * dt * wp;
+    if (P >= 4) g[i3(0, 0, 0)] -= dt * dt * dt / 24.0 * wp;
+    for (int a = 1; a <= d; ++a) {
+      if (P >= 3) g[i2(a, 0)] -= dt * dt / 4.0 * wm * w[a];
+      if (P >= 4) g[i3(a, 0, 0)] -= dt * dt * dt / 8.0 * wm * w[a];
+      for (int b = 1; b <= d; ++b) {
+        if (P >= 3) g[i2(a, b)] -= dt * dt / 8.0 * wp * w[a] * w[b];
+        if (P >= 4) g[i3(a, b, 0)] -= dt * dt * dt / 16.0 * wp * w[a] * w[b];
+      }
+    }
+  }
+  return out;
+}
+
+// The tables of the unknown populations (device) and the record buffer, on first use.
 static lhe_status ensure_jet_buffers(lhe_lbm *l) {
-  if (l->broff) return LHE_OK;
-  LHE_CK(l, cudaMalloc((void **)&l->broff, sizeof(int32_t) * l->broff_host.size()));
+  if (l->brec) return LHE_OK;
+  const int d = l->p.d;
+  std::vector<int2> links;
+  links.reserve((size_t)l->nrec);
+  for (size_t j = 0; j < l->bsites_host.size(); ++j) {
+    int64_t r = l->bsites_host[j], idx[kMaxD];
+    for (int i = 0; i < d; ++i) {
+      idx[i] = r % l->p.n[i];
+      r /= l->p.n[i];
+    }
+    for (int k = 0; k < l->Q; ++k) {
+      bool unknown = false;
+      for (int i = 0; i < d; ++i) {
+        const int64_t src = idx[i] - l->e[k * d + i];
+        if (src < 0 || src >= l->p.n[i]) unknown = true;
+      }
+      if (unknown) links.push_back(make_int2((int)j, k));
+    }
+  }
+  l->jidx = jet_index_table(d);
+  const std::vector<double> w = jet_weights(l, l->jidx.data());
+  if (!l->blinks) LHE_CK(l, cudaMalloc((void **)&l->blinks, sizeof(int2) * std::max<size_t>(links.size(), 1)));
+  LHE_CK(l, cudaMemcpy(l->blinks, links.data(), sizeof(int2) * links.size(), cudaMemcpyHostToDevice));
+  if (!l->bjetw) LHE_CK(l, cudaMalloc((void **)&l->bjetw, sizeof(double) * w.size()));
+  LHE_CK(l, cudaMemcpy(l->bjetw, w.data(), sizeof(double) * w.size(), cudaMemcpyHostToDevice));
+  if (!l->broff) LHE_CK(l, cudaMalloc((void **)&l->broff, sizeof(int32_t) * l->broff_host.size()));
   LHE_CK(l, cudaMemcpy(l->broff, l->broff_host.data(), sizeof(int32_t) * l->broff_host.size(), cudaMemcpyHostToDevice));
   LHE_CK(l, cudaMalloc((void **)&l->brec, sizeof(double) * (size_t)std::max<int64_t>(l->nrec, 1)));
   return LHE_OK;
@@ -987,7 +1034,7 @@ lhe_status lhe_lbm_set_boundary_jet(lhe_lbm *l, const double *jet_dev) {
   // the schemes' R terms (a source varying in time): full-way at the new time t_{n+1} (the source of
   // this step's collision), half-way at t_n (the source of the collision of f*_kbar)
   b.Rfield = l->p.bc == LHE_BC_FULLWAY ? next_source(l) : l->Rfield;
-  LHE_CK(l, launch_jet_records(l->p.d, l->p.bc, b, jet_dev, jet_index_table(l->p.d).data(), l->brec, l->stream));
+  LHE_CK(l, launch_jet_records(l->p.d, l->p.bc, b, l->blinks, l->nrec, l->e, jet_dev, l->jidx.data(), l->brec, l->stream));
   l->jet_mode = true;
   l->jet_ready = true;
   l->sp_mode = false;
@@ -1059,7 +1106,7 @@ lhe_status lhe_lbm_set_boundary_sine_product(lhe_lbm *l, const lhe_sine_product 
     b.roff = l->broff;
     b.rmap = l->bmap;
     b.Rfield = l->sp_R0;  // data and source share the time factor in both schemes
-    e = launch_jet_records(d, l->p.bc, b, djet, jet_index_table(d).data(), l->sp_rec0, l->stream);
+    e = launch_jet_records(d, l->p.bc, b, l->blinks, l->nrec, l->e, djet, l->jidx.data(), l->sp_rec0, l->stream);
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(l->stream);
   release();
@@ -1083,7 +1130,7 @@ lhe_status lhe_lbm_adjoint_jet_grad(lhe_lbm *l, double *out) {
   b.roff = l->broff;
   b.src = l->adj[l->acur];
   b.phi_src = l->adjW[l->acur];
-  LHE_CK(l, launch_jet_grad(l->p.d, l->p.bc, l->p.precision == LHE_FP32_DEV, b, jet_index_table(l->p.d).data(), out,
+  LHE_CK(l, launch_jet_grad(l->p.d, l->p.bc, l->p.precision == LHE_FP32_DEV, b, l->blinks, l->nrec, l->bjetw, out,
                             l->stream));
   return LHE_OK;
 }
@@ -1171,7 +1218,7 @@ lhe_status lhe_lbm_step(lhe_lbm *l, int64_t n) {
         double gu = 0.0;
         for (int i = 0; i < d; ++i) gu += l->wave.g[i] * l->p.u[i];
         for (int k = 0; k < l->Q; ++k) {
-          const double wk = l->p.bc == LHE_BC_FULLWAY ? l->omega[k] : l->omega[k] + l->omega[opposite_link(l, k)];
+          const double wk = l->p.bc == LHE_BC_FULLWAY ? l->omega[k] : l->omega[k] + l->omega[l->kbar[k]];
           rest.lt[k] = wk * (l->R - gu) * rest.t_eval;
         }
       }

@@ -113,118 +113,122 @@ __global__ void __launch_bounds__(128) k_boundary(const BoundaryArgs a) {
 // R is the source at the node (the per-site field of the step, when there is one).
 // A jet holds every derivative of order <= 3 in (t, x_1..x_d); J.i3[a*36 + b*6 + e] and
 // J.i2[a*6 + b] give the position of the derivative in the variables a, b(, e) (0: t, i: x_i), in
-// any order.
-struct JetIndex {
+// any order. One thread per record (links[r]: the record's boundary node and link), so that a node's links, up to 40
+// dependent chains of up to 27 terms, run side by side: with a thread per node these chains were the whole
+// time of small boxes (D2Q9 48 x 40, 172 nodes, 516 records: 27.5 -> 8 us). The sums keep their order of terms.
+struct JetTables {
   int16_t i3[216];
   int16_t i2[36];
+  int8_t e[kMaxQ * kMaxD];
 };
 
 template <int D, int KIND>
-__global__ void __launch_bounds__(128) k_jet_records(const BoundaryArgs a, const double *__restrict__ jet,
-                                                     const JetIndex J, double *__restrict__ rec) {
-  constexpr Lattice<D> L{};
-  constexpr int Q = Lattice<D>::Q;
+__global__ void __launch_bounds__(64) k_jet_records(const BoundaryArgs a, const int2 *__restrict__ links, int64_t nrec,
+                                                    const double *__restrict__ jet, const JetTables T,
+                                                    double *__restrict__ rec) {
   constexpr int JL = (D + 4) * (D + 3) * (D + 2) / 6;
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= a.nsites) return;
-  const int32_t site = a.sites[t];
-  int x[D];
-  {
-    uint32_t r = (uint32_t)site;
-#pragma unroll
-    for (int i = 0; i < D; ++i) {
-      if (i == D - 1) {
-        x[i] = (int)r;
-      } else {
-        const uint32_t q = a.g.dv[i].div(r);
-        x[i] = (int)(r - q * (uint32_t)a.g.n[i]);
-        r = q;
-      }
-    }
-  }
-  const int32_t r0 = a.roff[t];
-  const int P = a.order;
+  __shared__ JetTables J;  // links differ within a warp: the parameter bank would serialise
+  for (int i = threadIdx.x; i < (int)(sizeof(JetTables) / 2); i += blockDim.x)
+    reinterpret_cast<int16_t *>(&J)[i] = reinterpret_cast<const int16_t *>(&T)[i];
+  __syncthreads();
+  const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (r >= nrec) return;
+  const int2 nk = __ldg(links + r);
+  const int k = nk.y, P = a.order;
   const double dt = a.dt;
-  const double R = a.Rfield ? a.Rfield[site] : a.R;  // the source at the node
-  int ju = 0;
-  for (int k = 0; k < Q; ++k) {
-    bool inside = true;
-    for (int i = 0; i < D; ++i) {
-      const int xs = x[i] - L.e[k][i];
-      if (xs < 0 || xs >= a.g.n[i]) inside = false;
+  const double R = a.Rfield ? a.Rfield[a.sites[nk.x]] : a.R;  // the source at the node
+  const double *__restrict__ j = jet + (size_t)(KIND == 1 ? nk.x : r) * JL;
+  double w[D + 1];  // weights of the variables in (d_t + c.grad): 1 for t, c_i for x_i
+  int var[3] = {0, 0, 0}, nv = 1;  // the variables of non-zero weight, t first
+  w[0] = 1.0;
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    const int e = J.e[k * D + i];
+    w[i + 1] = a.c * e;
+    if (e != 0) {
+      if (nv == 1) var[1] = i + 1;
+      else var[2] = i + 1;
+      ++nv;
     }
-    if (inside) continue;
-    const double *j = jet + (size_t)(KIND == 1 ? t : r0 + ju) * JL;
-    double w[D + 1];  // weights of the variables in (d_t + c.grad): 1 for t, c_i for x_i
-    w[0] = 1.0;
-    for (int i = 0; i < D; ++i) w[i + 1] = a.c * L.e[k][i];
-    double val;
-    if (KIND == 1) {
-      const double wk = a.omega[k];
-      val = wk * j[0];
-      if (P >= 3) {
-        double d1 = 0.0;
-        for (int v = 0; v <= D; ++v) d1 += w[v] * j[1 + v];
-        val = wk * (j[0] - 0.5 * dt * d1) + 0.5 * dt * wk * R;
-      }
-      if (P >= 4) {
-        double d3 = 0.0;
-        for (int p0 = 0; p0 <= D; ++p0)
-          for (int p1 = 0; p1 <= D; ++p1)
-            for (int p2 = 0; p2 <= D; ++p2) {
-              const double ww = w[p0] * w[p1] * w[p2];
-              if (ww != 0.0) d3 += ww * j[J.i3[p0 * 36 + p1 * 6 + p2]];
-            }
-        val += wk * dt * dt * dt / 24.0 * d3;
-      }
-    } else {
-      const int kb = L.opp[k];
-      const double wp = a.omega[k] + a.omega[kb], wm = a.omega[k] - a.omega[kb];
-      val = wp * j[0];
-      if (P >= 2) val += 0.5 * dt * wp * (j[1] + R);
-      if (P >= 3) {
-        double cch = 0.0, cgt = 0.0;
-        for (int p0 = 1; p0 <= D; ++p0) {
-          cgt += w[p0] * j[J.i2[p0 * 6]];
-          for (int p1 = 1; p1 <= D; ++p1) cch += w[p0] * w[p1] * j[J.i2[p0 * 6 + p1]];
-        }
-        val -= dt * dt / 8.0 * wp * cch + dt * dt / 4.0 * wm * cgt;
-      }
-      if (P >= 4) {
-        double ccht = 0.0, cgtt = 0.0;
-        for (int p0 = 1; p0 <= D; ++p0) {
-          cgtt += w[p0] * j[J.i3[p0 * 36]];
-          for (int p1 = 1; p1 <= D; ++p1) ccht += w[p0] * w[p1] * j[J.i3[p0 * 36 + p1 * 6]];
-        }
-        val -= dt * dt * dt / 16.0 * wp * ccht + dt * dt * dt / 24.0 * wp * j[J.i3[0]] + dt * dt * dt / 8.0 * wm * cgtt;
-      }
-    }
-    rec[a.rmap ? a.rmap[r0 + ju] : r0 + ju] = val;  // node-major, or in the order of the dense entries
-    ++ju;
   }
+  double val;
+  if (KIND == 1) {
+    const double wk = a.omega[k];
+    val = wk * j[0];
+    if (P >= 3) {
+      double d1 = 0.0;
+#pragma unroll
+      for (int v = 0; v <= D; ++v) d1 += w[v] * j[1 + v];
+      val = wk * (j[0] - 0.5 * dt * d1) + 0.5 * dt * wk * R;
+    }
+    if (P >= 4) {
+      double wv[3] = {1.0, 0.0, 0.0};
+#pragma unroll
+      for (int i = 1; i < 3; ++i) wv[i] = i < nv ? a.c * J.e[k * D + var[i] - 1] : 0.0;
+      double d3 = 0.0;
+#pragma unroll
+      for (int p0 = 0; p0 < 3; ++p0)
+#pragma unroll
+        for (int p1 = 0; p1 < 3; ++p1)
+#pragma unroll
+          for (int p2 = 0; p2 < 3; ++p2)
+            if (p0 < nv && p1 < nv && p2 < nv) {
+              const double ww = wv[p0] * wv[p1] * wv[p2];
+              d3 += ww * j[J.i3[var[p0] * 36 + var[p1] * 6 + var[p2]]];
+            }
+      val += wk * dt * dt * dt / 24.0 * d3;
+    }
+  } else {
+    const int kb = a.kbar[k];
+    const double wp = a.omega[k] + a.omega[kb], wm = a.omega[k] - a.omega[kb];
+    val = wp * j[0];
+    if (P >= 2) val += 0.5 * dt * wp * (j[1] + R);
+    if (P >= 3) {
+      double cch = 0.0, cgt = 0.0;
+#pragma unroll
+      for (int p0 = 1; p0 <= D; ++p0) {
+        cgt += w[p0] * j[J.i2[p0 * 6]];
+#pragma unroll
+        for (int p1 = 1; p1 <= D; ++p1) cch += w[p0] * w[p1] * j[J.i2[p0 * 6 + p1]];
+      }
+      val -= dt * dt / 8.0 * wp * cch + dt * dt / 4.0 * wm * cgt;
+    }
+    if (P >= 4) {
+      double ccht = 0.0, cgtt = 0.0;
+#pragma unroll
+      for (int p0 = 1; p0 <= D; ++p0) {
+        cgtt += w[p0] * j[J.i3[p0 * 36]];
+#pragma unroll
+        for (int p1 = 1; p1 <= D; ++p1) ccht += w[p0] * w[p1] * j[J.i3[p0 * 36 + p1 * 6]];
+      }
+      val -= dt * dt * dt / 16.0 * wp * ccht + dt * dt * dt / 24.0 * wp * j[J.i3[0]] + dt * dt * dt / 8.0 * wm * cgtt;
+    }
+  }
+  rec[a.rmap ? a.rmap[r] : r] = val;  // node-major, or in the order of the dense entries
 }
 
 template <int D>
-static cudaError_t jet_records_d(int kind, const BoundaryArgs &a, const double *jet, const JetIndex &J, double *rec,
-                                 cudaStream_t st) {
-  if (a.nsites <= 0) return cudaSuccess;
-  const unsigned blocks = (unsigned)((a.nsites + 127) / 128);
-  if (kind == 1) k_jet_records<D, 1><<<blocks, 128, 0, st>>>(a, jet, J, rec);
-  else k_jet_records<D, 2><<<blocks, 128, 0, st>>>(a, jet, J, rec);
+static cudaError_t jet_records_d(int kind, const BoundaryArgs &a, const int2 *links, int64_t nrec, const double *jet,
+                                 const JetTables &T, double *rec, cudaStream_t st) {
+  if (nrec <= 0) return cudaSuccess;
+  const unsigned blocks = (unsigned)((nrec + 63) / 64);
+  if (kind == 1) k_jet_records<D, 1><<<blocks, 64, 0, st>>>(a, links, nrec, jet, T, rec);
+  else k_jet_records<D, 2><<<blocks, 64, 0, st>>>(a, links, nrec, jet, T, rec);
   return cudaGetLastError();
 }
 
-cudaError_t launch_jet_records(int d, int kind, const BoundaryArgs &a, const double *jet, const int16_t *jidx,
-                               double *rec, cudaStream_t st) {
-  JetIndex J;
-  for (int i = 0; i < 216; ++i) J.i3[i] = jidx[i];
-  for (int i = 0; i < 36; ++i) J.i2[i] = jidx[216 + i];
+cudaError_t launch_jet_records(int d, int kind, const BoundaryArgs &a, const int2 *links, int64_t nrec, const int32_t *e,
+                               const double *jet, const int16_t *jidx, double *rec, cudaStream_t st) {
+  JetTables T{};
+  for (int i = 0; i < 216; ++i) T.i3[i] = jidx[i];
+  for (int i = 0; i < 36; ++i) T.i2[i] = jidx[216 + i];
+  for (int i = 0; i < (2 * d * d + 1) * d; ++i) T.e[i] = (int8_t)e[i];
   switch (d) {
-    case 1: return jet_records_d<1>(kind, a, jet, J, rec, st);
-    case 2: return jet_records_d<2>(kind, a, jet, J, rec, st);
-    case 3: return jet_records_d<3>(kind, a, jet, J, rec, st);
-    case 4: return jet_records_d<4>(kind, a, jet, J, rec, st);
-    case 5: return jet_records_d<5>(kind, a, jet, J, rec, st);
+    case 1: return jet_records_d<1>(kind, a, links, nrec, jet, T, rec, st);
+    case 2: return jet_records_d<2>(kind, a, links, nrec, jet, T, rec, st);
+    case 3: return jet_records_d<3>(kind, a, links, nrec, jet, T, rec, st);
+    case 4: return jet_records_d<4>(kind, a, links, nrec, jet, T, rec, st);
+    case 5: return jet_records_d<5>(kind, a, links, nrec, jet, T, rec, st);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -232,116 +236,58 @@ cudaError_t launch_jet_records(int d, int kind, const BoundaryArgs &a, const dou
 // Cotangent of the jets of one Dirichlet step (lhe_lbm_adjoint_jet_grad): the transpose of
 // k_jet_records. a.src holds the adjoint state rho_k(x) = omega_k dL/df_k(x) of the pre-collision
 // populations that the step produced, so the cotangent of an unknown population's value is
-// rho_k / omega_k (the R terms and the half-way -f*_kbar do not depend on the jets). Full-way: one row
-// per boundary node, summed over its unknown links (omega_k times the cotangent is rho_k); half-way:
-// one row per unknown population, w+ and w- times rho_k / omega_k. Each thread owns the rows of its
-// node and zeroes them first. FP32 deviations (DEV): rho_k = omega_k W + eps_k.
+// rho_k / omega_k (the R terms and the half-way -f*_kbar do not depend on the jets). The records are linear in
+// the jets with weights that depend on the link alone: w[k JL + q] is the weight of derivative q in the record of link k, over
+// omega_k (formed once per handle). Full-way: one row per boundary node, summed over its unknown links;
+// half-way: one row per unknown population. One thread per entry of the result, so that the weights and the
+// result are read and written contiguously (a thread per node walked its links and up to 84 derivatives
+// in turn: D2Q9 48 x 40 26.3 -> 4.8 us). FP32 deviations (DEV): rho_k = omega_k W + eps_k.
 template <int D, int KIND, bool DEV>
-__global__ void __launch_bounds__(128) k_jet_grad(const BoundaryArgs a, const JetIndex J, double *__restrict__ out) {
-  constexpr Lattice<D> L{};
-  constexpr int Q = Lattice<D>::Q;
+__global__ void __launch_bounds__(128) k_jet_grad(const BoundaryArgs a, const int2 *__restrict__ links, int64_t nrec,
+                                                  const double *__restrict__ w, double *__restrict__ out) {
   constexpr int JL = (D + 4) * (D + 3) * (D + 2) / 6;
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= a.nsites) return;
-  const int32_t site = a.sites[t];
-  int x[D];
-  {
-    uint32_t r = (uint32_t)site;
-#pragma unroll
-    for (int i = 0; i < D; ++i) {
-      if (i == D - 1) {
-        x[i] = (int)r;
-      } else {
-        const uint32_t q = a.g.dv[i].div(r);
-        x[i] = (int)(r - q * (uint32_t)a.g.n[i]);
-        r = q;
-      }
-    }
-  }
-  const double *__restrict__ rho = static_cast<const double *>(a.src);
+  const int64_t row = t / JL;
+  const int q = (int)(t - row * JL);
+  if (row >= (KIND == 1 ? a.nsites : nrec)) return;
   const int64_t S = a.g.S;
-  const int32_t r0 = a.roff[t];
-  const int P = a.order;
-  const double dt = a.dt;
-  if (KIND == 1)
-    for (int e = 0; e < JL; ++e) out[t * JL + e] = 0.0;
-  int ju = 0;
-  for (int k = 0; k < Q; ++k) {
-    bool inside = true;
-    for (int i = 0; i < D; ++i) {
-      const int xs = x[i] - L.e[k][i];
-      if (xs < 0 || xs >= a.g.n[i]) inside = false;
-    }
-    if (inside) continue;
-    double *g = out + (size_t)(KIND == 1 ? t : r0 + ju) * JL;
-    double w[D + 1];  // weights of the variables in (d_t + c.grad): 1 for t, c_i for x_i
-    w[0] = 1.0;
-    for (int i = 0; i < D; ++i) w[i + 1] = a.c * L.e[k][i];
-    const double rk = DEV ? fma(a.omega[k], df_value(a.phi_src[site]), (double)static_cast<const float *>(a.src)[k * S + site])
-                          : rho[k * S + site];
-    if (KIND == 1) {
-      g[0] += rk;
-      if (P >= 3)
-        for (int v = 0; v <= D; ++v) g[1 + v] -= 0.5 * dt * w[v] * rk;
-      if (P >= 4) {
-        const double c3 = dt * dt * dt / 24.0 * rk;
-        for (int p0 = 0; p0 <= D; ++p0)
-          for (int p1 = 0; p1 <= D; ++p1)
-            for (int p2 = 0; p2 <= D; ++p2) {
-              const double ww = w[p0] * w[p1] * w[p2];
-              if (ww != 0.0) g[J.i3[p0 * 36 + p1 * 6 + p2]] += ww * c3;
-            }
-      }
-    } else {
-      for (int e = 0; e < JL; ++e) g[e] = 0.0;
-      const int kb = L.opp[k];
-      const double lam = rk / a.omega[k];
-      const double wp = (a.omega[k] + a.omega[kb]) * lam, wm = (a.omega[k] - a.omega[kb]) * lam;
-      g[0] = wp;
-      if (P >= 2) g[1] += 0.5 * dt * wp;
-      if (P >= 3)
-        for (int p0 = 1; p0 <= D; ++p0) {
-          g[J.i2[p0 * 6]] -= dt * dt / 4.0 * wm * w[p0];
-          for (int p1 = 1; p1 <= D; ++p1) g[J.i2[p0 * 6 + p1]] -= dt * dt / 8.0 * wp * w[p0] * w[p1];
-        }
-      if (P >= 4) {
-        g[J.i3[0]] -= dt * dt * dt / 24.0 * wp;
-        for (int p0 = 1; p0 <= D; ++p0) {
-          g[J.i3[p0 * 36]] -= dt * dt * dt / 8.0 * wm * w[p0];
-          for (int p1 = 1; p1 <= D; ++p1) g[J.i3[p0 * 36 + p1 * 6]] -= dt * dt * dt / 16.0 * wp * w[p0] * w[p1];
-        }
-      }
-    }
-    ++ju;
+  const int64_t r0 = KIND == 1 ? a.roff[row] : row;
+  const int64_t r1 = KIND == 1 ? (row + 1 < a.nsites ? a.roff[row + 1] : nrec) : row + 1;
+  double acc = 0.0;
+  for (int64_t r = r0; r < r1; ++r) {
+    const int2 nk = __ldg(links + r);
+    const int32_t site = a.sites[nk.x];
+    const double rk = DEV ? fma(a.omega[nk.y], df_value(a.phi_src[site]), (double)static_cast<const float *>(a.src)[nk.y * S + site])
+                          : static_cast<const double *>(a.src)[nk.y * S + site];
+    acc = fma(__ldg(w + nk.y * JL + q), rk, acc);
   }
+  out[t] = acc;
 }
 
 template <int D>
-static cudaError_t jet_grad_d(int kind, bool dev, const BoundaryArgs &a, const JetIndex &J, double *out,
-                              cudaStream_t st) {
-  if (a.nsites <= 0) return cudaSuccess;
-  const unsigned blocks = (unsigned)((a.nsites + 127) / 128);
+static cudaError_t jet_grad_d(int kind, bool dev, const BoundaryArgs &a, const int2 *links, int64_t nrec,
+                              const double *w, double *out, cudaStream_t st) {
+  if (nrec <= 0) return cudaSuccess;
+  constexpr int64_t JL = (D + 4) * (D + 3) * (D + 2) / 6;
+  const unsigned blocks = (unsigned)(((kind == 1 ? a.nsites : nrec) * JL + 127) / 128);
   if (kind == 1) {
-    if (dev) k_jet_grad<D, 1, true><<<blocks, 128, 0, st>>>(a, J, out);
-    else k_jet_grad<D, 1, false><<<blocks, 128, 0, st>>>(a, J, out);
+    if (dev) k_jet_grad<D, 1, true><<<blocks, 128, 0, st>>>(a, links, nrec, w, out);
+    else k_jet_grad<D, 1, false><<<blocks, 128, 0, st>>>(a, links, nrec, w, out);
   } else {
-    if (dev) k_jet_grad<D, 2, true><<<blocks, 128, 0, st>>>(a, J, out);
-    else k_jet_grad<D, 2, false><<<blocks, 128, 0, st>>>(a, J, out);
+    if (dev) k_jet_grad<D, 2, true><<<blocks, 128, 0, st>>>(a, links, nrec, w, out);
+    else k_jet_grad<D, 2, false><<<blocks, 128, 0, st>>>(a, links, nrec, w, out);
   }
   return cudaGetLastError();
 }
 
-cudaError_t launch_jet_grad(int d, int kind, bool dev, const BoundaryArgs &a, const int16_t *jidx, double *out,
-                            cudaStream_t st) {
-  JetIndex J;
-  for (int i = 0; i < 216; ++i) J.i3[i] = jidx[i];
-  for (int i = 0; i < 36; ++i) J.i2[i] = jidx[216 + i];
+cudaError_t launch_jet_grad(int d, int kind, bool dev, const BoundaryArgs &a, const int2 *links, int64_t nrec,
+                            const double *w, double *out, cudaStream_t st) {
   switch (d) {
-    case 1: return jet_grad_d<1>(kind, dev, a, J, out, st);
-    case 2: return jet_grad_d<2>(kind, dev, a, J, out, st);
-    case 3: return jet_grad_d<3>(kind, dev, a, J, out, st);
-    case 4: return jet_grad_d<4>(kind, dev, a, J, out, st);
-    case 5: return jet_grad_d<5>(kind, dev, a, J, out, st);
+    case 1: return jet_grad_d<1>(kind, dev, a, links, nrec, w, out, st);
+    case 2: return jet_grad_d<2>(kind, dev, a, links, nrec, w, out, st);
+    case 3: return jet_grad_d<3>(kind, dev, a, links, nrec, w, out, st);
+    case 4: return jet_grad_d<4>(kind, dev, a, links, nrec, w, out, st);
+    case 5: return jet_grad_d<5>(kind, dev, a, links, nrec, w, out, st);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -199,10 +199,12 @@ struct AdjGradArgs {
 cudaError_t launch_step_fp64(int d, bool adjoint, bool interior, const StepArgs &a, cudaStream_t st);
 cudaError_t launch_step_dev(int d, bool adjoint, bool interior, const StepArgs &a, cudaStream_t st);
 cudaError_t launch_boundary(int d, int kind, bool dev, const BoundaryArgs &a, cudaStream_t st);
-cudaError_t launch_jet_records(int d, int kind, const BoundaryArgs &a, const double *jet, const int16_t *jidx,
-                               double *rec, cudaStream_t st);
-cudaError_t launch_jet_grad(int d, int kind, bool dev, const BoundaryArgs &a, const int16_t *jidx, double *out,
-                            cudaStream_t st);
+// links[r]: boundary node (position in the node list) and link of record r; e: the lattice vectors; w: the weights of a
+// record's derivatives per link, over omega_k (lhe_boundary.cu).
+cudaError_t launch_jet_records(int d, int kind, const BoundaryArgs &a, const int2 *links, int64_t nrec, const int32_t *e,
+                               const double *jet, const int16_t *jidx, double *rec, cudaStream_t st);
+cudaError_t launch_jet_grad(int d, int kind, bool dev, const BoundaryArgs &a, const int2 *links, int64_t nrec,
+                            const double *w, double *out, cudaStream_t st);
 cudaError_t launch_sp_jets(int d, const SineProductArgs &a, const double *pts, int64_t P, const int8_t *tup,
                            double *jet, cudaStream_t st);
 cudaError_t launch_sp_source(const SineProductArgs &a, const Geom &g, double *R0, cudaStream_t st);
@@ -253,6 +255,7 @@ struct lhe_lbm {
   double omega[lhe::kMaxQ] = {};
   double m4[10] = {};
   int32_t e[lhe::kMaxQ * lhe::kMaxD] = {};
+  int8_t kbar[lhe::kMaxQ] = {};  // the link opposite to k
   double x0[lhe::kMaxD] = {};
   cudaStream_t stream = nullptr;
   int sms = 0;                  // multiprocessors of the device
@@ -292,10 +295,13 @@ struct lhe_lbm {
   bool jet_mode = false;        // the data come from jets (else from the wave)
   bool jet_ready = false;       // jets set for the next step
   std::vector<int32_t> bsites_host;  // boundary nodes in the library's order
+  std::vector<int16_t> jidx;         // positions of the derivatives in a jet (jet_index_table)
   std::vector<int32_t> broff_host;   // per boundary node: first record (unknown links in the order of k)
   int64_t nrec = 0;             // records = (boundary node, unknown link) pairs
   int64_t nrow_ent = 0;         // dense boundary data: entries of row links (the first ones)
   int32_t *broff = nullptr;     // device copies, allocated by the first lhe_lbm_set_boundary_jet
+  int2 *blinks = nullptr;       // per record: its boundary node (position in bsites) and link
+  double *bjetw = nullptr;      // per link: the weights of the jet's derivatives in its record, over omega_k
   double *brec = nullptr;
   // lhe_lbm_set_boundary_sine_product: records and source at unit time factor, scaled every step
   bool sp_mode = false;
