@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(256) k_adj_grads(const AdjGradArgs a) {
     top = max(top, DEV ? ((unsigned)__float_as_int((float)z[k]) >> 23) & 0xFFu : (unsigned)__double2hiint((double)z[k]) & kExpField);
   }
   double Z = 0.0, E[D];
-  if (top == (DEV ? 0xFFu : kExpField)) {  // infinities or NaN: the floating sums
+  if (top == (DEV ? 0xFFu : kExpField) || (!DEV && top < kFixedLeast)) {  // plain sums (infinities, NaN, and values below 2^-954)
 #pragma unroll
     for (int i = 0; i < D; ++i) E[i] = 0.0;
 #pragma unroll
@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(256) k_adj_grads(const AdjGradArgs a) {
     }
   } else {
     constexpr int G = 10 - ceil_log2(Q);
-    const unsigned emf = DEV ? (max(top, 1u) + 896u) << 20 : max(top, 0x00100000u);
+    const unsigned emf = DEV ? (max(top, 1u) + 896u) << 20 : top;
     long long accz = 0, acce[D];
 #pragma unroll
     for (int i = 0; i < D; ++i) acce[i] = 0;
