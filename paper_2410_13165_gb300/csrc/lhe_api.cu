@@ -198,6 +198,7 @@ StepArgs step_args(const lhe_lbm *l) {
   a.gsc = a.dt;
   a.pscale = 1.0;
   a.pdl = 0;
+  a.sms = l->sms;
   return a;
 }
 

@@ -281,10 +281,18 @@ __device__ __forceinline__ float2 ff_split(double x) {
 __device__ __forceinline__ void st_stream(double *p, double v) { *p = v; }
 __device__ __forceinline__ void st_stream(float *p, float v) { *p = v; }
 
-// Programmatic dependent launch. A step kernel lets the next kernel of its stream be scheduled as
-// soon as every CTA of this one is running (pdl_trigger), and waits for the kernel before it to
+// Programmatic dependent launch. A step kernel lets the next kernel of its stream be scheduled once
+// every CTA of this one has reached pdl_trigger, and waits for the kernel before it to
 // complete, with its memory visible, before it touches global memory (pdl_wait). When the kernel was
-// launched without the programmatic-serialization attribute both are no-ops.
+// launched without the programmatic-serialization attribute both are no-ops. A trigger on entry puts the
+// next grid's CTAs wherever a place is left beside this grid's, so that a grid of about one wave ends up
+// two deep on some SMs. The register kernels therefore trigger just before their stores; the FP64 step, in grids of
+// about one wave (at most kTriggerCtasPerSM CTAs per SM), not before it ends. us per step with the trigger on entry /
+// before the stores / at the end: FP64 D2Q9 256^2 5.93 / 3.93 / 3.66, 500 x 333 (8.6 CTAs per SM) 7.16 / 6.76 / 6.01,
+// 1000^2 (51) 23.7 / 23.4 / 25.3, D3Q19 32^3 8.94 / 4.86 / 4.03, 45 x 37 x 51 9.52 / 8.12 / 6.87, 64^3 (13.5) 13.5 / 13.5 / 14.0;
+// 128^3 and larger the same (the adjoint, which also updates dL/dR, is faster with the trigger at the end at every size:
+// 64^3 13.7 / 13.3, 128^3 100.4 / 99.2); FP32 deviations the same before the stores and at the end. (A run-time choice in
+// one kernel measured like the trigger at the end everywhere, so the two are separate instantiations.)
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

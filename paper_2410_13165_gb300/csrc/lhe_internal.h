@@ -46,6 +46,7 @@ struct StepArgs {
   double mu, sig, rho_dt, rho_dtR, gsc;
   double pscale;           // macro: factor from the stored populations to f* (1 unless scaled)
   int32_t collide;         // kCollideGeneral / kCollideScaled (s != 2 only)
+  int32_t sms;             // multiprocessors of the device
   int32_t pdl;             // launch with programmatic stream serialization (the kernel calls pdl_wait)
   int64_t nwork;           // number of sites processed (S, or the interior count)
 };
@@ -68,6 +69,9 @@ cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_
   cfg.numAttrs = pdl ? 1u : 0u;
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
+
+// Grids of at most this many CTAs per SM let their successor start only when they end (lhe_device.cuh).
+constexpr int64_t kTriggerCtasPerSM = 10;
 
 // Plan of the staged FP32-deviation step on periodic D3Q19 boxes (lhe_step_dev_tma.cu).
 constexpr int kTmaMaxStages = 4;

@@ -74,7 +74,6 @@ __global__ void __launch_bounds__(LHE_STEP_THREADS) k_step_box(const StepArgs a,
   constexpr Lattice<D> L{};
   constexpr int Q = Lattice<D>::Q;
   constexpr int J = 2 * D - 1;
-  pdl_trigger();
   pdl_wait();
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= a.nwork) return;
@@ -100,6 +99,7 @@ __global__ void __launch_bounds__(LHE_STEP_THREADS) k_step_box(const StepArgs a,
   const double sum = split_moment_sum<Q, kBoxFixedTerms<Q>>(f);  // the split moment sum of the larger lattices (lhe_device.cuh)
   const double psi = MODE == kModeS2 ? fma(2.0, sum, a.Rfield ? a.dt * Rs : a.dtR)
                                      : fma(a.sig, sum, a.Rfield ? a.rho_dt * Rs : a.rho_dtR);
+  pdl_trigger();
 #pragma unroll
   for (int k = 0; k < Q; ++k) {
     const double out = MODE == kModeS2 ? fma(a.omega[k], psi, -f[k]) : fma(a.omega[k], psi, a.mu * f[k]);
@@ -263,7 +263,6 @@ template <int D, int MODE>
 __global__ void __launch_bounds__(LHE_STEP_THREADS) k_step_box_dense(const StepArgs a, const double *__restrict__ bdata) {
   constexpr Lattice<D> L{};
   constexpr int Q = Lattice<D>::Q;
-  pdl_trigger();
   pdl_wait();
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= a.nwork) return;
@@ -294,6 +293,7 @@ __global__ void __launch_bounds__(LHE_STEP_THREADS) k_step_box_dense(const StepA
   const double sum = split_moment_sum<Q, kBoxFixedTerms<Q>>(f);
   const double psi = MODE == kModeS2 ? fma(2.0, sum, a.Rfield ? a.dt * Rs : a.dtR)
                                      : fma(a.sig, sum, a.Rfield ? a.rho_dt * Rs : a.rho_dtR);
+  pdl_trigger();
 #pragma unroll
   for (int k = 0; k < Q; ++k) {
     const double out = MODE == kModeS2 ? fma(a.omega[k], psi, -f[k]) : fma(a.omega[k], psi, a.mu * f[k]);

@@ -36,7 +36,6 @@ template <int D, bool ADJ, bool INTERIOR, bool S2>
 __global__ void __launch_bounds__(LHE_STEP_THREADS, dev_min_blocks<D>()) k_step_dev(const StepArgs a) {
   constexpr Lattice<D> L{};
   constexpr int Q = Lattice<D>::Q;
-  pdl_trigger();
   pdl_wait();
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= a.nwork) return;
@@ -74,6 +73,7 @@ __global__ void __launch_bounds__(LHE_STEP_THREADS, dev_min_blocks<D>()) k_step_
   if (ADJ && a.gR) a.gR[site] = fma(a.dt, df_value(pn), a.gR[site]);
   float dtR = 0.0f;
   if (field) dtR = (float)(a.dt * __ldg(a.Rfield + site));
+  pdl_trigger();
 #pragma unroll
   for (int k = 0; k < Q; ++k) {
     const float r = fmaf(a.omega_f[k], dl[k] - Delta, gk[k]);  // pre-collision deviation g_k

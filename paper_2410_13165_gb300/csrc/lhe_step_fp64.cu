@@ -20,11 +20,11 @@ namespace lhe {
 // Template collision forms: s = 2, general s (mu, sig, rho from StepArgs), scaled representation.
 constexpr int kModeGeneral = 0, kModeS2 = 1, kModeScaled = 2;
 
-template <int D, bool ADJ, bool INTERIOR, int MODE>
+// TRIGGER: let the next step kernel be scheduled before the stores (else at the end; lhe_device.cuh).
+template <int D, bool ADJ, bool INTERIOR, int MODE, bool TRIGGER>
 __global__ void __launch_bounds__(LHE_STEP_THREADS) k_step_fp64(const StepArgs a) {
   constexpr Lattice<D> L{};
   constexpr int Q = Lattice<D>::Q;
-  pdl_trigger();
   pdl_wait();
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= a.nwork) return;
@@ -64,6 +64,7 @@ __global__ void __launch_bounds__(LHE_STEP_THREADS) k_step_fp64(const StepArgs a
   } else {
     psi = fma(a.sig, fixed_moment_sum<Q, 0>(f), a.Rfield ? a.rho_dt * __ldg(a.Rfield + site) : a.rho_dtR);
   }
+  if constexpr (TRIGGER) pdl_trigger();
 #pragma unroll
   for (int k = 0; k < Q; ++k) {
     const double out = MODE == kModeS2      ? fma(a.omega[k], psi, -f[k])
@@ -88,16 +89,25 @@ __global__ void __launch_bounds__(256) k_macro_fp64(const StepArgs a, double *__
   phi[t] = fma(fixed_moment_sum<Q, 0>(f), a.pscale, -dtR);
 }
 
+template <int D, bool ADJ, bool INTERIOR, bool TRIGGER>
+static cudaError_t launch_step_fp64_m(const StepArgs &a, unsigned blocks, cudaStream_t st) {
+  const int threads = LHE_STEP_THREADS;
+  const bool pdl = a.pdl != 0;
+  if (a.s == 2.0) return launch_kernel(k_step_fp64<D, ADJ, INTERIOR, kModeS2, TRIGGER>, blocks, threads, 0, st, pdl, a);
+  if (a.collide == kCollideScaled)
+    return launch_kernel(k_step_fp64<D, ADJ, INTERIOR, kModeScaled, TRIGGER>, blocks, threads, 0, st, pdl, a);
+  return launch_kernel(k_step_fp64<D, ADJ, INTERIOR, kModeGeneral, TRIGGER>, blocks, threads, 0, st, pdl, a);
+}
+
 template <int D, bool ADJ, bool INTERIOR>
 static cudaError_t launch_step_fp64_t(const StepArgs &a, cudaStream_t st) {
   if (a.nwork <= 0) return cudaSuccess;
-  const int threads = LHE_STEP_THREADS;
-  const unsigned blocks = (unsigned)((a.nwork + threads - 1) / threads);
-  const bool pdl = a.pdl != 0;
-  if (a.s == 2.0) return launch_kernel(k_step_fp64<D, ADJ, INTERIOR, kModeS2>, blocks, threads, 0, st, pdl, a);
-  if (a.collide == kCollideScaled)
-    return launch_kernel(k_step_fp64<D, ADJ, INTERIOR, kModeScaled>, blocks, threads, 0, st, pdl, a);
-  return launch_kernel(k_step_fp64<D, ADJ, INTERIOR, kModeGeneral>, blocks, threads, 0, st, pdl, a);
+  const unsigned blocks = (unsigned)((a.nwork + LHE_STEP_THREADS - 1) / LHE_STEP_THREADS);
+  if constexpr (!INTERIOR) {
+    if (ADJ || (int64_t)blocks <= kTriggerCtasPerSM * a.sms) return launch_step_fp64_m<D, ADJ, false, false>(a, blocks, st);
+  }
+  if constexpr (INTERIOR || !ADJ) return launch_step_fp64_m<D, ADJ, INTERIOR, true>(a, blocks, st);
+  return cudaErrorInvalidValue;  // not reached
 }
 
 template <int D>
