@@ -75,7 +75,8 @@ typedef enum { LHE_M4_RULE = 0, LHE_M4_EXPLICIT = 1 } lhe_m4_mode;
 /* lhe_lbm_params.flags. LHE_FLAG_NO_STAGING: run the FP32-deviation step of periodic D3Q19 boxes
  * with the register-pull kernel instead of the one that stages the pulled rows in shared memory
  * by bulk asynchronous copies (both compute the same bits; the staged one is the default where
- * its layout conditions hold: n_1 a multiple of 4 and at most 512). */
+ * its layout conditions hold, n_1 a multiple of 4 and at most 512, and it is the faster one: large
+ * grids whose rows fill its tiles). */
 #define LHE_FLAG_NO_STAGING 1
 /* LHE_FLAG_NO_PDL: launch every step kernel with plain stream ordering. By default the second and
  * later step kernels of one lhe_lbm_step / lhe_lbm_adjoint_step call are launched with programmatic

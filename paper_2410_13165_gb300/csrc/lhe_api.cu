@@ -574,7 +574,8 @@ lhe_status lhe_lbm_create(const lhe_lbm_params *p, lhe_lbm **out) {
   }
   if (p->d == 3 && p->bc == LHE_BC_PERIODIC && p->precision == LHE_FP32_DEV && !(p->flags & LHE_FLAG_NO_STAGING)) {
     const int sms = l->sms;
-    if (sms > 0 && plan_dev3_tma(l->g, sms, l->tma)) {
+    if (sms > 0 && plan_dev3_tma(l->g, sms, l->tma) &&
+        ((p->flags & LHE_FLAG_TEST_EXPIRE_WAIT) || staged_pays(l->tma, false) || staged_pays(l->tma, true))) {
       e = cudaHostAlloc((void **)&l->tma_err_host, sizeof(int32_t), cudaHostAllocMapped);
       if (e != cudaSuccess) return bail(cuda_fail(l, e, "cudaHostAlloc(pipeline flag)"));
       *l->tma_err_host = 0;
@@ -582,7 +583,9 @@ lhe_status lhe_lbm_create(const lhe_lbm_params *p, lhe_lbm **out) {
       if (e != cudaSuccess) return bail(cuda_fail(l, e, "cudaHostGetDevicePointer(pipeline flag)"));
       e = prepare_dev3_tma(l->tma);
       if (e != cudaSuccess) return bail(cuda_fail(l, e, "shared-memory size of the staged step"));
-      l->staged = true;
+      const bool hook = (p->flags & LHE_FLAG_TEST_EXPIRE_WAIT) != 0;
+      l->staged[0] = hook || staged_pays(l->tma, false);
+      l->staged[1] = hook || staged_pays(l->tma, true);
       l->tma_expire_armed = (p->flags & LHE_FLAG_TEST_EXPIRE_WAIT) != 0;
     }
   }
@@ -1229,7 +1232,7 @@ lhe_status lhe_lbm_step(lhe_lbm *l, int64_t n) {
       e = launch_step_box_dense(d, a, l->bdata, l->stream);
       if (e != cudaSuccess) return cuda_fail(l, e, "step kernel launch");
     } else {
-      e = l->staged ? launch_step_dev3_tma(false, a, staged_plan(l), l->stream)
+      e = l->staged[0] ? launch_step_dev3_tma(false, a, staged_plan(l), l->stream)
           : fused   ? launch_step_box_fp64(d, l->p.bc, a, rest, l->xface, l->g.S_rows / l->g.n[0], l->stream)
           : dev     ? launch_step_dev(d, false, !periodic, a, l->stream)
                     : launch_step_fp64(d, false, !periodic, a, l->stream);
@@ -1376,7 +1379,7 @@ lhe_status lhe_lbm_adjoint_step(lhe_lbm *l, int64_t n) {
     a.phi_src = l->adjW[l->acur];
     a.phi_dst = l->adjW[1 - l->acur];
     a.pdl = (it > 0 || chained) && pdl_ok(l);
-    cudaError_t e = l->staged ? launch_step_dev3_tma(true, a, staged_plan(l), l->stream)
+    cudaError_t e = l->staged[1] ? launch_step_dev3_tma(true, a, staged_plan(l), l->stream)
                     : dev         ? launch_step_dev(l->p.d, true, !periodic, a, l->stream)
                                   : launch_step_fp64(l->p.d, true, !periodic, a, l->stream);
     if (e != cudaSuccess) return cuda_fail(l, e, "adjoint step kernel launch");

@@ -241,6 +241,7 @@ cudaError_t launch_adjoint_seed(int d, bool dev, const Geom &g, const double *om
 cudaError_t launch_df_to_double(const float2 *src, double *dst, int64_t n, cudaStream_t st);
 cudaError_t launch_scale_fp64(double *p, int64_t n, double factor, cudaStream_t st);
 bool plan_dev3_tma(const Geom &g, int sms, DevTmaPlan &p);
+bool staged_pays(const DevTmaPlan &p, bool adjoint);
 cudaError_t prepare_dev3_tma(const DevTmaPlan &p);
 cudaError_t launch_step_dev3_tma(bool adjoint, const StepArgs &a, const DevTmaPlan &p, cudaStream_t st);
 cudaError_t launch_adjoint_grads(int d, bool dev, const AdjGradArgs &a, cudaStream_t st);
@@ -324,7 +325,7 @@ struct lhe_lbm {
   // are K f* with K = (1 - s)^-j; j = 0 means the state is stored as f* itself. [0] forward, [1]
   // adjoint. acc accumulates the relative error of the rounded s/(1 - s) factors.
   // staged FP32-deviation step (periodic D3Q19)
-  bool staged = false;
+  bool staged[2] = {false, false};  // forward, adjoint
   lhe::DevTmaPlan tma{};
   int32_t *tma_err_host = nullptr;
   bool tma_expire_armed = false; // LHE_FLAG_TEST_EXPIRE_WAIT: the next staged launch gives up its waits

@@ -361,6 +361,18 @@ bool plan_dev3_tma(const Geom &g, int sms, DevTmaPlan &p) {
   return true;
 }
 
+// Whether the staged kernel beats the register kernel, which reads the pulled rows through L1 and L2: it pays
+// where the state leaves L2 and its tiles are full. us per step, staged / register (the register kernel won by up to
+// 2.7 x on small grids): forward 64^3 13.6 / 6.4, 96^3 36.5 / 26.9, 160^3 161 / 117, 224^3 325 / 321 (rows of runtime
+// length: never ahead); 128 x 128 x 96 46.1 / 45.9, 128^3 58.6 / 60.5, 256 x 64 x 32 16.3 / 12.8, 256 x 64^2 30.4 / 31.7, 256^3 413 / 469.
+// Adjoint: 64^3 13.9 / 7.0, 256 x 64 x 32 17.9 / 15.4, 128^2 x 64 33.3 / 36.8, 192^3 (tiles of 384 nodes) 237 / 232, 200^3 (400)
+// 258 / 264, 256^3 458 / 543.
+bool staged_pays(const DevTmaPlan &p, bool adjoint) {
+  const int64_t S = (int64_t)p.nx * p.ny * p.nz;
+  if (adjoint) return S >= (1 << 20) && p.R * p.nx >= 400;
+  return p.R * p.nx == kTileNodes && ((p.nx == 128 && S >= (7 << 18)) || (p.nx == 256 && S >= (1 << 20)));
+}
+
 cudaError_t prepare_dev3_tma(const DevTmaPlan &p) {
   const int bytes = p.NS * (int)p.stage_bytes;
   cudaError_t e;
