@@ -247,6 +247,11 @@ LHE_API lhe_status lhe_lbm_set_boundary_jet(lhe_lbm *lbm, const double *jet_dev)
  * with boundary jets when n > 1 or no jets were set since the last step. */
 LHE_API lhe_status lhe_lbm_step(lhe_lbm *lbm, int64_t n);
 
+/* n steps of a Dirichlet box, each with its own jets: lhe_lbm_set_boundary_jet(jets_dev + i * P * LHE_JET_LEN(d))
+ * and lhe_lbm_step(1) for i = 0..n-1 in one call (jets_dev: device, n blocks of P * LHE_JET_LEN(d) doubles).
+ * Errors: those of the two calls. */
+LHE_API lhe_status lhe_lbm_step_jets(lhe_lbm *lbm, const double *jets_dev, int64_t n);
+
 /* Macroscopic variable phi(x, t_step) = sum_k f_k (Eq. (0-1-meq)) into phi_dev (S doubles). */
 LHE_API lhe_status lhe_lbm_macro(lhe_lbm *lbm, double *phi_dev);
 
@@ -337,6 +342,10 @@ LHE_API lhe_status lhe_lbm_set_boundary_sine_product(lhe_lbm *lbm, const lhe_sin
  * unchanged. Errors: LHE_ERR_STATE on a periodic box or before lhe_lbm_adjoint_seed, LHE_ERR_ARG for
  * NULL, LHE_ERR_CUDA. */
 LHE_API lhe_status lhe_lbm_adjoint_jet_grad(lhe_lbm *lbm, double *dL_djet_dev);
+
+/* The reverse of lhe_lbm_step_jets: lhe_lbm_adjoint_jet_grad(dL_djets_dev + i * P * LHE_JET_LEN(d)) and
+ * lhe_lbm_adjoint_step(1) for i = n-1..0 in one call. Errors: those of the two calls. */
+LHE_API lhe_status lhe_lbm_adjoint_step_jets(lhe_lbm *lbm, double *dL_djets_dev, int64_t n);
 
 /* ---------------- stability maps (Sec. 4) ----------------
  * For npoints velocities sigma = u/c (sigma_host: npoints*d doubles, point-major, host memory):

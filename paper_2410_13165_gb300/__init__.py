@@ -182,6 +182,13 @@ class LBM:
         self._stream()
         _abi.lhe_lbm_set_boundary_jet(self.h, self._ptr(jet, P * jet_len(self.d), "jet"))
 
+    def step_jets(self, jets):
+        """One step per block of jets (jets: (T, P, jet_len(d)), contiguous): set_boundary_jet(jets[i]) and step(1) for
+        every i in one call."""
+        T, P = int(jets.shape[0]), _abi.lhe_lbm_boundary_count(self.h)
+        self._stream()
+        _abi.lhe_lbm_step_jets(self.h, self._ptr(jets, T * P * jet_len(self.d), "jets"), T)
+
     def step(self, n: int = 1):
         self._stream()
         _abi.lhe_lbm_step(self.h, n)
@@ -237,6 +244,14 @@ class LBM:
             out = self._torch.empty((P, JL), dtype=self._torch.float64, device=self.device)
         self._stream()
         _abi.lhe_lbm_adjoint_jet_grad(self.h, self._ptr(out, P * JL, "out"))
+        return out
+
+    def adjoint_step_jets(self, out):
+        """The reverse of step_jets: adjoint_jet_grad(out[i]) and adjoint_step(1) for i = T - 1 .. 0 in one call (out:
+        (T, P, jet_len(d)), contiguous)."""
+        T, P = int(out.shape[0]), _abi.lhe_lbm_boundary_count(self.h)
+        self._stream()
+        _abi.lhe_lbm_adjoint_step_jets(self.h, self._ptr(out, T * P * jet_len(self.d), "out"), T)
         return out
 
     def close(self):

@@ -33,7 +33,8 @@ EXPORTS = [
     "lhe_lbm_set_boundary_wave", "lhe_lbm_step", "lhe_lbm_macro", "lhe_lbm_diagnostics", "lhe_lbm_get_state",
     "lhe_lbm_set_state", "lhe_lbm_adjoint_seed", "lhe_lbm_adjoint_step", "lhe_lbm_adjoint_grads",
     "lhe_lbm_diagnostics_noalloc", "lhe_lbm_stability_map", "lhe_lbm_boundary_points", "lhe_lbm_set_boundary_jet",
-    "lhe_lbm_adjoint_jet_grad", "lhe_lbm_set_source", "lhe_lbm_set_boundary_sine_product",
+    "lhe_lbm_adjoint_jet_grad", "lhe_lbm_set_source", "lhe_lbm_set_boundary_sine_product", "lhe_lbm_step_jets",
+    "lhe_lbm_adjoint_step_jets",
 ]
 
 
@@ -113,6 +114,8 @@ def load(path: str | None = None):
         "lhe_lbm_boundary_points": (st, [_H, _D, ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_double)]),
         "lhe_lbm_set_boundary_jet": (st, [_H, _D]),
         "lhe_lbm_step": (st, [_H, ctypes.c_int64]),
+        "lhe_lbm_step_jets": (st, [_H, _D, ctypes.c_int64]),
+        "lhe_lbm_adjoint_step_jets": (st, [_H, _D, ctypes.c_int64]),
         "lhe_lbm_macro": (st, [_H, _D]),
         "lhe_lbm_diagnostics": (st, [_H, ctypes.POINTER(ctypes.c_double)]),
         "lhe_lbm_get_state": (st, [_H, _D]),
@@ -221,6 +224,14 @@ def lhe_lbm_boundary_points(h, d: int):
 
 def lhe_lbm_set_boundary_jet(h, jet_ptr: int) -> None:
     check(load().lhe_lbm_set_boundary_jet(h, jet_ptr), h)
+
+
+def lhe_lbm_step_jets(h, jets_ptr: int, n: int) -> None:
+    check(load().lhe_lbm_step_jets(h, jets_ptr, n), h)
+
+
+def lhe_lbm_adjoint_step_jets(h, out_ptr: int, n: int) -> None:
+    check(load().lhe_lbm_adjoint_step_jets(h, out_ptr, n), h)
 
 
 def lhe_lbm_set_source(h, R_ptr) -> None:

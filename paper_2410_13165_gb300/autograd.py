@@ -46,9 +46,7 @@ class LBMBoxFunction(torch.autograd.Function):
     def forward(ctx, phi0: torch.Tensor, grad: torch.Tensor, jets: torch.Tensor, sim: LBM):
         jets = jets.detach().contiguous()
         sim.init(phi0.detach().contiguous(), grad.detach().contiguous())
-        for n in range(jets.shape[0]):
-            sim.set_boundary_jet(jets[n])
-            sim.step(1)
+        sim.step_jets(jets)
         ctx.sim, ctx.shape = sim, tuple(jets.shape)
         ctx.shapes = (phi0.shape, grad.shape)
         return sim.macro()
@@ -58,9 +56,7 @@ class LBMBoxFunction(torch.autograd.Function):
         sim = ctx.sim
         sim.adjoint_seed(g.contiguous())
         gjets = torch.empty(ctx.shape, dtype=torch.float64, device=g.device)
-        for n in range(ctx.shape[0] - 1, -1, -1):
-            sim.adjoint_jet_grad(out=gjets[n])
-            sim.adjoint_step(1)
+        sim.adjoint_step_jets(gjets)
         gphi0, ggrad, _ = sim.adjoint_grads(want_grad=True, want_R=False)
         return gphi0.view(ctx.shapes[0]), ggrad.view(ctx.shapes[1]), gjets, None
 

@@ -1253,6 +1253,32 @@ lhe_status lhe_lbm_step(lhe_lbm *l, int64_t n) {
   return LHE_OK;
 }
 
+lhe_status lhe_lbm_step_jets(lhe_lbm *l, const double *jets, int64_t n) {
+  if (lhe_status s = check_handle(l)) return s;
+  if (n < 0) return fail(l, LHE_ERR_ARG, "n must be >= 0");
+  int64_t P = 0;
+  if (lhe_status s = lhe_lbm_boundary_points(l, nullptr, &P, nullptr)) return s;
+  if (n > 0 && !jets) return fail(l, LHE_ERR_ARG, "jets is NULL");
+  for (int64_t it = 0; it < n; ++it) {
+    if (lhe_status s = lhe_lbm_set_boundary_jet(l, jets + it * P * LHE_JET_LEN(l->p.d))) return s;
+    if (lhe_status s = lhe_lbm_step(l, 1)) return s;
+  }
+  return LHE_OK;
+}
+
+lhe_status lhe_lbm_adjoint_step_jets(lhe_lbm *l, double *dL_djets, int64_t n) {
+  if (lhe_status s = check_handle(l)) return s;
+  if (n < 0) return fail(l, LHE_ERR_ARG, "n must be >= 0");
+  int64_t P = 0;
+  if (lhe_status s = lhe_lbm_boundary_points(l, nullptr, &P, nullptr)) return s;
+  if (n > 0 && !dL_djets) return fail(l, LHE_ERR_ARG, "dL/djets is NULL");
+  for (int64_t it = n - 1; it >= 0; --it) {
+    if (lhe_status s = lhe_lbm_adjoint_jet_grad(l, dL_djets + it * P * LHE_JET_LEN(l->p.d))) return s;
+    if (lhe_status s = lhe_lbm_adjoint_step(l, 1)) return s;
+  }
+  return LHE_OK;
+}
+
 lhe_status lhe_lbm_macro(lhe_lbm *l, double *phi_out) {
   if (lhe_status s = check_handle(l)) return s;
   if (!phi_out) return fail(l, LHE_ERR_ARG, "phi_out is NULL");
