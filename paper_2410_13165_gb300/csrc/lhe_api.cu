@@ -197,6 +197,7 @@ StepArgs step_args(const lhe_lbm *l) {
   a.rho_dtR = a.dtR;
   a.gsc = a.dt;
   a.pscale = 1.0;
+  a.Rscale = 1.0;
   a.pdl = 0;
   a.sms = l->sms;
   return a;
@@ -1035,6 +1036,7 @@ lhe_status lhe_lbm_set_boundary_jet(lhe_lbm *l, const double *jet_dev) {
   BoundaryArgs b = boundary_args(l);
   b.roff = l->broff;  // the kernel writes l->brec; b.rec stays null (the data are being formed)
   b.rmap = l->bmap;   // in the order of the dense entries when the handle has them
+  b.pdl = pdl_ok(l) && continues_own_steps(l);
   // the schemes' R terms (a source varying in time): full-way at the new time t_{n+1} (the source of
   // this step's collision), half-way at t_n (the source of the collision of f*_kbar)
   b.Rfield = l->p.bc == LHE_BC_FULLWAY ? next_source(l) : l->Rfield;
@@ -1134,6 +1136,7 @@ lhe_status lhe_lbm_adjoint_jet_grad(lhe_lbm *l, double *out) {
   b.roff = l->broff;
   b.src = l->adj[l->acur];
   b.phi_src = l->adjW[l->acur];
+  b.pdl = pdl_ok(l) && continues_own_steps(l);
   LHE_CK(l, launch_jet_grad(l->p.d, l->p.bc, l->p.precision == LHE_FP32_DEV, b, l->blinks, l->nrec, l->bjetw, out,
                             l->stream));
   return LHE_OK;
@@ -1163,6 +1166,9 @@ lhe_status lhe_lbm_step(lhe_lbm *l, int64_t n) {
   const bool scaled = scaled_eligible(l);
   const bool chained = n > 0 && pdl_ok(l) && continues_own_steps(l);
   if (n > 0) note_own_steps(l);
+  // FP64 Dirichlet boxes: the whole box as rows with dense boundary data (default), or the interior
+  // rows with their x_1-face nodes and then the other boundary nodes one by one (LHE_FLAG_NODE_BOUNDARY)
+  const bool dense = !periodic && !dev && l->bdata;
   for (int64_t it = 0; it < n; ++it) {
     if (scaled) plan_scaled_step(l, 0, a);
     a.src = l->pop[l->cur];
@@ -1172,6 +1178,7 @@ lhe_status lhe_lbm_step(lhe_lbm *l, int64_t n) {
     a.nwork = periodic ? l->g.S : l->g.S_rows;
     a.pdl = (it > 0 || chained) && pdl_ok(l);
     if (!periodic) {
+      b.pdl = a.pdl;
       b.src = a.src;
       b.dst = a.dst;
       b.phi_src = a.phi_src;
@@ -1187,14 +1194,20 @@ lhe_status lhe_lbm_step(lhe_lbm *l, int64_t n) {
     double rec_scale = 1.0;
     if (l->sp_mode) {
       // the manufactured solution: its source at t_{n+1} (this step's collision) and its records at the
-      // time of the step's data, both the unit-factor fields times exp(-lambda t)
-      if (!l->Rnext) LHE_CK(l, cudaMalloc(&l->Rnext, sizeof(double) * (size_t)l->g.S));
-      cudaError_t e0 = launch_scale_field(l->sp_R0, std::exp(-l->sp_lambda * (double)(l->step + 1) * l->dt), l->g.S, l->Rnext,
-                              l->sms, l->stream);
-      if (e0 != cudaSuccess) return cuda_fail(l, e0, "source kernel launch");
-      std::swap(l->Rfield, l->Rnext);
-      a.Rfield = l->Rfield;
-      b.Rfield = l->Rfield;
+      // time of the step's data, both the unit-factor fields times exp(-lambda t). The dense rows scale
+      // the unit-factor source as they read it, so that the field itself (for macro, diagnostics and the other
+      // kernels) is formed once per call, at its last step
+      const double at = std::exp(-l->sp_lambda * (double)(l->step + 1) * l->dt);
+      a.Rfield = l->sp_R0;
+      a.Rscale = at;
+      if (!dense || it == n - 1) {
+        if (!l->Rnext) LHE_CK(l, cudaMalloc(&l->Rnext, sizeof(double) * (size_t)l->g.S));
+        cudaError_t e0 = launch_scale_field(l->sp_R0, at, l->g.S, l->Rnext, l->sms, l->stream);
+        if (e0 != cudaSuccess) return cuda_fail(l, e0, "source kernel launch");
+        std::swap(l->Rfield, l->Rnext);
+        if (!dense) a.Rfield = l->Rfield;
+        b.Rfield = l->Rfield;
+      }
       rec_scale = std::exp(-l->sp_lambda * (double)(l->p.bc == LHE_BC_FULLWAY ? l->step + 1 : l->step) * l->dt);
     }
     // boundary data of the step: the exact-solution family, or records (jets, the manufactured solution)
@@ -1210,9 +1223,6 @@ lhe_status lhe_lbm_step(lhe_lbm *l, int64_t n) {
         l->jet_ready = false;
       }
     }
-    // FP64 Dirichlet boxes: the whole box as rows with dense boundary data (default), or the interior
-    // rows with their x_1-face nodes and then the other boundary nodes one by one (LHE_FLAG_NODE_BOUNDARY)
-    const bool dense = !periodic && !dev && l->bdata;
     const bool fused = !periodic && !dev && l->xface && !dense;
     cudaError_t e = cudaSuccess;
     if (dense) {
@@ -1229,6 +1239,7 @@ lhe_status lhe_lbm_step(lhe_lbm *l, int64_t n) {
       e = launch_bdata_step(l->p.bc, rest.rec != nullptr, rest, l->bent, l->bdst, l->bopp, l->nrec,
                             rest.rec ? rest.rec : l->fsep, l->bdata, l->stream);
       if (e != cudaSuccess) return cuda_fail(l, e, "boundary data kernel launch");
+      a.pdl = pdl_ok(l);  // behind this step's own kernel
       e = launch_step_box_dense(d, a, l->bdata, l->stream);
       if (e != cudaSuccess) return cuda_fail(l, e, "step kernel launch");
     } else {
@@ -1243,6 +1254,7 @@ lhe_status lhe_lbm_step(lhe_lbm *l, int64_t n) {
           rest.nsites = b.nsites - l->nb_xface;
           if (rest.roff) rest.roff += l->nb_xface;
         }
+        rest.pdl = pdl_ok(l);
         e = launch_boundary(d, l->p.bc, dev, rest, l->stream);
         if (e != cudaSuccess) return cuda_fail(l, e, "boundary kernel launch");
       }
@@ -1410,6 +1422,7 @@ lhe_status lhe_lbm_adjoint_step(lhe_lbm *l, int64_t n) {
                                   : launch_step_fp64(l->p.d, true, !periodic, a, l->stream);
     if (e != cudaSuccess) return cuda_fail(l, e, "adjoint step kernel launch");
     if (!periodic) {
+      b.pdl = pdl_ok(l);
       b.src = a.src;
       b.dst = a.dst;
       b.phi_src = a.phi_src;

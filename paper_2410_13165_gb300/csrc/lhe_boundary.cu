@@ -32,6 +32,7 @@ __global__ void __launch_bounds__(128) k_boundary(const BoundaryArgs a) {
   constexpr Lattice<D> L{};
   constexpr int Q = Lattice<D>::Q;
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  pdl_wait();
   if (t >= a.nsites) return;
   const int32_t site = a.sites[t];
   const int64_t S = a.g.S;
@@ -131,6 +132,7 @@ __global__ void __launch_bounds__(64) k_jet_records(const BoundaryArgs a, const 
   for (int i = threadIdx.x; i < (int)(sizeof(JetTables) / 2); i += blockDim.x)
     reinterpret_cast<int16_t *>(&J)[i] = reinterpret_cast<const int16_t *>(&T)[i];
   __syncthreads();
+  pdl_wait();
   const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (r >= nrec) return;
   const int2 nk = __ldg(links + r);
@@ -212,9 +214,8 @@ static cudaError_t jet_records_d(int kind, const BoundaryArgs &a, const int2 *li
                                  const JetTables &T, double *rec, cudaStream_t st) {
   if (nrec <= 0) return cudaSuccess;
   const unsigned blocks = (unsigned)((nrec + 63) / 64);
-  if (kind == 1) k_jet_records<D, 1><<<blocks, 64, 0, st>>>(a, links, nrec, jet, T, rec);
-  else k_jet_records<D, 2><<<blocks, 64, 0, st>>>(a, links, nrec, jet, T, rec);
-  return cudaGetLastError();
+  return launch_kernel(kind == 1 ? k_jet_records<D, 1> : k_jet_records<D, 2>, blocks, 64, 0, st, a.pdl != 0, a, links, nrec,
+                       jet, T, rec);
 }
 
 cudaError_t launch_jet_records(int d, int kind, const BoundaryArgs &a, const int2 *links, int64_t nrec, const int32_t *e,
@@ -249,6 +250,7 @@ __global__ void __launch_bounds__(128) k_jet_grad(const BoundaryArgs a, const in
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t row = t / JL;
   const int q = (int)(t - row * JL);
+  pdl_wait();
   if (row >= (KIND == 1 ? a.nsites : nrec)) return;
   const int64_t S = a.g.S;
   const int64_t r0 = KIND == 1 ? a.roff[row] : row;
@@ -270,14 +272,9 @@ static cudaError_t jet_grad_d(int kind, bool dev, const BoundaryArgs &a, const i
   if (nrec <= 0) return cudaSuccess;
   constexpr int64_t JL = (D + 4) * (D + 3) * (D + 2) / 6;
   const unsigned blocks = (unsigned)(((kind == 1 ? a.nsites : nrec) * JL + 127) / 128);
-  if (kind == 1) {
-    if (dev) k_jet_grad<D, 1, true><<<blocks, 128, 0, st>>>(a, links, nrec, w, out);
-    else k_jet_grad<D, 1, false><<<blocks, 128, 0, st>>>(a, links, nrec, w, out);
-  } else {
-    if (dev) k_jet_grad<D, 2, true><<<blocks, 128, 0, st>>>(a, links, nrec, w, out);
-    else k_jet_grad<D, 2, false><<<blocks, 128, 0, st>>>(a, links, nrec, w, out);
-  }
-  return cudaGetLastError();
+  auto kernel = kind == 1 ? (dev ? k_jet_grad<D, 1, true> : k_jet_grad<D, 1, false>)
+                          : (dev ? k_jet_grad<D, 2, true> : k_jet_grad<D, 2, false>);
+  return launch_kernel(kernel, blocks, 128, 0, st, a.pdl != 0, a, links, nrec, w, out);
 }
 
 cudaError_t launch_jet_grad(int d, int kind, bool dev, const BoundaryArgs &a, const int2 *links, int64_t nrec,
@@ -307,6 +304,7 @@ __global__ void __launch_bounds__(128) k_adj_boundary(const BoundaryArgs a) {
   constexpr Lattice<D> L{};
   constexpr int Q = Lattice<D>::Q;
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  pdl_wait();
   if (t >= a.nsites) return;
   const int32_t site = a.sites[t];
   const int64_t S = a.g.S;
@@ -374,14 +372,9 @@ template <int D>
 static cudaError_t adj_boundary_d(int kind, bool dev, const BoundaryArgs &a, cudaStream_t st) {
   if (a.nsites <= 0) return cudaSuccess;
   const unsigned blocks = (unsigned)((a.nsites + 127) / 128);
-  if (kind == 1) {
-    if (dev) k_adj_boundary<D, 1, true><<<blocks, 128, 0, st>>>(a);
-    else k_adj_boundary<D, 1, false><<<blocks, 128, 0, st>>>(a);
-  } else {
-    if (dev) k_adj_boundary<D, 2, true><<<blocks, 128, 0, st>>>(a);
-    else k_adj_boundary<D, 2, false><<<blocks, 128, 0, st>>>(a);
-  }
-  return cudaGetLastError();
+  auto kernel = kind == 1 ? (dev ? k_adj_boundary<D, 1, true> : k_adj_boundary<D, 1, false>)
+                          : (dev ? k_adj_boundary<D, 2, true> : k_adj_boundary<D, 2, false>);
+  return launch_kernel(kernel, blocks, 128, 0, st, a.pdl != 0, a);
 }
 
 cudaError_t launch_adjoint_boundary(int d, int kind, bool dev, const BoundaryArgs &a, cudaStream_t st) {
@@ -400,14 +393,9 @@ static cudaError_t boundary_d(int kind, bool dev, const BoundaryArgs &a, cudaStr
   if (a.nsites <= 0) return cudaSuccess;
   const int threads = 128;
   const unsigned blocks = (unsigned)((a.nsites + threads - 1) / threads);
-  if (kind == 1) {
-    if (dev) k_boundary<D, 1, true><<<blocks, threads, 0, st>>>(a);
-    else k_boundary<D, 1, false><<<blocks, threads, 0, st>>>(a);
-  } else {
-    if (dev) k_boundary<D, 2, true><<<blocks, threads, 0, st>>>(a);
-    else k_boundary<D, 2, false><<<blocks, threads, 0, st>>>(a);
-  }
-  return cudaGetLastError();
+  auto kernel = kind == 1 ? (dev ? k_boundary<D, 1, true> : k_boundary<D, 1, false>)
+                          : (dev ? k_boundary<D, 2, true> : k_boundary<D, 2, false>);
+  return launch_kernel(kernel, blocks, threads, 0, st, a.pdl != 0, a);
 }
 
 cudaError_t launch_boundary(int d, int kind, bool dev, const BoundaryArgs &a, cudaStream_t st) {

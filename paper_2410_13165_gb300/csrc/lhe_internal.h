@@ -47,6 +47,7 @@ struct StepArgs {
   double pscale;           // macro: factor from the stored populations to f* (1 unless scaled)
   int32_t collide;         // kCollideGeneral / kCollideScaled (s != 2 only)
   int32_t sms;             // multiprocessors of the device
+  double Rscale;           // dense Dirichlet rows: factor on Rfield (the manufactured solution's time factor)
   int32_t pdl;             // launch with programmatic stream serialization (the kernel calls pdl_wait)
   int64_t nwork;           // number of sites processed (S, or the interior count)
 };
@@ -148,6 +149,7 @@ struct BoundaryArgs {
   // dense array (k S + x) and half-way partners (kbar S + x) follow from the entry's (k, x)
   int64_t nrow_ent;
   int8_t kbar[kMaxQ];      // the link opposite to k
+  int32_t pdl = 0;         // launch with programmatic stream serialization (the kernel calls pdl_wait)
 };
 
 struct InitArgs {

@@ -243,6 +243,7 @@ __global__ void __launch_bounds__(256) k_bdata_step(const BoundaryArgs b, const 
                                                     int64_t nent, const double *__restrict__ data,
                                                     double *__restrict__ bdata) {
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  pdl_wait();
   if (e >= nent) return;
   // (full-way records need no (k, x): their dst[e] costs the same bytes as the entry)
   const bool row = (!REC || KIND == 2) && e < b.nrow_ent;
@@ -275,7 +276,7 @@ __global__ void __launch_bounds__(LHE_STEP_THREADS) k_step_box_dense(const StepA
   const double *__restrict__ src = static_cast<const double *>(a.src);
   double *__restrict__ dst = static_cast<double *>(a.dst);
   const int64_t S = a.g.S;
-  const double Rs = a.Rfield ? __ldg(a.Rfield + site) : 0.0;
+  const double Rs = a.Rfield ? a.Rscale * __ldg(a.Rfield + site) : 0.0;
   double f[Q];
   const uint64_t row_out = row_links_out<D>(a.g, x);
   const uint64_t x_out = side1 > 0 ? face_links<D>(0, 1) : (side1 < 0 ? face_links<D>(0, -1) : 0ull);
@@ -328,14 +329,9 @@ cudaError_t launch_bdata_step(int kind, bool rec, const BoundaryArgs &b, const l
                               const long long *opp, int64_t nent, const double *data, double *bdata, cudaStream_t st) {
   if (nent <= 0) return cudaSuccess;
   const unsigned blocks = (unsigned)((nent + 255) / 256);
-  if (kind == 1) {
-    if (rec) k_bdata_step<1, true><<<blocks, 256, 0, st>>>(b, ent, dst, opp, nent, data, bdata);
-    else k_bdata_step<1, false><<<blocks, 256, 0, st>>>(b, ent, dst, opp, nent, data, bdata);
-  } else {
-    if (rec) k_bdata_step<2, true><<<blocks, 256, 0, st>>>(b, ent, dst, opp, nent, data, bdata);
-    else k_bdata_step<2, false><<<blocks, 256, 0, st>>>(b, ent, dst, opp, nent, data, bdata);
-  }
-  return cudaGetLastError();
+  auto kernel = kind == 1 ? (rec ? k_bdata_step<1, true> : k_bdata_step<1, false>)
+                          : (rec ? k_bdata_step<2, true> : k_bdata_step<2, false>);
+  return launch_kernel(kernel, blocks, 256, 0, st, b.pdl != 0, b, ent, dst, opp, nent, data, bdata);
 }
 
 cudaError_t launch_family_sep(int d, int kind, const BoundaryArgs &b, const long long *ent, int64_t nent, double *sep,
