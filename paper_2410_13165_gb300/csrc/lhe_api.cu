@@ -336,6 +336,24 @@ void forget_steps_of(const lhe_lbm *l) {
   if (g_last_steps_handle == l) g_last_steps_handle = nullptr;
 }
 
+// h steps in one launch (a: buffers and pdl set), each with its own collision constants.
+lhe_status multi_steps(lhe_lbm *l, int which, int h, StepArgs &a, bool scaled) {
+  MultiArgs m{};
+  m.p = shorter_multi(l->g, l->p.precision == LHE_FP32_DEV, l->multi, h);
+  for (int j = 0; j < m.p.H; ++j) {
+    if (scaled) plan_scaled_step(l, which, a);
+    m.mu[j] = a.mu;
+    m.sig[j] = a.sig;
+    m.rho_dt[j] = a.rho_dt;
+    m.rho_dtR[j] = a.rho_dtR;
+    m.gsc[j] = a.gsc;
+    m.collide[j] = a.collide;
+  }
+  m.a = a;
+  const cudaError_t e = launch_multi(l->p.d, l->p.precision == LHE_FP32_DEV, which == 1, m, l->stream);
+  return e == cudaSuccess ? LHE_OK : cuda_fail(l, e, "step kernel launch");
+}
+
 lhe_status check_handle(lhe_lbm *l) {
   if (!l) return fail(nullptr, LHE_ERR_ARG, "handle is NULL");
   return LHE_OK;
@@ -572,6 +590,10 @@ lhe_status lhe_lbm_create(const lhe_lbm_params *p, lhe_lbm **out) {
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&l->sms, cudaDevAttrMultiProcessorCount, dev);
+  }
+  if (p->bc == LHE_BC_PERIODIC && plan_multi(l->g, p->precision == LHE_FP32_DEV, l->sms, l->multi)) {
+    e = prepare_multi(p->d, p->precision == LHE_FP32_DEV, l->multi);
+    if (e != cudaSuccess) return bail(cuda_fail(l, e, "shared-memory size of the multi-step kernel"));
   }
   if (p->d == 3 && p->bc == LHE_BC_PERIODIC && p->precision == LHE_FP32_DEV && !(p->flags & LHE_FLAG_NO_STAGING)) {
     const int sms = l->sms;
@@ -1170,6 +1192,18 @@ lhe_status lhe_lbm_step(lhe_lbm *l, int64_t n) {
   // rows with their x_1-face nodes and then the other boundary nodes one by one (LHE_FLAG_NODE_BOUNDARY)
   const bool dense = !periodic && !dev && l->bdata;
   for (int64_t it = 0; it < n; ++it) {
+    if (const int h = (int)std::min<int64_t>(l->multi.H, n - it); h > 1) {
+      a.src = l->pop[l->cur];
+      a.dst = l->pop[1 - l->cur];
+      a.phi_src = l->phi[l->cur];
+      a.phi_dst = l->phi[1 - l->cur];
+      a.pdl = (it > 0 || chained) && pdl_ok(l);
+      if (lhe_status st = multi_steps(l, 0, h, a, scaled)) return st;
+      l->cur ^= 1;
+      l->step += h;
+      it += h - 1;
+      continue;
+    }
     if (scaled) plan_scaled_step(l, 0, a);
     a.src = l->pop[l->cur];
     a.dst = l->pop[1 - l->cur];
@@ -1411,6 +1445,17 @@ lhe_status lhe_lbm_adjoint_step(lhe_lbm *l, int64_t n) {
   const bool chained = n > 0 && pdl_ok(l) && continues_own_steps(l);
   if (n > 0) note_own_steps(l);
   for (int64_t it = 0; it < n; ++it) {
+    if (const int h = (int)std::min<int64_t>(l->multi.H, n - it); h > 1) {
+      a.src = l->adj[l->acur];
+      a.dst = l->adj[1 - l->acur];
+      a.phi_src = l->adjW[l->acur];
+      a.phi_dst = l->adjW[1 - l->acur];
+      a.pdl = (it > 0 || chained) && pdl_ok(l);
+      if (lhe_status st = multi_steps(l, 1, h, a, scaled)) return st;
+      l->acur ^= 1;
+      it += h - 1;
+      continue;
+    }
     if (scaled) plan_scaled_step(l, 1, a);
     a.src = l->adj[l->acur];
     a.dst = l->adj[1 - l->acur];

@@ -96,6 +96,26 @@ struct DevTmaPlan {
 constexpr int kCollideGeneral = 0;  // two FP64 operations per population
 constexpr int kCollideScaled = 1;   // scaled representation, one FMA per population
 
+// Several steps of a periodic 1D / 2D box in one launch (lhe_step_multi.cu).
+constexpr int kMultiMaxSteps = 8;
+constexpr int kMultiThreads = 1024;            // at most
+constexpr int kMultiMaxSmem = 227 * 1024;
+struct MultiPlan {
+  int32_t H = 0;                  // steps per launch (0: not used)
+  int32_t tx = 0, ty = 1;         // nodes of a tile
+  int32_t w = 0, h = 1;           // extents of the first step's region: the tile and H - 1 rings
+  int32_t tiles_x = 0, grid = 0, threads = 0;
+  size_t smem = 0;
+};
+
+struct MultiArgs {
+  StepArgs a;
+  MultiPlan p;
+  // the collision constants of each step (StepArgs)
+  double mu[kMultiMaxSteps], sig[kMultiMaxSteps], rho_dt[kMultiMaxSteps], rho_dtR[kMultiMaxSteps], gsc[kMultiMaxSteps];
+  int32_t collide[kMultiMaxSteps];
+};
+
 // The manufactured solution A exp(-lambda t) prod_i sin(kappa_i x_i + theta_i) and the node grid
 // x_i = x0_i + j_i dx (lhe_provider.cu).
 struct SineProductArgs {
@@ -246,6 +266,10 @@ bool plan_dev3_tma(const Geom &g, int sms, DevTmaPlan &p);
 bool staged_pays(const DevTmaPlan &p, bool adjoint);
 cudaError_t prepare_dev3_tma(const DevTmaPlan &p);
 cudaError_t launch_step_dev3_tma(bool adjoint, const StepArgs &a, const DevTmaPlan &p, cudaStream_t st);
+bool plan_multi(const Geom &g, bool dev, int sms, MultiPlan &p);
+MultiPlan shorter_multi(const Geom &g, bool dev, const MultiPlan &p, int H);  // the same tiles, 2 <= H <= p.H
+cudaError_t prepare_multi(int d, bool dev, const MultiPlan &p);
+cudaError_t launch_multi(int d, bool dev, bool adjoint, const MultiArgs &m, cudaStream_t st);
 cudaError_t launch_adjoint_grads(int d, bool dev, const AdjGradArgs &a, cudaStream_t st);
 
 // Record the message lhe_lbm_last_error(NULL) returns on this thread; returns `status`.
@@ -326,6 +350,7 @@ struct lhe_lbm {
   // Scaled representation of the FP64 state when s != 2 on periodic boxes: the stored populations
   // are K f* with K = (1 - s)^-j; j = 0 means the state is stored as f* itself. [0] forward, [1]
   // adjoint. acc accumulates the relative error of the rounded s/(1 - s) factors.
+  lhe::MultiPlan multi;  // periodic 1D / 2D boxes: several steps per launch (H = 0: one)
   // staged FP32-deviation step (periodic D3Q19)
   bool staged[2] = {false, false};  // forward, adjoint
   lhe::DevTmaPlan tma{};
