@@ -96,15 +96,19 @@ struct DevTmaPlan {
 constexpr int kCollideGeneral = 0;  // two FP64 operations per population
 constexpr int kCollideScaled = 1;   // scaled representation, one FMA per population
 
-// Several steps of a periodic 1D / 2D box in one launch (lhe_step_multi.cu).
+// Several steps of a periodic 1D, 2D or 3D box in one launch (lhe_step_multi.cu).
 constexpr int kMultiMaxSteps = 8;
-constexpr int kMultiThreads = 1024;            // at most
+constexpr int kMultiThreads = 1024;            // at most (64 registers)
+__host__ __device__ constexpr int multi_threads(int d) { return d == 3 ? 512 : kMultiThreads; }
 constexpr int kMultiMaxSmem = 227 * 1024;
 struct MultiPlan {
   int32_t H = 0;                  // steps per launch (0: not used)
-  int32_t tx = 0, ty = 1;         // nodes of a tile
-  int32_t w = 0, h = 1;           // extents of the first step's region: the tile and H - 1 rings
-  int32_t tiles_x = 0, grid = 0, threads = 0;
+  int32_t t[3] = {0, 1, 1};       // extents of a tile
+  int32_t w[3] = {0, 1, 1};       // extents of the first step's region: the tile and H - 1 rings
+  int32_t tiles[3] = {0, 1, 1};   // tiles along each axis
+  int32_t own = 0, nodes = 0;     // nodes of a tile, of the first region
+  int32_t copies = 0;             // of the region in shared memory
+  int32_t grid = 0, threads = 0;
   size_t smem = 0;
 };
 
@@ -350,7 +354,7 @@ struct lhe_lbm {
   // Scaled representation of the FP64 state when s != 2 on periodic boxes: the stored populations
   // are K f* with K = (1 - s)^-j; j = 0 means the state is stored as f* itself. [0] forward, [1]
   // adjoint. acc accumulates the relative error of the rounded s/(1 - s) factors.
-  lhe::MultiPlan multi;  // periodic 1D / 2D boxes: several steps per launch (H = 0: one)
+  lhe::MultiPlan multi;  // small periodic boxes: several steps per launch (H = 0: one)
   // staged FP32-deviation step (periodic D3Q19)
   bool staged[2] = {false, false};  // forward, adjoint
   lhe::DevTmaPlan tma{};

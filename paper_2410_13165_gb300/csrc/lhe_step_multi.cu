@@ -1,4 +1,4 @@
-// lhe_step_multi.cu -- several steps of a small or 32-bit periodic 1D / 2D box in one launch.
+// lhe_step_multi.cu -- several steps of a small or 32-bit periodic box (1D to 3D) in one launch.
 //
 // A step of such a grid is bound by its launch (~1.8 us from one step kernel to the next) and, in 32 bits, by L2,
 // not by arithmetic. A CTA owns a tile of nodes and takes it through H steps in shared memory: the first
@@ -25,23 +25,53 @@ __device__ __forceinline__ int wrap_once(int v, int n) { return v < 0 ? v + n : 
 // Where a CTA's tile lies and how the nodes of a step are numbered.
 template <int D>
 struct MultiTile {
-  int W, x0, y0, nx, ny, own_x, own_y;
+  int x0[D], n[D], own[D], stride[D];  // origin of the first region, box, the tile's own nodes, strides within a copy
   __device__ __forceinline__ explicit MultiTile(const StepArgs &a, const MultiPlan &p) {
-    const int ty = D == 2 ? blockIdx.x / p.tiles_x : 0, tx = blockIdx.x - ty * p.tiles_x;
-    W = p.w;
-    nx = a.g.n[0];
-    ny = D == 2 ? a.g.n[1] : 1;
-    x0 = tx * p.tx - (p.H - 1);
-    y0 = D == 2 ? ty * p.ty - (p.H - 1) : 0;
-    // the tile's own nodes (a last tile may stick out of the box: the nodes beyond are another tile's)
-    own_x = min(p.tx, nx - tx * p.tx);
-    own_y = D == 2 ? min(p.ty, ny - ty * p.ty) : 1;
+    int b = blockIdx.x, st = 1;
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      const int q = i == D - 1 ? 0 : b / p.tiles[i];
+      const int first = (i == D - 1 ? b : b - q * p.tiles[i]) * p.t[i];
+      b = q;
+      n[i] = a.g.n[i];
+      x0[i] = first - (p.H - 1);
+      own[i] = min(p.t[i], n[i] - first);  // (a last tile may stick out of the box: the nodes beyond are another tile's)
+      stride[i] = st;
+      st *= p.w[i];
+    }
   }
-  // node of the box at (ix, iy) of the first step's region
-  __device__ __forceinline__ int32_t site(int ix, int iy, int &gx, int &gy) const {
-    gx = wrap_once(x0 + ix, nx);
-    gy = D == 2 ? wrap_once(y0 + iy, ny) : 0;
-    return gx + nx * gy;
+  // place of a node of the region in a copy, and in the box
+  __device__ __forceinline__ int at(const int (&i)[D]) const {
+    int c = 0;
+#pragma unroll
+    for (int q = 0; q < D; ++q) c += i[q] * stride[q];
+    return c;
+  }
+  __device__ __forceinline__ int32_t site(const Geom &g, const int (&i)[D], int (&x)[D]) const {
+    int32_t s = 0;
+#pragma unroll
+    for (int q = 0; q < D; ++q) {
+      x[q] = wrap_once(x0[q] + i[q], n[q]);
+      s += x[q] * g.stride[q];
+    }
+    return s;
+  }
+  __device__ __forceinline__ int32_t site(const Geom &g, const int (&i)[D]) const {
+    int x[D];
+    return site(g, i, x);
+  }
+  // place among the tile's own nodes, or -1
+  __device__ __forceinline__ int mine(const MultiPlan &p, const int (&i)[D]) const {
+    int c = 0, st = 1;
+    bool in = true;
+#pragma unroll
+    for (int q = 0; q < D; ++q) {
+      const int l = i[q] - (p.H - 1);
+      in = in && l >= 0 && l < own[q];
+      c += l * st;
+      st *= p.t[q];
+    }
+    return in ? c : -1;
   }
 };
 
@@ -49,66 +79,84 @@ struct MultiTile {
 // least 1 / (2 w) from an integer.
 __device__ __forceinline__ int row_of(int t, float inv) { return (int)(((float)t + 0.5f) * inv); }
 
-// Calls node(ix, iy, t) for the nodes of step j (1 .. H) of the region, one after another per thread.
+// Calls node(i) for the nodes i of step j (1 .. H) of the region, one after another per thread.
 template <int D, class F>
 __device__ __forceinline__ void multi_nodes(const MultiPlan &p, int j, F node) {
-  const int o = j - 1, w = p.w - 2 * o, nodes = w * (D == 2 ? p.h - 2 * o : 1);
-  const float inv = __fdividef(1.0f, (float)w);
+  const int o = j - 1;
+  int w[D], nodes = 1;
+#pragma unroll
+  for (int q = 0; q < D; ++q) {
+    w[q] = p.w[q] - 2 * o;
+    nodes *= w[q];
+  }
+  const float inv0 = __fdividef(1.0f, (float)w[0]), inv1 = __fdividef(1.0f, (float)w[D > 1 ? 1 : 0]);
   for (int t = threadIdx.x; t < nodes; t += blockDim.x) {
-    const int r = D == 2 ? row_of(t, inv) : 0;
-    node(t - r * w + o, D == 2 ? r + o : 0);
+    int i[D];
+    if constexpr (D == 1) {
+      i[0] = t + o;
+    } else {
+      const int r = row_of(t, inv0);
+      i[0] = t - r * w[0] + o;
+      if constexpr (D == 2) {
+        i[1] = r + o;
+      } else {
+        const int z = row_of(r, inv1);
+        i[1] = r - z * w[1] + o;
+        i[2] = z + o;
+      }
+    }
+    node(i);
   }
 }
 
-// The two copies hold the nodes' populations together (Q consecutive values a node): a neighbour's address is one
-// of three row addresses plus a constant, and Q is odd, so that the lanes of a warp fall on different banks.
-// (With population-major copies each access took its own address arithmetic: 329 instructions a node and
+// The copies hold the nodes' populations together (Q consecutive values a node): a neighbour's address is one
+// of 3^(D-1) row addresses plus a constant, and Q is odd, so that the lanes of a warp fall on different banks.
+// (With population-major copies each access took its own address arithmetic: 329 instructions a D2Q9 node and
 // step in 32 bits, twice the arithmetic's.)
+template <int D, bool ADJ>
+__device__ __forceinline__ int pull_row(const MultiTile<D> &tile, int k) {
+  constexpr Lattice<D> L{};
+  int r = 0;
+#pragma unroll
+  for (int q = 1; q < D; ++q) r += (ADJ ? L.e[k][q] : -L.e[k][q]) * tile.stride[q];
+  return r;
+}
+
 template <int D, bool ADJ, class T>
-__device__ __forceinline__ void pull_shared(const T *__restrict__ from, int c, int W, T (&f)[Lattice<D>::Q]) {
+__device__ __forceinline__ void pull_shared(const T *__restrict__ from, int c, const MultiTile<D> &tile, T (&f)[Lattice<D>::Q]) {
   constexpr Lattice<D> L{};
   constexpr int Q = Lattice<D>::Q;
-  const T *row[3];
-  row[1] = from + c * Q;
-  row[0] = D == 2 ? row[1] - W * Q : row[1];
-  row[2] = D == 2 ? row[1] + W * Q : row[1];
 #pragma unroll
-  for (int k = 0; k < Q; ++k) {
-    const int ex = ADJ ? L.e[k][0] : -L.e[k][0], ey = D == 2 ? (ADJ ? L.e[k][D - 1] : -L.e[k][D - 1]) : 0;
-    f[k] = row[1 + ey][ex * Q + k];
-  }
+  for (int k = 0; k < Q; ++k) f[k] = from[(c + pull_row<D, ADJ>(tile, k)) * Q + (ADJ ? L.e[k][0] : -L.e[k][0]) * Q + k];
 }
 
 template <int D, bool ADJ, int MODE>
-__global__ void __launch_bounds__(kMultiThreads) k_multi_fp64(const __grid_constant__ MultiArgs m) {
+__global__ void __launch_bounds__(multi_threads(D)) k_multi_fp64(const __grid_constant__ MultiArgs m) {
   constexpr Lattice<D> L{};
   constexpr int Q = Lattice<D>::Q;
   extern __shared__ __align__(16) unsigned char smem[];
   const StepArgs &a = m.a;
   const MultiPlan &p = m.p;
-  const int H = p.H, N = p.w * p.h;
-  double *buf = reinterpret_cast<double *>(smem);  // two copies of N x Q
-  double *acc = buf + 2 * N * Q;                   // adjoint: dL/dR of the tile
+  const int H = p.H, N = p.nodes;
+  double *buf = reinterpret_cast<double *>(smem);  // p.copies of N x Q
+  double *acc = buf + p.copies * N * Q;            // adjoint: dL/dR of the tile
   const MultiTile<D> tile(a, p);
   const int64_t S = a.g.S;
-  // the collision of step o + 1 at (ix, iy): psi from the pulled populations, dL/dR on the way
-  auto collide = [&](const double (&f)[Q], int o, int ix, int iy) {
+  // the collision of step o + 1 at node i: psi from the pulled populations, dL/dR on the way
+  auto collide = [&](const double (&f)[Q], int o, const int (&i)[D]) {
     double psi;
     if (ADJ) {
       const double w2 = MODE == kModeS2 ? fixed_moment_sum<Q, 1>(f) : fixed_moment_sum<Q, 0>(f);
       psi = MODE == kModeS2 ? w2 : m.sig[o] * w2;
-      const int lx = ix - (H - 1), ly = D == 2 ? iy - (H - 1) : 0;
-      if (a.gR && lx >= 0 && lx < tile.own_x && ly >= 0 && ly < tile.own_y) {
-        int gx, gy;
-        const int32_t site = tile.site(ix, iy, gx, gy);
-        const int c = lx + p.tx * ly;
+      const int c = a.gR ? tile.mine(p, i) : -1;
+      if (c >= 0) {
+        const int32_t site = tile.site(a.g, i);
         const double g = fma(MODE == kModeS2 ? a.half_dt : m.gsc[o], w2, o == 0 ? a.gR[site] : acc[c]);
         if (o == H - 1) a.gR[site] = g;
         else acc[c] = g;
       }
     } else {
-      int gx, gy;
-      const double R = a.Rfield ? __ldg(a.Rfield + tile.site(ix, iy, gx, gy)) : 0.0;
+      const double R = a.Rfield ? __ldg(a.Rfield + tile.site(a.g, i)) : 0.0;
       if (MODE == kModeS2) psi = fixed_moment_sum<Q, 1>(f) + (a.Rfield ? a.dt * R : a.dtR);
       else psi = fma(m.sig[o], fixed_moment_sum<Q, 0>(f), a.Rfield ? m.rho_dt[o] * R : m.rho_dtR[o]);
     }
@@ -120,18 +168,16 @@ __global__ void __launch_bounds__(kMultiThreads) k_multi_fp64(const __grid_const
   };
   pdl_wait();
   const double *__restrict__ src = static_cast<const double *>(a.src);
-  multi_nodes<D>(p, 1, [&](int ix, int iy) {
-    int x[D], gx, gy;
-    const int32_t site = tile.site(ix, iy, gx, gy);
-    x[0] = gx;
-    if (D == 2) x[D - 1] = gy;
+  multi_nodes<D>(p, 1, [&](const int (&i)[D]) {
+    int x[D];
+    const int32_t site = tile.site(a.g, i, x);
     int32_t om[D], op[D];
     axis_offsets<D, false>(a.g, x, om, op);
     double f[Q];
 #pragma unroll
     for (int k = 0; k < Q; ++k) f[k] = __ldg(src + k * S + source_site<D, ADJ>(L, k, site, om, op));
-    const double psi = collide(f, 0, ix, iy);
-    double *to = buf + (ix + tile.W * iy) * Q;
+    const double psi = collide(f, 0, i);
+    double *to = buf + tile.at(i) * Q;
 #pragma unroll
     for (int k = 0; k < Q; ++k) to[k] = out(f[k], psi, 0, k);
   });
@@ -140,11 +186,11 @@ __global__ void __launch_bounds__(kMultiThreads) k_multi_fp64(const __grid_const
   for (int j = 2; j < H; ++j) {
     const double *from = buf + cur * N * Q;
     double *dst = buf + (cur ^ 1) * N * Q;
-    multi_nodes<D>(p, j, [&](int ix, int iy) {
-      const int c = ix + tile.W * iy;
+    multi_nodes<D>(p, j, [&](const int (&i)[D]) {
+      const int c = tile.at(i);
       double f[Q];
-      pull_shared<D, ADJ>(from, c, tile.W, f);
-      const double psi = collide(f, j - 1, ix, iy);
+      pull_shared<D, ADJ>(from, c, tile, f);
+      const double psi = collide(f, j - 1, i);
       double *to = dst + c * Q;
 #pragma unroll
       for (int k = 0; k < Q; ++k) to[k] = out(f[k], psi, j - 1, k);
@@ -154,35 +200,34 @@ __global__ void __launch_bounds__(kMultiThreads) k_multi_fp64(const __grid_const
   }
   const double *from = buf + cur * N * Q;
   double *__restrict__ dst = static_cast<double *>(a.dst);
-  multi_nodes<D>(p, H, [&](int ix, int iy) {
-    if (ix - (H - 1) >= tile.own_x || (D == 2 && iy - (H - 1) >= tile.own_y)) return;
-    int gx, gy;
-    const int32_t site = tile.site(ix, iy, gx, gy);
+  multi_nodes<D>(p, H, [&](const int (&i)[D]) {
+    if (tile.mine(p, i) < 0) return;
+    const int32_t site = tile.site(a.g, i);
     double f[Q];
-    pull_shared<D, ADJ>(from, ix + tile.W * iy, tile.W, f);
-    const double psi = collide(f, H - 1, ix, iy);
+    pull_shared<D, ADJ>(from, tile.at(i), tile, f);
+    const double psi = collide(f, H - 1, i);
 #pragma unroll
     for (int k = 0; k < Q; ++k) dst[k * S + site] = out(f[k], psi, H - 1, k);
   });
 }
 
 template <int D, bool ADJ, bool S2>
-__global__ void __launch_bounds__(kMultiThreads) k_multi_dev(const __grid_constant__ MultiArgs m) {
+__global__ void __launch_bounds__(multi_threads(D)) k_multi_dev(const __grid_constant__ MultiArgs m) {
   constexpr Lattice<D> L{};
   constexpr int Q = Lattice<D>::Q;
   extern __shared__ __align__(16) unsigned char smem[];
   const StepArgs &a = m.a;
   const MultiPlan &p = m.p;
-  const int H = p.H, N = p.w * p.h;
-  double *acc = reinterpret_cast<double *>(smem);                           // adjoint: dL/dR of the tile
-  float2 *bphi = reinterpret_cast<float2 *>(acc + (ADJ ? p.tx * p.ty : 0));  // two copies of N
-  float *buf = reinterpret_cast<float *>(bphi + 2 * N);                     // two copies of N x Q
+  const int H = p.H, N = p.nodes;
+  double *acc = reinterpret_cast<double *>(smem);                         // adjoint: dL/dR of the tile
+  float2 *bphi = reinterpret_cast<float2 *>(acc + (ADJ ? p.own : 0));      // p.copies of N
+  float *buf = reinterpret_cast<float *>(bphi + p.copies * N);            // p.copies of N x Q
   const MultiTile<D> tile(a, p);
   const int64_t S = a.g.S;
   const bool field = !ADJ && a.Rfield != nullptr;
   const float oms = (float)a.oms;
-  // step o + 1 at (ix, iy) from the pulled deviations and the differences of phi: the new pair of phi; gk becomes the new deviations
-  auto collide = [&](float (&gk)[Q], const float (&dl)[Q], float2 p0, int o, int ix, int iy) {
+  // step o + 1 at node i from the pulled deviations and the differences of phi: the new pair of phi; gk becomes the new deviations
+  auto collide = [&](float (&gk)[Q], const float (&dl)[Q], float2 p0, int o, const int (&i)[D]) {
     float accw = 0.0f, accg = 0.0f;
 #pragma unroll
     for (int k = 0; k < Q; ++k) {
@@ -193,18 +238,15 @@ __global__ void __launch_bounds__(kMultiThreads) k_multi_dev(const __grid_consta
     const float2 pn = df_add(p0.x, p0.y + Delta);
     float dtR = 0.0f;
     if (ADJ) {
-      const int lx = ix - (H - 1), ly = D == 2 ? iy - (H - 1) : 0;
-      if (a.gR && lx >= 0 && lx < tile.own_x && ly >= 0 && ly < tile.own_y) {
-        int gx, gy;
-        const int32_t site = tile.site(ix, iy, gx, gy);
-        const int q = lx + p.tx * ly;
+      const int q = a.gR ? tile.mine(p, i) : -1;
+      if (q >= 0) {
+        const int32_t site = tile.site(a.g, i);
         const double g = fma(a.dt, df_value(pn), o == 0 ? a.gR[site] : acc[q]);
         if (o == H - 1) a.gR[site] = g;
         else acc[q] = g;
       }
     } else if (field) {
-      int gx, gy;
-      dtR = (float)(a.dt * __ldg(a.Rfield + tile.site(ix, iy, gx, gy)));
+      dtR = (float)(a.dt * __ldg(a.Rfield + tile.site(a.g, i)));
     }
 #pragma unroll
     for (int k = 0; k < Q; ++k) {
@@ -216,17 +258,12 @@ __global__ void __launch_bounds__(kMultiThreads) k_multi_dev(const __grid_consta
   };
   // pulled values of a node from the shared copies
   auto pull = [&](const float *from, const float2 *pf, int c, float (&gk)[Q], float (&dl)[Q]) {
-    pull_shared<D, ADJ>(from, c, tile.W, gk);
-    const float2 *row[3];
-    row[1] = pf + c;
-    row[0] = D == 2 ? row[1] - tile.W : row[1];
-    row[2] = D == 2 ? row[1] + tile.W : row[1];
-    const float2 p0 = *row[1];
+    pull_shared<D, ADJ>(from, c, tile, gk);
+    const float2 p0 = pf[c];
     dl[0] = 0.0f;
 #pragma unroll
     for (int k = 1; k < Q; ++k) {
-      const int ex = ADJ ? L.e[k][0] : -L.e[k][0], ey = D == 2 ? (ADJ ? L.e[k][D - 1] : -L.e[k][D - 1]) : 0;
-      const float2 pk = row[1 + ey][ex];
+      const float2 pk = pf[(c + pull_row<D, ADJ>(tile, k)) + (ADJ ? L.e[k][0] : -L.e[k][0])];
       dl[k] = (pk.x - p0.x) + (pk.y - p0.y);
     }
     return p0;
@@ -234,11 +271,9 @@ __global__ void __launch_bounds__(kMultiThreads) k_multi_dev(const __grid_consta
   pdl_wait();
   const float *__restrict__ src = static_cast<const float *>(a.src);
   const float2 *__restrict__ phis = a.phi_src;
-  multi_nodes<D>(p, 1, [&](int ix, int iy) {
-    int x[D], gx, gy;
-    const int32_t site = tile.site(ix, iy, gx, gy);
-    x[0] = gx;
-    if (D == 2) x[D - 1] = gy;
+  multi_nodes<D>(p, 1, [&](const int (&i)[D]) {
+    int x[D];
+    const int32_t site = tile.site(a.g, i, x);
     int32_t om[D], op[D];
     axis_offsets<D, false>(a.g, x, om, op);
     const float2 p0 = __ldg(phis + site);
@@ -253,8 +288,8 @@ __global__ void __launch_bounds__(kMultiThreads) k_multi_dev(const __grid_consta
         dl[k] = (pk.x - p0.x) + (pk.y - p0.y);
       }
     }
-    const int c = ix + tile.W * iy;
-    bphi[c] = collide(gk, dl, p0, 0, ix, iy);
+    const int c = tile.at(i);
+    bphi[c] = collide(gk, dl, p0, 0, i);
 #pragma unroll
     for (int k = 0; k < Q; ++k) buf[c * Q + k] = gk[k];
   });
@@ -265,11 +300,11 @@ __global__ void __launch_bounds__(kMultiThreads) k_multi_dev(const __grid_consta
     float *to = buf + (cur ^ 1) * N * Q;
     const float2 *pf = bphi + cur * N;
     float2 *pt = bphi + (cur ^ 1) * N;
-    multi_nodes<D>(p, j, [&](int ix, int iy) {
-      const int c = ix + tile.W * iy;
+    multi_nodes<D>(p, j, [&](const int (&i)[D]) {
+      const int c = tile.at(i);
       float gk[Q], dl[Q];
       const float2 p0 = pull(from, pf, c, gk, dl);
-      pt[c] = collide(gk, dl, p0, j - 1, ix, iy);
+      pt[c] = collide(gk, dl, p0, j - 1, i);
 #pragma unroll
       for (int k = 0; k < Q; ++k) to[c * Q + k] = gk[k];
     });
@@ -279,13 +314,12 @@ __global__ void __launch_bounds__(kMultiThreads) k_multi_dev(const __grid_consta
   const float *from = buf + cur * N * Q;
   const float2 *pf = bphi + cur * N;
   float *__restrict__ dst = static_cast<float *>(a.dst);
-  multi_nodes<D>(p, H, [&](int ix, int iy) {
-    if (ix - (H - 1) >= tile.own_x || (D == 2 && iy - (H - 1) >= tile.own_y)) return;
-    int gx, gy;
-    const int32_t site = tile.site(ix, iy, gx, gy);
+  multi_nodes<D>(p, H, [&](const int (&i)[D]) {
+    if (tile.mine(p, i) < 0) return;
+    const int32_t site = tile.site(a.g, i);
     float gk[Q], dl[Q];
-    const float2 p0 = pull(from, pf, ix + tile.W * iy, gk, dl);
-    a.phi_dst[site] = collide(gk, dl, p0, H - 1, ix, iy);
+    const float2 p0 = pull(from, pf, tile.at(i), gk, dl);
+    a.phi_dst[site] = collide(gk, dl, p0, H - 1, i);
 #pragma unroll
     for (int k = 0; k < Q; ++k) dst[k * S + site] = gk[k];
   });
@@ -293,38 +327,47 @@ __global__ void __launch_bounds__(kMultiThreads) k_multi_dev(const __grid_consta
 
 namespace {
 
-// H steps over tiles of tx x ty nodes, a thread per node of the first region up to `most`.
-MultiPlan make_multi(const Geom &g, bool dev, int tx, int ty, int H, int most) {
+// H steps over tiles of t nodes, a thread per node of the first region up to `most`.
+MultiPlan make_multi(const Geom &g, bool dev, int tx, int ty, int tz, int H, int most) {
   MultiPlan p;
+  const int t[3] = {tx, g.d > 1 ? ty : 1, g.d > 2 ? tz : 1};
   p.H = H;
-  p.tx = tx;
-  p.ty = g.d == 2 ? ty : 1;
-  p.w = tx + 2 * (H - 1);
-  p.h = g.d == 2 ? ty + 2 * (H - 1) : 1;
-  p.tiles_x = (g.n[0] + tx - 1) / tx;
-  p.grid = p.tiles_x * (g.d == 2 ? (g.n[1] + ty - 1) / ty : 1);
-  p.threads = std::min(most, (p.w * p.h + 31) / 32 * 32);
-  const size_t Q = 2 * g.d * g.d + 1, N = (size_t)p.w * p.h;
-  p.smem = 8 * (size_t)p.tx * p.ty + 2 * N * (dev ? 4 * Q + 8 : 8 * Q);
+  p.copies = H > 2 ? 2 : 1;
+  p.nodes = p.own = p.grid = 1;
+  for (int i = 0; i < 3; ++i) {
+    p.t[i] = t[i];
+    p.w[i] = t[i] + (i < g.d ? 2 * (H - 1) : 0);
+    p.tiles[i] = i < g.d ? (g.n[i] + t[i] - 1) / t[i] : 1;
+    p.nodes *= p.w[i];
+    p.own *= t[i];
+    p.grid *= p.tiles[i];
+  }
+  p.threads = std::min(most, (p.nodes + 31) / 32 * 32);
+  const size_t Q = 2 * g.d * g.d + 1;
+  p.smem = 8 * (size_t)p.own + p.copies * (size_t)p.nodes * (dev ? 4 * Q + 8 : 8 * Q);
   return p;
 }
 
 template <int D>
-const void *multi_kernel(bool dev, bool adjoint, bool s2) {
-  if (dev)
-    return adjoint ? (s2 ? (const void *)k_multi_dev<D, true, true> : (const void *)k_multi_dev<D, true, false>)
-                   : (s2 ? (const void *)k_multi_dev<D, false, true> : (const void *)k_multi_dev<D, false, false>);
+const void *multi_kernel_dev(bool adjoint, bool s2) {
+  return adjoint ? (s2 ? (const void *)k_multi_dev<D, true, true> : (const void *)k_multi_dev<D, true, false>)
+                 : (s2 ? (const void *)k_multi_dev<D, false, true> : (const void *)k_multi_dev<D, false, false>);
+}
+
+template <int D>
+const void *multi_kernel_fp64(bool adjoint, bool s2) {
   return adjoint ? (s2 ? (const void *)k_multi_fp64<D, true, kModeS2> : (const void *)k_multi_fp64<D, true, kModeGeneral>)
                  : (s2 ? (const void *)k_multi_fp64<D, false, kModeS2> : (const void *)k_multi_fp64<D, false, kModeGeneral>);
 }
 
 const void *multi_kernel(int d, bool dev, bool adjoint, bool s2) {
-  return d == 1 ? multi_kernel<1>(dev, adjoint, s2) : multi_kernel<2>(dev, adjoint, s2);
+  if (!dev) return d == 1 ? multi_kernel_fp64<1>(adjoint, s2) : multi_kernel_fp64<2>(adjoint, s2);
+  return d == 1 ? multi_kernel_dev<1>(adjoint, s2) : (d == 2 ? multi_kernel_dev<2>(adjoint, s2) : multi_kernel_dev<3>(adjoint, s2));
 }
 
 }  // namespace
 
-// The plan of a periodic 1D / 2D box, or none (one step per launch). Small grids: one tile per SM, the one with the
+// The plan of a periodic box, or none (one step per launch). Small grids: one tile per SM, the one with the
 // smallest first region, a thread per node of it, and as many steps as pay for the rings that the tiles share
 // with their neighbours: FP64 is held back by the FP64 pipe (~2 operations per clock per SM, 10 a node), so that H
 // falls with the tile's size, and none pays from ~260^2 on. 32 bits pay further on, where a launch is short beside a
@@ -334,40 +377,47 @@ const void *multi_kernel(int d, bool dev, bool adjoint, bool s2) {
 //     adjoint 3.52 / 3.69 (not taken), 500 x 333 5.9 / 7.1 (32 x 8, H = 2; not taken); D1Q3 64 1.92 / 0.74, 30000 2.01 / 1.03,
 //     10^6 16.4 / 18.4 (not taken)
 //   32 bits D2Q9 16^2 1.90 / 0.60, 64^2 1.90 / 0.70, 128^2 1.90 / 0.84, 256^2 2.05 / 1.42, 320^2 2.29 / 2.23, 500 x 333 3.33 / 2.97, 1000^2
-//     11.7 / 12.1 (not taken), 1250^2 23.3 / 19.8, 2048^2 58.7 / 50.5; D1Q3 4096 1.89 / 0.47, 10^5 1.96 / 1.13, 2 10^6 17.1 / 8.3
+//     11.7 / 12.1 (not taken), 1250^2 23.3 / 19.8, 2048^2 58.7 / 50.5; D1Q3 4096 1.89 / 0.47, 10^5 1.96 / 1.13, 2 10^6 17.1 / 8.3;
+//     D3Q19 8^3 1.93 / 1.14, 16^3 1.95 / 1.44, 24^3 1.94 / 1.75, 28^3 2.18 / 2.13 (not taken); FP64 D3Q19 16^3 2.89 / 2.82, 20^3 2.94 / 3.05 (not taken)
 bool plan_multi(const Geom &g, bool dev, int sms, MultiPlan &best) {
   best = MultiPlan{};
-  if (g.d > 2 || sms <= 0) return false;
+  if (g.d > 3 || sms <= 0) return false;
   const int64_t S = g.S, share = (S + sms - 1) / sms;  // nodes per SM
-  const int ny = g.d == 2 ? g.n[1] : 1;
   // (a region that wraps around the box once at most)
-  auto fits = [&](int tx, int ty, int H) { return tx + H - 1 <= g.n[0] && (g.d < 2 || ty + H - 1 <= ny); };
+  auto fits = [&](int tx, int ty, int tz, int H) {
+    return tx + H - 1 <= g.n[0] && (g.d < 2 || ty + H - 1 <= g.n[1]) && (g.d < 3 || tz + H - 1 <= g.n[2]);
+  };
+  // one tile per SM, the smallest first region
+  auto search = [&](int H, int step, int most_x, int most_y, int most_z, int64_t most_nodes) {
+    int64_t least = INT64_MAX;
+    for (int tz = 1; tz <= most_z; ++tz)
+      for (int ty = 1; ty <= most_y; ++ty)
+        for (int tx = step; tx <= most_x; tx += step) {
+          if (!fits(tx, ty, tz, H)) continue;
+          const MultiPlan p = make_multi(g, dev, tx, ty, tz, H, multi_threads(g.d));
+          if (p.grid > sms || p.nodes > most_nodes || p.nodes >= least || p.smem > (size_t)kMultiMaxSmem) continue;
+          least = p.nodes;
+          best = p;
+        }
+  };
   if (g.d == 1) {
     if (!dev && share > 200) return false;
     const int tx = (int)std::min<int64_t>(512, std::max<int64_t>(32, share));
-    if (fits(tx, 1, kMultiMaxSteps)) best = make_multi(g, dev, tx, 1, kMultiMaxSteps, 256);
+    if (fits(tx, 1, 1, kMultiMaxSteps)) best = make_multi(g, dev, tx, 1, 1, kMultiMaxSteps, 256);
+  } else if (g.d == 3) {
+    if (dev && S <= 14000) search(S <= 4200 ? 3 : 2, 1, 24, 24, 24, 2048);
   } else if (share <= (dev ? 480 : 440)) {
-    const int H = dev ? (share <= 160 ? 6 : 4) : (share <= 48 ? 4 : (share <= 160 ? 3 : 2));
-    int64_t least = INT64_MAX;
-    for (int tx = 4; tx <= 64; tx += 4)
-      for (int ty = 1; ty <= 64; ++ty) {
-        if (!fits(tx, ty, H)) continue;
-        const int64_t tiles = (int64_t)((g.n[0] + tx - 1) / tx) * ((ny + ty - 1) / ty);
-        const int64_t region = (int64_t)(tx + 2 * (H - 1)) * (ty + 2 * (H - 1));
-        if (tiles > sms || region > kMultiThreads || region >= least) continue;
-        least = region;
-        best = make_multi(g, dev, tx, ty, H, kMultiThreads);
-      }
-  } else if (dev && S <= 180000 && fits(32, 8, 3)) {
-    best = make_multi(g, dev, 32, 8, 3, 192);
-  } else if (dev && S >= 1500000 && fits(32, 16, 2)) {
-    best = make_multi(g, dev, 32, 16, 2, 320);
+    search(dev ? (share <= 160 ? 6 : 4) : (share <= 48 ? 4 : (share <= 160 ? 3 : 2)), 4, 64, 64, 1, kMultiThreads);
+  } else if (dev && S <= 180000 && fits(32, 8, 1, 3)) {
+    best = make_multi(g, dev, 32, 8, 1, 3, 192);
+  } else if (dev && S >= 1500000 && fits(32, 16, 1, 2)) {
+    best = make_multi(g, dev, 32, 16, 1, 2, 320);
   }
   return best.H > 1;
 }
 
 MultiPlan shorter_multi(const Geom &g, bool dev, const MultiPlan &p, int H) {
-  return H == p.H ? p : make_multi(g, dev, p.tx, p.ty, H, p.threads);
+  return H == p.H ? p : make_multi(g, dev, p.t[0], p.t[1], p.t[2], H, p.threads);
 }
 
 cudaError_t prepare_multi(int d, bool dev, const MultiPlan &p) {

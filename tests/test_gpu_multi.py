@@ -1,4 +1,4 @@
-"""GPU: periodic 1D / 2D boxes taken several steps per launch give, bit for bit, the state, phi and gradients of one step per
+"""GPU: periodic boxes taken several steps per launch give, bit for bit, the state, phi and gradients of one step per
 call (which is one step per launch): grids on either side of every line of the rule, minimal and ragged extents (tiles that
 stick out, regions that wrap), counts of steps that are and are not multiples of a launch's, every collision form (over a
 return of the scaled state), constant and per-site sources, both precisions."""
@@ -23,7 +23,7 @@ def _run(n, precision, tau, R, Rf, calls, back, phi0, seed, pdl=True):
     import torch
 
     d = len(n)
-    sim = LBM(d, list(n), hi=[m / n[0] for m in n], u=(0.1, 0.05)[:d], R=R, tau=tau, precision=precision, pdl=pdl)
+    sim = LBM(d, list(n), hi=[m / n[0] for m in n], u=(0.1, 0.05, 0.02)[:d], R=R, tau=tau, precision=precision, pdl=pdl)
     sim.init(phi0, None, Rf)
     out = []
     for k in calls:
@@ -39,7 +39,8 @@ def _run(n, precision, tau, R, Rf, calls, back, phi0, seed, pdl=True):
 
 
 GRIDS = [(3,), (9,), (39,), (40,), (131,), (4096,), (30400,), (30401,), (77825,), (3, 3), (4, 5), (7, 6), (9, 13), (16, 16), (64, 64), (61, 67), (85, 86),
-         (33, 7), (300, 5), (156, 156), (157, 155), (258, 259), (270, 270), (271, 272), (500, 333), (430, 420), (1224, 1227)]
+         (33, 7), (300, 5), (156, 156), (157, 155), (258, 259), (270, 270), (271, 272), (500, 333), (430, 420), (1224, 1227),
+         (3, 3, 3), (5, 4, 6), (8, 8, 8), (16, 16, 16), (17, 15, 17), (24, 24, 24), (25, 23, 25), (7, 40, 11)]
 
 
 @pytest.mark.parametrize("n", GRIDS)
