@@ -90,8 +90,8 @@ __global__ void __launch_bounds__(256) k_macro_fp64(const StepArgs a, double *__
 }
 
 template <int D, bool ADJ, bool INTERIOR, bool TRIGGER>
-static cudaError_t launch_step_fp64_m(const StepArgs &a, unsigned blocks, cudaStream_t st) {
-  const int threads = LHE_STEP_THREADS;
+static cudaError_t launch_step_fp64_m(const StepArgs &a, int threads, cudaStream_t st) {
+  const unsigned blocks = (unsigned)((a.nwork + threads - 1) / threads);
   const bool pdl = a.pdl != 0;
   if (a.s == 2.0) return launch_kernel(k_step_fp64<D, ADJ, INTERIOR, kModeS2, TRIGGER>, blocks, threads, 0, st, pdl, a);
   if (a.collide == kCollideScaled)
@@ -102,11 +102,15 @@ static cudaError_t launch_step_fp64_m(const StepArgs &a, unsigned blocks, cudaSt
 template <int D, bool ADJ, bool INTERIOR>
 static cudaError_t launch_step_fp64_t(const StepArgs &a, cudaStream_t st) {
   if (a.nwork <= 0) return cudaSuccess;
-  const unsigned blocks = (unsigned)((a.nwork + LHE_STEP_THREADS - 1) / LHE_STEP_THREADS);
+  // about one wave: half-size CTAs share the nodes out more evenly (and, in the smallest grids, over more SMs' FP64 pipes): us
+  // per step with CTAs of 128 / 64 threads: D3Q19 40^3 5.81 / 5.46, 45 x 37 x 51 6.74 / 6.55, 16^3 2.89 / 2.77, D4Q33 12^4 5.84 / 5.07, 16^4 8.81 / 8.32;
+  // 24^4 28.8 / 28.6 and larger the same
+  const bool wave = a.nwork <= kTriggerCtasPerSM * a.sms * LHE_STEP_THREADS;
+  const int threads = wave ? LHE_STEP_THREADS / 2 : LHE_STEP_THREADS;
   if constexpr (!INTERIOR) {
-    if (ADJ || (int64_t)blocks <= kTriggerCtasPerSM * a.sms) return launch_step_fp64_m<D, ADJ, false, false>(a, blocks, st);
+    if (ADJ || wave) return launch_step_fp64_m<D, ADJ, false, false>(a, threads, st);
   }
-  if constexpr (INTERIOR || !ADJ) return launch_step_fp64_m<D, ADJ, INTERIOR, true>(a, blocks, st);
+  if constexpr (INTERIOR || !ADJ) return launch_step_fp64_m<D, ADJ, INTERIOR, true>(a, threads, st);
   return cudaErrorInvalidValue;  // not reached
 }
 
