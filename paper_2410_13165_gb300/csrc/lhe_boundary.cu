@@ -23,16 +23,24 @@
 // grouped by face signature so that a warp shares one set of unknown populations. The per-node
 // evaluation (lhe_bnode.cuh) is shared with the FP64 interior kernel of Dirichlet boxes, which treats
 // the nodes of the two x_1 faces (whose other coordinates are interior) in the lanes of their rows.
+#include <type_traits>
+
 #include "lhe_bnode.cuh"
 
 namespace lhe {
 
-template <int D, int KIND, bool DEV>
+template <int D, int KIND, bool DEV, bool EARLY>
 __global__ void __launch_bounds__(128) k_boundary(const BoundaryArgs a) {
   constexpr Lattice<D> L{};
   constexpr int Q = Lattice<D>::Q;
+  // the family's coefficients in shared memory: an unknown link's loads are behind a branch and follow one another
+  extern __shared__ double table[];
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   pdl_wait();
+  if (a.rec == nullptr) {
+    for (int i = threadIdx.x; i < 2 * (a.nmodes + 1) * Q; i += blockDim.x) table[i] = __ldg(a.table + i);
+    __syncthreads();
+  }
   if (t >= a.nsites) return;
   const int32_t site = a.sites[t];
   const int64_t S = a.g.S;
@@ -52,13 +60,24 @@ __global__ void __launch_bounds__(128) k_boundary(const BoundaryArgs a) {
   }
   BNode<D> nd;
   const bool jets = a.rec != nullptr;  // data from jet records (else from the exact-solution family)
-  if (!jets) bnode_prepare<D, KIND>(a, x, nd);
   const double *__restrict__ rec = jets ? a.rec + a.roff[t] : nullptr;
-  int ju = 0;
-
-  const double *__restrict__ fsrc = static_cast<const double *>(a.src);
-  const float *__restrict__ gsrc = static_cast<const float *>(a.src);
+  // EARLY: every load first, so that they are in flight together: a population is read at its pull source, or for an
+  // unknown link where the half-way scheme's f*_kbar lies, at the node itself. Else the loads are behind the branch on `inside` and
+  // follow one another, Q trips to L2 a node, which is what few nodes wait for; many nodes hide them, and are held back by the
+  // registers and the unknown links' extra loads instead. FP32 deviations, us per step, late / early, full-way and half-way:
+  // D3Q19 16^3 18.9 / 16.4 and 24.6 / 16.0, 48^3 (13,000 nodes) 20.9 / 18.4 and 27.0 / 18.1, D4Q33 16^4 (27,000) 36 / 32 and 47 / 32,
+  // 24^4 (97,500) 99 / 107 and 117 / 101, 32^4 (239,000) 241 / 326 and 275 / 312.
+  using T = typename std::conditional<DEV, float, double>::type;
+  const T *__restrict__ src = static_cast<const T *>(a.src);
+  T raw[EARLY ? Q : 1];
+  float2 ph[EARLY && DEV ? Q : 1];
   double v[Q];
+  uint64_t in = 0;  // links whose pull source lies in the box
+  int ju = 0;
+  auto value = [&](int k, int32_t o) {  // f*_k at o
+    return DEV ? fma(a.omega[k], df_value(a.phi_src[o]), (double)src[k * S + o]) : (double)src[k * S + o];
+  };
+  if (!EARLY && !jets) bnode_prepare<D, KIND>(a, x, nd);
 #pragma unroll
   for (int k = 0; k < Q; ++k) {
     bool inside = true;
@@ -71,15 +90,35 @@ __global__ void __launch_bounds__(128) k_boundary(const BoundaryArgs a) {
         o -= L.e[k][i] * a.g.stride[i];
       }
     }
-    if (inside) {
-      v[k] = DEV ? fma(a.omega[k], df_value(a.phi_src[o]), (double)gsrc[k * S + o]) : fsrc[k * S + o];
-      continue;
-    }
-    if (jets) {
-      const double b = a.rec_scale * __ldg(rec + ju++);
-      v[k] = KIND == 1 ? b : b - bnode_fkb<D, DEV>(a, k, site);
+    if constexpr (EARLY) {
+      in |= (uint64_t)inside << k;
+      raw[k] = __ldg(src + (inside ? k * S + o : (KIND == 2 ? L.opp[k] * S + site : site)));
+      if (DEV) ph[k] = __ldg(a.phi_src + (inside ? o : site));
+      v[k] = jets && !inside ? __ldg(rec + ju) : 0.0;
+      ju += inside ? 0 : 1;
+    } else if (inside) {
+      v[k] = value(k, o);
     } else {
-      v[k] = bnode_unknown<D, KIND, DEV>(a, nd, k, site);
+      // (one rounding for a record's scale and the half-way difference, as in k_bdata_step)
+      const double less = KIND == 1 ? 0.0 : value(L.opp[k], site);
+      if (jets) v[k] = KIND == 1 ? a.rec_scale * __ldg(rec + ju++) : fma(a.rec_scale, __ldg(rec + ju++), -less);
+      else v[k] = KIND == 1 ? bnode_data<D, KIND>(a, table, nd, k) : bnode_data<D, KIND>(a, table, nd, k) - less;
+    }
+  }
+  if constexpr (EARLY) {
+    if (!jets) bnode_prepare<D, KIND>(a, x, nd);
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+      const bool inside = (in >> k) & 1ull;
+      const double there = DEV ? fma(inside ? a.omega[k] : a.omega[L.opp[k]], float_to_double(ph[k].x) + float_to_double(ph[k].y),
+                                     float_to_double((float)raw[k]))
+                               : (double)raw[k];
+      if (inside) {
+        v[k] = there;
+        continue;
+      }
+      if (jets) v[k] = KIND == 1 ? a.rec_scale * v[k] : fma(a.rec_scale, v[k], -there);
+      else v[k] = KIND == 1 ? bnode_data<D, KIND>(a, table, nd, k) : bnode_data<D, KIND>(a, table, nd, k) - there;
     }
   }
   // collision, as in the bulk: phi = sum_k f_k (the split moment sum of the row kernels), f*_k = (1 - s) f_k +
@@ -299,7 +338,7 @@ cudaError_t launch_jet_grad(int d, int kind, bool dev, const BoundaryArgs &a, co
 // rho_k <- (1 - s) mu_k + s omega_k sum_j mu_j, as in the bulk. FP32 deviations (DEV): the adjoint state
 // is rho_k = omega_k W + eps_k (W a double-float pair, eps in FP32), formed in FP64 here, and the result
 // is stored as the forward boundary kernel stores a state: W' = sum_j mu_j, eps'_k = rho'_k - omega_k W'.
-template <int D, int KIND, bool DEV>
+template <int D, int KIND, bool DEV, bool EARLY>
 __global__ void __launch_bounds__(128) k_adj_boundary(const BoundaryArgs a) {
   constexpr Lattice<D> L{};
   constexpr int Q = Lattice<D>::Q;
@@ -322,13 +361,16 @@ __global__ void __launch_bounds__(128) k_adj_boundary(const BoundaryArgs a) {
       }
     }
   }
-  const double *__restrict__ src = static_cast<const double *>(a.src);
-  const float *__restrict__ esrc = static_cast<const float *>(a.src);
-  // the adjoint state rho_j at node o
-  auto rho = [&](int j, int32_t o) {
-    return DEV ? fma(a.omega[j], df_value(a.phi_src[o]), (double)esrc[j * S + o]) : src[j * S + o];
-  };
+  using T = typename std::conditional<DEV, float, double>::type;
+  const T *__restrict__ src = static_cast<const T *>(a.src);
+  // EARLY as in k_boundary: every load first, rho_k at x + e_k, or for a link that leaves the box rho_kbar at the node
+  T raw[EARLY ? Q : 1];
+  float2 ph[EARLY && DEV ? Q : 1];
   double mu[Q];
+  uint64_t in = 0;
+  auto rho = [&](int k, int32_t o) {
+    return DEV ? fma(a.omega[k], df_value(a.phi_src[o]), (double)src[k * S + o]) : (double)src[k * S + o];
+  };
 #pragma unroll
   for (int k = 0; k < Q; ++k) {
     bool inside = true;
@@ -341,8 +383,24 @@ __global__ void __launch_bounds__(128) k_adj_boundary(const BoundaryArgs a) {
         o += L.e[k][i] * a.g.stride[i];
       }
     }
-    if (inside) mu[k] = rho(k, o);
-    else mu[k] = KIND == 2 ? -a.wratio[k] * rho(L.opp[k], site) : 0.0;
+    if constexpr (EARLY) {
+      in |= (uint64_t)inside << k;
+      raw[k] = __ldg(src + (inside ? k * S + o : L.opp[k] * S + site));
+      if (DEV) ph[k] = __ldg(a.phi_src + (inside ? o : site));
+    } else {
+      if (inside) mu[k] = rho(k, o);
+      else mu[k] = KIND == 2 ? -a.wratio[k] * rho(L.opp[k], site) : 0.0;
+    }
+  }
+  if constexpr (EARLY) {
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+      const bool inside = (in >> k) & 1ull;
+      const double there = DEV ? fma(inside ? a.omega[k] : a.omega[L.opp[k]], float_to_double(ph[k].x) + float_to_double(ph[k].y),
+                                     float_to_double((float)raw[k]))
+                               : (double)raw[k];
+      mu[k] = inside ? there : (KIND == 2 ? -a.wratio[k] * there : 0.0);
+    }
   }
   if (DEV) {
     const double M = fixed_moment_sum<Q, 0>(mu);
@@ -368,13 +426,21 @@ __global__ void __launch_bounds__(128) k_adj_boundary(const BoundaryArgs a) {
   }
 }
 
+constexpr int64_t kEarlyNodes = 40000;  // boundary nodes up to which the kernels issue every load first (k_boundary)
+
+// Threads per CTA of the boundary-node kernels: a node is ~150 FP64 operations behind several dependent loads, so few
+// nodes are spread over as many SMs as there are (128 threads: D3Q19 32^3, 5768 nodes, on 46 of 152 SMs).
+static int boundary_threads(int64_t nodes) { return nodes <= 152 * 4 * 32 ? 32 : (nodes <= 152 * 8 * 64 ? 64 : 128); }
+
 template <int D>
 static cudaError_t adj_boundary_d(int kind, bool dev, const BoundaryArgs &a, cudaStream_t st) {
   if (a.nsites <= 0) return cudaSuccess;
-  const unsigned blocks = (unsigned)((a.nsites + 127) / 128);
-  auto kernel = kind == 1 ? (dev ? k_adj_boundary<D, 1, true> : k_adj_boundary<D, 1, false>)
-                          : (dev ? k_adj_boundary<D, 2, true> : k_adj_boundary<D, 2, false>);
-  return launch_kernel(kernel, blocks, 128, 0, st, a.pdl != 0, a);
+  const int threads = boundary_threads(a.nsites);
+  const unsigned blocks = (unsigned)((a.nsites + threads - 1) / threads);
+  auto kernel = !dev ? (kind == 1 ? k_adj_boundary<D, 1, false, false> : k_adj_boundary<D, 2, false, false>)
+                : a.nsites <= kEarlyNodes ? (kind == 1 ? k_adj_boundary<D, 1, true, true> : k_adj_boundary<D, 2, true, true>)
+                                          : (kind == 1 ? k_adj_boundary<D, 1, true, false> : k_adj_boundary<D, 2, true, false>);
+  return launch_kernel(kernel, blocks, threads, 0, st, a.pdl != 0, a);
 }
 
 cudaError_t launch_adjoint_boundary(int d, int kind, bool dev, const BoundaryArgs &a, cudaStream_t st) {
@@ -391,11 +457,13 @@ cudaError_t launch_adjoint_boundary(int d, int kind, bool dev, const BoundaryArg
 template <int D>
 static cudaError_t boundary_d(int kind, bool dev, const BoundaryArgs &a, cudaStream_t st) {
   if (a.nsites <= 0) return cudaSuccess;
-  const int threads = 128;
+  const int threads = boundary_threads(a.nsites);
   const unsigned blocks = (unsigned)((a.nsites + threads - 1) / threads);
-  auto kernel = kind == 1 ? (dev ? k_boundary<D, 1, true> : k_boundary<D, 1, false>)
-                          : (dev ? k_boundary<D, 2, true> : k_boundary<D, 2, false>);
-  return launch_kernel(kernel, blocks, threads, 0, st, a.pdl != 0, a);
+  auto kernel = !dev ? (kind == 1 ? k_boundary<D, 1, false, false> : k_boundary<D, 2, false, false>)
+                : a.nsites <= kEarlyNodes ? (kind == 1 ? k_boundary<D, 1, true, true> : k_boundary<D, 2, true, true>)
+                                          : (kind == 1 ? k_boundary<D, 1, true, false> : k_boundary<D, 2, true, false>);
+  const size_t smem = a.rec ? 0 : sizeof(double) * 2 * (size_t)(a.nmodes + 1) * Lattice<D>::Q;
+  return launch_kernel(kernel, blocks, threads, smem, st, a.pdl != 0, a);
 }
 
 cudaError_t launch_boundary(int d, int kind, bool dev, const BoundaryArgs &a, cudaStream_t st) {
