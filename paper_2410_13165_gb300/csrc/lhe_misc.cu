@@ -83,7 +83,7 @@ cudaError_t launch_fd_grad_transpose_add(int d, const Geom &g, double dx, const 
 // (Ziv's rounding test, "Fast evaluation of elementary mathematical functions with correctly rounded last
 // bit", TOMS 1991), and every one outside the pairs' range (largest term outside 2^-60 .. 2^100, infinities, NaN),
 // is formed in FP64 instead, so the stored floats are those of the FP64 form at every node. D3Q19 128^3
-// 451 -> 80 us (memory floor 36), D5Q51 24^5 4.24 -> 0.89 ms (floor 0.26).
+// 451 -> 77 us (memory floor 36), D5Q51 24^5 4.24 -> 0.66 ms (floor 0.26).
 constexpr int kGradNone = 0, kGradGiven = 1, kGradFD = 2;
 
 // v_k = omega_k (B - sum_i e_ki h_i) for every k, with the arithmetic of T (double or float pairs).
@@ -186,16 +186,21 @@ __global__ void __launch_bounds__(256) k_init(const __grid_constant__ InitArgs a
       // of its operands) and the rounding of the FP64 differences, 2^-48 of the values that enter them
       err *= 0x1p-43f;
       if (GRAD == kGradFD) err = fmaf(a.werr * 0x1p-48f, ff_split(__hiloint2double((int)near, 0)).x, err);
+      uint64_t doubt = 0;  // populations whose rounding the pairs do not decide
       init_populations<D>(
           B, h, [](float2 p, float2 q) { return ff_add(p, q); }, [](float2 p, float2 q) { return ff_sub(p, q); },
           [&](int k, float2 v) {
             const float2 w = a.omega_f[k];
             const float p = __fmul_rn(w.x, v.x);
             const float e = __fmaf_rn(w.x, v.y, __fmaf_rn(w.y, v.x, __fmaf_rn(w.x, v.x, -p)));
-            float r = __fadd_rn(p, __fmaf_rn(w.x, err, e));
-            if (r != __fadd_rn(p, __fmaf_rn(-w.x, err, e))) r = deviation_fp64<D, GRAD>(a, site, k);
+            const float r = __fadd_rn(p, __fmaf_rn(w.x, err, e));
+            doubt |= (uint64_t)(r != __fadd_rn(p, __fmaf_rn(-w.x, err, e))) << k;
             dst[k * S + site] = r;
           });
+      for (; doubt; doubt &= doubt - 1) {  // (one place for the rare FP64 form: with a call per population D5Q51 24^5 took 0.89 ms)
+        const int k = __ffsll((long long)doubt) - 1;
+        dst[k * S + site] = deviation_fp64<D, GRAD>(a, site, k);
+      }
       return;
     }
     for (int k = 0; k < Lattice<D>::Q; ++k) dst[k * S + site] = deviation_fp64<D, GRAD>(a, site, k);
