@@ -179,18 +179,12 @@ __device__ __forceinline__ double fixed_moment_sum(const double (&f)[Q]) {
   return fixed_moment_sum_impl<Q, P2>([&](int k) { return f[k]; });
 }
 
-// Moment sum of the FP64 step kernels of the larger lattices. The fixed-point sum's integer work grows
-// with Q while the FP64 pipe, which the collision keeps about half busy, has room: the first NFX terms
-// are summed in fixed point and the rest added on the FP64 pipe. The split is chosen per kernel from
-// scans on GB300 (number of fixed-point terms): the periodic step splits D5Q51 only (38 of 51: 24^5
-// 1.269 -> 1.148 ms; a D4Q33 split made the 48^4 step slower, 0.444 -> 0.467 ms), the row kernels of
-// Dirichlet boxes split D4Q33 as well (29 of 33: 64^4 1.711 -> 1.672 ms). The error is within
-// (Q - NFX + 1) / 2 units in the last place of the sum (the oracle's sequential FP64 sum: up to
-// (Q - 1) / 2).
+// Moment sum of the boundary nodes of FP32-deviation boxes in d = 4, 5: the first NFX terms in fixed point, the rest
+// added on the FP64 pipe (their stored floats keep the rounding they had). The FP64 steps split their sums the same
+// way while a fixed-point term took ~30 integer instructions; at ~20 the whole sum in fixed point is faster, us per step, split /
+// whole: D5Q51 24^5 1021 / 930, 12^5 39.4 / 35.7, 8^5 8.8 / 8.4 (38 of 51 terms), D4Q33 boxes 32^4 106.5 / 102.0, 48^4 475 / 457 (29 of 33).
 template <int Q>
-constexpr int kPeriodicFixedTerms = Q == 51 ? 38 : Q;
-template <int Q>
-constexpr int kBoxFixedTerms = Q == 51 ? 38 : (Q == 33 ? 29 : Q);
+constexpr int kNodeFixedTerms = Q == 51 ? 38 : (Q == 33 ? 29 : Q);
 
 template <int Q, int NFX>
 __device__ __forceinline__ double split_moment_sum(const double (&f)[Q]) {

@@ -40,17 +40,7 @@ __global__ void __launch_bounds__(LHE_STEP_THREADS) k_step_fp64(const StepArgs a
 #pragma unroll
   for (int k = 0; k < Q; ++k) f[k] = __ldg(src + k * S + source_site<D, ADJ>(L, k, site, om, op));
   double psi;
-  if (kPeriodicFixedTerms<Q> < Q) {  // the split sum (lhe_device.cuh); 2 w and 2 phi are exact doublings
-    const double w = split_moment_sum<Q, kPeriodicFixedTerms<Q>>(f);
-    if (ADJ) {
-      psi = MODE == kModeS2 ? 2.0 * w : a.sig * w;
-      if (a.gR) a.gR[site] = MODE == kModeS2 ? fma(a.half_dt, psi, a.gR[site]) : fma(a.gsc, w, a.gR[site]);
-    } else if (MODE == kModeS2) {
-      psi = fma(2.0, w, a.Rfield ? a.dt * __ldg(a.Rfield + site) : a.dtR);
-    } else {
-      psi = fma(a.sig, w, a.Rfield ? a.rho_dt * __ldg(a.Rfield + site) : a.rho_dtR);
-    }
-  } else if (ADJ) {
+  if (ADJ) {
     if (MODE == kModeS2) {
       psi = fixed_moment_sum<Q, 1>(f);  // 2 w
       if (a.gR) a.gR[site] = fma(a.half_dt, psi, a.gR[site]);
