@@ -751,9 +751,13 @@ lhe_status lhe_lbm_init(lhe_lbm *l, const double *phi0, const double *grad, cons
     a.u[i] = l->p.u[i];
   }
   a.werr += (float)std::fabs(a.wc);
+  // 2^-94 of dt R and of each difference (8 and 1 times, or the gradient once) with its weights; products of the weights
+  // that float pairs take (2^-40 and up) with that lie far above the subnormals, whose own errors it covers
+  a.edrop = 0x1p-94f * (1.0f + 9.0f * a.werr);
   for (int k = 0; k < l->Q; ++k) {
     a.omega[k] = l->omega[k];
     a.omega_f[k] = pair(l->omega[k]);
+    a.pairs = a.pairs && in_range(a.omega[k]);
     a.c1[k] = (1.0 - l->s) * 0.5 * l->dt * l->omega[k];
     a.c2[k] = l->p.c * a.c1[k];
     for (int i = 0; i < d; ++i) a.e[k][i] = (int8_t)l->e[k * d + i];

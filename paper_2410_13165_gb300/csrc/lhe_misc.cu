@@ -82,7 +82,9 @@ cudaError_t launch_fd_grad_transpose_add(int d, const Geom &g, double dx, const 
 // pipe and only the differences of phi0 in FP64. A result whose rounding the pairs' error could change
 // (Ziv's rounding test, "Fast evaluation of elementary mathematical functions with correctly rounded last
 // bit", TOMS 1991), and every one outside the pairs' range (largest term outside 2^-60 .. 2^100, infinities, NaN),
-// is formed in FP64 instead, so the stored floats are those of the FP64 form at every node. D3Q19 128^3
+// is formed in FP64 instead, so the stored floats are those of the FP64 form at every node. (The test's bound counts
+// what ff_split drops of a term below 2^-70, at most 2^-94, with the largest weight it can meet: relative to the largest
+// term alone, a source of 2^-71 beside a gradient of 2^-58 was rounded wrongly at 2 to 3 of 100 populations.) D3Q19 128^3
 // 451 -> 77 us (memory floor 36), D5Q51 24^5 4.24 -> 0.66 ms (floor 0.26).
 constexpr int kGradNone = 0, kGradGiven = 1, kGradFD = 2;
 
@@ -183,8 +185,9 @@ __global__ void __launch_bounds__(256) k_init(const __grid_constant__ InitArgs a
         err = fmaf(a.werr, m, err);
       }
       // bound of the difference to the FP64 form: 2^-43 of the terms (an operation on pairs is within ~2^-45
-      // of its operands) and the rounding of the FP64 differences, 2^-48 of the values that enter them
+      // of its operands), what the split drops, and the rounding of the FP64 differences, 2^-48 of the values that enter them
       err *= 0x1p-43f;
+      if (top != -1023) err += a.edrop;
       if (GRAD == kGradFD) err = fmaf(a.werr * 0x1p-48f, ff_split(__hiloint2double((int)near, 0)).x, err);
       uint64_t doubt = 0;  // populations whose rounding the pairs do not decide
       init_populations<D>(
