@@ -192,7 +192,7 @@ struct InitArgs {
   float werr;              // |wc| + sum_i |wu_i|
   float edrop;             // largest error of a node from what ff_split drops of its terms
   int32_t pairs;           // the weights lie well inside the range of float pairs
-  // the FP64 form of one population (lhe_misc.cu deviation_fp64)
+  // the FP64 form of the populations (lhe_misc.cu deviations_fp64)
   double c1[kMaxQ];        // (1 - s)(dt/2) omega_k
   double c2[kMaxQ];        // c (1 - s)(dt/2) omega_k
   double u[kMaxD];

@@ -111,28 +111,59 @@ __device__ __forceinline__ void init_populations(T B, const T (&h)[D], Add add, 
     }
 }
 
-// g*_k of one node and population in FP64, rounded to float.
+// g*_k of one node in FP64, rounded to float, for the populations of `mask` at least. The gradient is formed once; a
+// few populations are formed one by one, and all of them together (the others' stored floats stay the same) once a
+// lane of the warp has half of them to do, as on plateaus of phi0, where the pairs decide no rounding.
 template <int D, int GRAD>
-__device__ __noinline__ float deviation_fp64(const InitArgs &a, int32_t site, int k) {
+__device__ __noinline__ void deviations_fp64(const InitArgs &a, int32_t site, uint64_t mask) {
+  constexpr Lattice<D> L{};
+  constexpr int Q = Lattice<D>::Q;
   const double dtR = a.Rfield ? a.dt * __ldg(a.Rfield + site) : a.dtR;
   int x[D];
   decode_site<D, false>(a.g, site, x);
-  double ug = 0.0, eg = 0.0;
+  double gr[D], ug = 0.0;
+#pragma unroll
   for (int i = 0; i < D; ++i) {
-    double gr = 0.0;
-    if (GRAD == kGradGiven) gr = __ldg(a.grad + i * a.g.S + site);
+    gr[i] = 0.0;
+    if (GRAD == kGradGiven) gr[i] = __ldg(a.grad + i * a.g.S + site);
     if (GRAD == kGradFD) {
       const double p2 = __ldg(a.phi0 + site + wrap_off(x[i], 2, a.g.n[i], a.g.stride[i]));
       const double p1 = __ldg(a.phi0 + site + wrap_off(x[i], 1, a.g.n[i], a.g.stride[i]));
       const double m1 = __ldg(a.phi0 + site + wrap_off(x[i], -1, a.g.n[i], a.g.stride[i]));
       const double m2 = __ldg(a.phi0 + site + wrap_off(x[i], -2, a.g.n[i], a.g.stride[i]));
-      gr = (fma(-8.0, m1, fma(8.0, p1, -p2)) + m2) * a.inv12dx;
+      gr[i] = (fma(-8.0, m1, fma(8.0, p1, -p2)) + m2) * a.inv12dx;
     }
-    ug = fma(a.u[i], gr, ug);
-    if (a.e[k][i] == 1) eg += gr;
-    if (a.e[k][i] == -1) eg -= gr;
+    ug = fma(a.u[i], gr[i], ug);
   }
-  return (float)fma(a.omega[k], dtR, fma(-a.c2[k], eg, a.c1[k] * ug));
+  float *__restrict__ dst = static_cast<float *>(a.dst) + site;
+  const auto value = [&](int k, double eg) { return (float)fma(a.omega[k], dtR, fma(-a.c2[k], eg, a.c1[k] * ug)); };
+  if (__any_sync(__activemask(), __popcll(mask) > Q / 2)) {
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+      double eg = 0.0;
+#pragma unroll
+      for (int i = 0; i < D; ++i) {
+        if (L.e[k][i] == 1) eg += gr[i];
+        if (L.e[k][i] == -1) eg -= gr[i];
+      }
+      dst[k * a.g.S] = value(k, eg);
+    }
+    return;
+  }
+  for (; mask; mask &= mask - 1) {
+    const int k = __ffsll((long long)mask) - 1;
+    double g0 = 0.0, g1 = 0.0;  // e_ki d_i phi0 of the link's first and last direction (a sum over all i is D FP64 operations)
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      const int e = a.e[k][i];
+      const double v = __hiloint2double(__double2hiint(gr[i]) ^ (e & (int)0x80000000), __double2loint(gr[i]));
+      if (e != 0) {
+        g0 = g1;
+        g1 = v;
+      }
+    }
+    dst[k * a.g.S] = value(k, g0 + g1);
+  }
 }
 
 template <int D, bool DEV, int GRAD>
@@ -168,6 +199,7 @@ __global__ void __launch_bounds__(256) k_init(const __grid_constant__ InitArgs a
     }
     const int ep = double_exponent(phi0), en = (int)(near >> 20) - 1023;
     a.phi_dst[site] = (ep >= -60 && ep <= 100) ? ff_split(phi0) : df_split(phi0);
+    uint64_t doubt = ~0ull;  // populations whose rounding the pairs do not decide
     if (a.pairs && en <= 100 && ((top >= -60 && top <= 100) || top == -1023)) {
       float2 h[D], B = ff_split(dtR);
       float err = fabsf(B.x);  // sum of the magnitudes of the terms
@@ -186,27 +218,25 @@ __global__ void __launch_bounds__(256) k_init(const __grid_constant__ InitArgs a
       }
       // bound of the difference to the FP64 form: 2^-43 of the terms (an operation on pairs is within ~2^-45
       // of its operands), what the split drops, and the rounding of the FP64 differences, 2^-48 of the values that enter them
+      const float terms = err;
       err *= 0x1p-43f;
       if (top != -1023) err += a.edrop;
       if (GRAD == kGradFD) err = fmaf(a.werr * 0x1p-48f, ff_split(__hiloint2double((int)near, 0)).x, err);
-      uint64_t doubt = 0;  // populations whose rounding the pairs do not decide
-      init_populations<D>(
-          B, h, [](float2 p, float2 q) { return ff_add(p, q); }, [](float2 p, float2 q) { return ff_sub(p, q); },
-          [&](int k, float2 v) {
-            const float2 w = a.omega_f[k];
-            const float p = __fmul_rn(w.x, v.x);
-            const float e = __fmaf_rn(w.x, v.y, __fmaf_rn(w.y, v.x, __fmaf_rn(w.x, v.x, -p)));
-            const float r = __fadd_rn(p, __fmaf_rn(w.x, err, e));
-            doubt |= (uint64_t)(r != __fadd_rn(p, __fmaf_rn(-w.x, err, e))) << k;
-            dst[k * S + site] = r;
-          });
-      for (; doubt; doubt &= doubt - 1) {  // (one place for the rare FP64 form: with a call per population D5Q51 24^5 took 0.89 ms)
-        const int k = __ffsll((long long)doubt) - 1;
-        dst[k * S + site] = deviation_fp64<D, GRAD>(a, site, k);
+      if (err <= terms * 0x1p-28f) {  // (else few roundings are decided: plateaus of phi0, or a small signal on a large mean)
+        doubt = 0;
+        init_populations<D>(
+            B, h, [](float2 p, float2 q) { return ff_add(p, q); }, [](float2 p, float2 q) { return ff_sub(p, q); },
+            [&](int k, float2 v) {
+              const float2 w = a.omega_f[k];
+              const float p = __fmul_rn(w.x, v.x);
+              const float e = __fmaf_rn(w.x, v.y, __fmaf_rn(w.y, v.x, __fmaf_rn(w.x, v.x, -p)));
+              const float r = __fadd_rn(p, __fmaf_rn(w.x, err, e));
+              doubt |= (uint64_t)(r != __fadd_rn(p, __fmaf_rn(-w.x, err, e))) << k;
+              dst[k * S + site] = r;
+            });
       }
-      return;
     }
-    for (int k = 0; k < Lattice<D>::Q; ++k) dst[k * S + site] = deviation_fp64<D, GRAD>(a, site, k);
+    if (doubt) deviations_fp64<D, GRAD>(a, site, doubt);
     return;
   }
   double h[D], B = phi0 + dtR;

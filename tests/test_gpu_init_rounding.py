@@ -43,3 +43,66 @@ def test_terms_far_apart_round_once(d, n, eg, er, dx):
     bad = np.abs(got - want) > 0.5 * ulp + 16 * 2.0 ** -53 * np.abs(w)[:, None] * size
     assert not bad.any(), (int(bad.sum()), bad.size)
     sim.close()
+
+
+# a constant field, one that varies along one axis only, a small signal on a large mean, and a velocity that keeps the
+# gradient's weights out of the range of float pairs: few roundings or none are decided by the pairs
+@pytest.mark.parametrize("kind", ["constant", "rows", "mean", "slow"])
+@pytest.mark.parametrize("d,n", [(2, (61, 53)), (3, (19, 17, 21)), (5, (7, 6, 7, 5, 6))])
+def test_undecided_nodes_round_once(d, n, kind):
+    import torch
+
+    rng = np.random.default_rng(d)
+    S = int(np.prod(n))
+    u = (1e-14,) * d if kind == "slow" else (0.1, 0.08, 0.06, 0.04, 0.02)[:d]
+    phi0 = {"constant": np.full(S, 1.37), "rows": np.sin(np.arange(S) % n[0] * 2 * np.pi / n[0]),
+            "mean": 1.37 + 2.0 ** -rng.integers(10, 40, S) * rng.standard_normal(S), "slow": rng.standard_normal(S)}[kind]
+    sim = LBM(d, n, hi=[float(m) for m in n], u=u, tau=0.8, precision="fp32dev")
+    t = torch.from_numpy(phi0).cuda()
+    v = phi0.reshape(n[::-1])
+    r = lambda i, k: np.roll(v, -k, d - 1 - i).ravel()  # noqa: E731
+    grad = np.stack([(-r(i, 2) + 8 * r(i, 1) - 8 * r(i, -1) + r(i, -2)) / 12 for i in range(d)])
+    sim.init(t)
+    got = sim.get_state().cpu().numpy()[: sim.Q * S * 4].view(np.float32).reshape(sim.Q, S)
+    w, e, half = np.array(sim.omega), np.array(sim.e, dtype=float), 0.5 * (1 - sim.s)
+    want = w[:, None] * (half * ((np.array(u) @ grad)[None] - e @ grad))
+    size = abs(half) * (np.abs(np.array(u)) @ np.abs(grad) + np.abs(e) @ np.abs(grad))
+    # the differences' own rounding: 24 |phi0| of rounded terms over 12, in each direction
+    tol = 16 * 2.0 ** -53 * np.abs(w)[:, None] * (size + 2 * d * abs(half) * np.abs(phi0).max())
+    ulp = np.spacing(np.abs(want).astype(np.float32)).astype(np.float64)
+    bad = np.abs(got - want) > 0.5 * ulp + tol
+    assert not bad.any(), (int(bad.sum()), bad.size)
+    sim.close()
+
+
+def _ms(fn):
+    import torch
+
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    best = 1e30
+    for _ in range(6):
+        a.record()
+        for _ in range(5):
+            fn()
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b) / 5)
+    return best
+
+
+@pytest.mark.parametrize("kind", ["constant", "mean", "slow"])
+@pytest.mark.parametrize("d,n,limit", [(3, 128, 4.0), (5, 16, 4.0)])
+def test_undecided_nodes_cost_like_fp64(d, n, limit, kind):
+    """Nodes whose roundings the pairs do not decide take one gradient and a few FP64 operations per population: within a
+    small multiple of the FP64 initialisation of the same field (a gradient per population took 8 times as long)."""
+    import torch
+
+    x = torch.sin(torch.arange(n ** d, dtype=torch.float64, device="cuda"))
+    x = {"constant": 0 * x + 1.37, "mean": 1.37 + 1e-6 * x, "slow": x}[kind]
+    ms = []
+    for precision in ("fp64", "fp32dev"):
+        sim = LBM(d, n, u=(1e-14 if kind == "slow" else 0.05,) * d, tau=0.8, precision=precision)
+        sim.init(x)
+        ms.append(_ms(lambda: sim.init(x)))
+        sim.close()
+    assert ms[1] < limit * ms[0], ms
