@@ -106,14 +106,15 @@ constexpr unsigned kExpField = 0x7FF00000u;  // exponent field in the high word 
 // rounded term is (t + 1) >> 1 for either sign. Zero and subnormal terms get an implicit bit too and fall
 // below the frame, whose lowest bit is at least 2^(68 - 1023 - 52 - G). About 20 integer instructions a term (the
 // direct form, half a unit added before the shift and the sign after it, took about 30: D3Q19 step, 994 -> 809
-// instructions a node).
+// instructions a node). LOW: for frames from 1 << 20 on, where subnormal terms count (two instructions more).
 constexpr unsigned kFixedLeast = 68u << 20;
 
-template <int G>
+template <int G, bool LOW = false>
 __device__ __forceinline__ long long fixed_align(double f, unsigned emf) {
-  const unsigned hi = (unsigned)__double2hiint(f), lo = (unsigned)__double2loint(f);
-  const unsigned sh = min((emf - (hi & kExpField)) >> 20, 63u);
-  const unsigned long long m = (((unsigned long long)((hi & 0x000FFFFFu) | 0x00100000u)) << 32 | lo) << (G + 1);
+  const unsigned hi = (unsigned)__double2hiint(f), lo = (unsigned)__double2loint(f), ef = hi & kExpField;
+  const unsigned sh = min((emf - (LOW ? max(ef, 0x00100000u) : ef)) >> 20, 63u);
+  const unsigned one = LOW ? min(ef, 0x00100000u) : 0x00100000u;  // the implicit bit
+  const unsigned long long m = (((unsigned long long)((hi & 0x000FFFFFu) | one)) << 32 | lo) << (G + 1);
   const long long t = (long long)(m >> sh) ^ (long long)((int)hi >> 31);
   return (t + 1) >> 1;
 }
@@ -162,15 +163,26 @@ __device__ __forceinline__ double fixed_moment_sum_impl(Get f) {
 #pragma unroll
   for (int k = 0; k < Q; ++k) emf = max(emf, (unsigned)__double2hiint(f(k)) & kExpField);
   if (emf == kExpField) return __longlong_as_double(0x7FF8000000000000ll);
-  if (emf < kFixedLeast) {  // every term below 2^-954 (a field of zeros, for one): plain sum
-    double s = 0.0;
+  if constexpr (Q > 3) {
+    if (emf < kFixedLeast) {
+      // Every term below 2^-954. Zeros take no FP64 operation: summed as the tiny terms are, regions of them were stepped 1.4 to
+      // 1.7 times slower than others (D3Q19 256^3: 1.26 ms, now 0.73; 1000^2: 40 us, now 23). Tiny terms in fixed point too,
+      // here or in a function apart, made every step of small grids 1 to 3 % slower.
+      unsigned any = 0u;
 #pragma unroll
-    for (int k = 0; k < Q; ++k) s += f(k);
-    return s * (double)(1 << P2);
+      for (int k = 0; k < Q; ++k) any |= ((unsigned)__double2hiint(f(k)) & 0x7FFFFFFFu) | (unsigned)__double2loint(f(k));
+      if (any == 0u) return 0.0;
+      double s = 0.0;
+#pragma unroll
+      for (int k = 0; k < Q; ++k) s += f(k);
+      return s * (double)(1 << P2);
+    }
+  } else {  // three terms: the branch would be predicated, and its additions cost as much as if it were taken (D1Q3, 1.35 M nodes: 19.5 us a step, now 12.7)
+    emf = max(emf, 0x00100000u);
   }
   long long acc = 0;
 #pragma unroll
-  for (int k = 0; k < Q; ++k) acc += fixed_align<G>(f(k), emf);
+  for (int k = 0; k < Q; ++k) acc += fixed_align<G, (Q <= 3)>(f(k), emf);
   return fixed_value<G, P2>(acc, emf);
 }
 
