@@ -260,7 +260,11 @@ __global__ void __launch_bounds__(256) k_bdata_step(const BoundaryArgs b, const 
 // one or, when unknown, the entry of the dense array that k_bdata_step set for this step; then the
 // collision of the bulk. No arithmetic per link: on GB300 an FP64 operation per link costs as much as
 // the collision (the FP64 pipe retires ~2 per clock per SM).
-template <int D, int MODE>
+// SRC: constant R, a source field, or a field times Rscale. (Apart, because an FP64 operation of a form that is not taken
+// costs as much as one that runs: with the scale chosen at run time the rows of 4000^2 boxes without a source took 667 us a step, now 604 (638 before there was a scale).)
+constexpr int kSrcConst = 0, kSrcField = 1, kSrcScaled = 2;
+
+template <int D, int MODE, int SRC>
 __global__ void __launch_bounds__(LHE_STEP_THREADS) k_step_box_dense(const StepArgs a, const double *__restrict__ bdata) {
   constexpr Lattice<D> L{};
   constexpr int Q = Lattice<D>::Q;
@@ -276,7 +280,7 @@ __global__ void __launch_bounds__(LHE_STEP_THREADS) k_step_box_dense(const StepA
   const double *__restrict__ src = static_cast<const double *>(a.src);
   double *__restrict__ dst = static_cast<double *>(a.dst);
   const int64_t S = a.g.S;
-  const double Rs = a.Rfield ? a.Rscale * __ldg(a.Rfield + site) : 0.0;
+  const double Rs = SRC == kSrcConst ? 0.0 : (SRC == kSrcScaled ? a.Rscale * __ldg(a.Rfield + site) : __ldg(a.Rfield + site));
   double f[Q];
   const uint64_t row_out = row_links_out<D>(a.g, x);
   const uint64_t x_out = side1 > 0 ? face_links<D>(0, 1) : (side1 < 0 ? face_links<D>(0, -1) : 0ull);
@@ -291,8 +295,8 @@ __global__ void __launch_bounds__(LHE_STEP_THREADS) k_step_box_dense(const StepA
     f[k] = __ldg(row_unknown ? bdata + k * S + site : (x_unknown ? xrow + jx : src + k * S + o));
   }
   const double sum = fixed_moment_sum<Q, 0>(f);
-  const double psi = MODE == kModeS2 ? fma(2.0, sum, a.Rfield ? a.dt * Rs : a.dtR)
-                                     : fma(a.sig, sum, a.Rfield ? a.rho_dt * Rs : a.rho_dtR);
+  const double psi = MODE == kModeS2 ? fma(2.0, sum, SRC != kSrcConst ? a.dt * Rs : a.dtR)
+                                     : fma(a.sig, sum, SRC != kSrcConst ? a.rho_dt * Rs : a.rho_dtR);
   pdl_trigger();
 #pragma unroll
   for (int k = 0; k < Q; ++k) {
@@ -306,8 +310,10 @@ static cudaError_t step_box_dense_d(const StepArgs &a, const double *bdata, cuda
   const int threads = LHE_STEP_THREADS;
   const unsigned blocks = (unsigned)((a.nwork + threads - 1) / threads);
   const bool pdl = a.pdl != 0;
-  if (a.s == 2.0) return launch_kernel(k_step_box_dense<D, kModeS2>, blocks, threads, 0, st, pdl, a, bdata);
-  return launch_kernel(k_step_box_dense<D, kModeGeneral>, blocks, threads, 0, st, pdl, a, bdata);
+  auto kernel = !a.Rfield          ? (a.s == 2.0 ? k_step_box_dense<D, kModeS2, kSrcConst> : k_step_box_dense<D, kModeGeneral, kSrcConst>)
+                : a.Rscale == 1.0 ? (a.s == 2.0 ? k_step_box_dense<D, kModeS2, kSrcField> : k_step_box_dense<D, kModeGeneral, kSrcField>)
+                                  : (a.s == 2.0 ? k_step_box_dense<D, kModeS2, kSrcScaled> : k_step_box_dense<D, kModeGeneral, kSrcScaled>);
+  return launch_kernel(kernel, blocks, threads, 0, st, pdl, a, bdata);
 }
 
 cudaError_t launch_step_box_dense(int d, const StepArgs &a, const double *bdata, cudaStream_t st) {
