@@ -48,22 +48,21 @@ __device__ __forceinline__ void bnode_prepare(const BoundaryArgs &a, const int (
 
 // The part of unknown population k that depends on the boundary data only: the population itself
 // (full-way) or B_k of f_k = B_k - f*_kbar(x) (half-way).
-// table: a.table, or a copy of it.
-template <int D, int KIND>
-__device__ __forceinline__ double bnode_data(const BoundaryArgs &a, const double *table, const BNode<D> &nd, int k) {
+// coef(i): entry i of a.table, or of a copy of it.
+template <int D, int KIND, class Coef>
+__device__ __forceinline__ double bnode_data(const BoundaryArgs &a, Coef coef, const BNode<D> &nd, int k) {
   constexpr int Q = Lattice<D>::Q;
   const int M = a.nmodes;
-  const double *coef = table;                         // [m][k][2]
-  const double *kconst = table + 2 * a.nmodes * Q;    // [k][2]
+  const int kconst = 2 * (a.nmodes * Q + k);  // [m][k][2], then [k][2]
   if (KIND == 1) {
-    double acc = nd.H - kconst[2 * k];
-    for (int m = 0; m < M; ++m) acc = fma(-coef[2 * (m * Q + k)], nd.cs[m], acc);
+    double acc = nd.H - coef(kconst);
+    for (int m = 0; m < M; ++m) acc = fma(-coef(2 * (m * Q + k)), nd.cs[m], acc);
     return a.omega[k] * acc;
   }
-  double acc = fma(kconst[2 * k], nd.lin0, kconst[2 * k + 1]);
+  double acc = fma(coef(kconst), nd.lin0, coef(kconst + 1));
   for (int m = 0; m < M; ++m) {
-    acc = fma(coef[2 * (m * Q + k)], nd.sn[m], acc);
-    acc = fma(coef[2 * (m * Q + k) + 1], nd.cs[m], acc);
+    acc = fma(coef(2 * (m * Q + k)), nd.sn[m], acc);
+    acc = fma(coef(2 * (m * Q + k) + 1), nd.cs[m], acc);
   }
   return acc;
 }
@@ -80,8 +79,8 @@ __device__ __forceinline__ double bnode_fkb(const BoundaryArgs &a, int k, int32_
 
 // Pre-collision population k at `site` whose source lies outside the box.
 template <int D, int KIND, bool DEV>
-__device__ __forceinline__ double bnode_unknown(const BoundaryArgs &a, const double *table, const BNode<D> &nd, int k, int32_t site) {
-  const double acc = bnode_data<D, KIND>(a, table, nd, k);
+__device__ __forceinline__ double bnode_unknown(const BoundaryArgs &a, const BNode<D> &nd, int k, int32_t site) {
+  const double acc = bnode_data<D, KIND>(a, [&](int i) { return __ldg(a.table + i); }, nd, k);
   return KIND == 1 ? acc : acc - bnode_fkb<D, DEV>(a, k, site);
 }
 

@@ -33,11 +33,13 @@ template <int D, int KIND, bool DEV, bool EARLY>
 __global__ void __launch_bounds__(128) k_boundary(const BoundaryArgs a) {
   constexpr Lattice<D> L{};
   constexpr int Q = Lattice<D>::Q;
-  // the family's coefficients in shared memory: an unknown link's loads are behind a branch and follow one another
+  // FP32 deviations: the family's coefficients in shared memory, since an unknown link's loads are behind a branch and
+  // follow one another. FP64 boxes (LHE_FLAG_NODE_BOUNDARY) read them through L1 in CTAs of 128 threads: 33^3 full-way
+  // 50 us a step with the copy and smaller CTAs, now 33 (37 before them), 1200^2 97, now 85 (88)
   extern __shared__ double table[];
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   pdl_wait();
-  if (a.rec == nullptr) {
+  if (DEV && a.rec == nullptr) {
     for (int i = threadIdx.x; i < 2 * (a.nmodes + 1) * Q; i += blockDim.x) table[i] = __ldg(a.table + i);
     __syncthreads();
   }
@@ -58,6 +60,7 @@ __global__ void __launch_bounds__(128) k_boundary(const BoundaryArgs a) {
       }
     }
   }
+  const auto coef = [&](int i) { return DEV ? table[i] : __ldg(a.table + i); };
   BNode<D> nd;
   const bool jets = a.rec != nullptr;  // data from jet records (else from the exact-solution family)
   const double *__restrict__ rec = jets ? a.rec + a.roff[t] : nullptr;
@@ -102,7 +105,7 @@ __global__ void __launch_bounds__(128) k_boundary(const BoundaryArgs a) {
       // (one rounding for a record's scale and the half-way difference, as in k_bdata_step)
       const double less = KIND == 1 ? 0.0 : value(L.opp[k], site);
       if (jets) v[k] = KIND == 1 ? a.rec_scale * __ldg(rec + ju++) : fma(a.rec_scale, __ldg(rec + ju++), -less);
-      else v[k] = KIND == 1 ? bnode_data<D, KIND>(a, table, nd, k) : bnode_data<D, KIND>(a, table, nd, k) - less;
+      else v[k] = KIND == 1 ? bnode_data<D, KIND>(a, coef, nd, k) : bnode_data<D, KIND>(a, coef, nd, k) - less;
     }
   }
   if constexpr (EARLY) {
@@ -118,7 +121,7 @@ __global__ void __launch_bounds__(128) k_boundary(const BoundaryArgs a) {
         continue;
       }
       if (jets) v[k] = KIND == 1 ? a.rec_scale * v[k] : fma(a.rec_scale, v[k], -there);
-      else v[k] = KIND == 1 ? bnode_data<D, KIND>(a, table, nd, k) : bnode_data<D, KIND>(a, table, nd, k) - there;
+      else v[k] = KIND == 1 ? bnode_data<D, KIND>(a, coef, nd, k) : bnode_data<D, KIND>(a, coef, nd, k) - there;
     }
   }
   // collision, as in the bulk: phi = sum_k f_k, f*_k = (1 - s) f_k + omega_k (s phi + dt R)
@@ -456,12 +459,12 @@ cudaError_t launch_adjoint_boundary(int d, int kind, bool dev, const BoundaryArg
 template <int D>
 static cudaError_t boundary_d(int kind, bool dev, const BoundaryArgs &a, cudaStream_t st) {
   if (a.nsites <= 0) return cudaSuccess;
-  const int threads = boundary_threads(a.nsites);
+  const int threads = dev ? boundary_threads(a.nsites) : 128;  // (k_boundary)
   const unsigned blocks = (unsigned)((a.nsites + threads - 1) / threads);
   auto kernel = !dev ? (kind == 1 ? k_boundary<D, 1, false, false> : k_boundary<D, 2, false, false>)
                 : a.nsites <= kEarlyNodes ? (kind == 1 ? k_boundary<D, 1, true, true> : k_boundary<D, 2, true, true>)
                                           : (kind == 1 ? k_boundary<D, 1, true, false> : k_boundary<D, 2, true, false>);
-  const size_t smem = a.rec ? 0 : sizeof(double) * 2 * (size_t)(a.nmodes + 1) * Lattice<D>::Q;
+  const size_t smem = a.rec || !dev ? 0 : sizeof(double) * 2 * (size_t)(a.nmodes + 1) * Lattice<D>::Q;
   return launch_kernel(kernel, blocks, threads, smem, st, a.pdl != 0, a);
 }
 

@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(128) k_xface_data(const BoundaryArgs b, double
   bnode_prepare<D, KIND>(b, x, nd);
 #pragma unroll
   for (int k = 0; k < Q; ++k)
-    if (L.e[k][0] == sgn) xb[t * J + xface_link<D>(k, sgn)] = bnode_unknown<D, KIND, false>(b, b.table, nd, k, site);
+    if (L.e[k][0] == sgn) xb[t * J + xface_link<D>(k, sgn)] = bnode_unknown<D, KIND, false>(b, nd, k, site);
 }
 
 // Forward step of a Dirichlet box (FP64; constant R or a per-site source), whole x-rows through the interior: the interior
