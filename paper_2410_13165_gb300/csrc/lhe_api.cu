@@ -604,7 +604,7 @@ lhe_status lhe_lbm_create(const lhe_lbm_params *p, lhe_lbm **out) {
       *l->tma_err_host = 0;
       e = cudaHostGetDevicePointer((void **)&l->tma.err, l->tma_err_host, 0);
       if (e != cudaSuccess) return bail(cuda_fail(l, e, "cudaHostGetDevicePointer(pipeline flag)"));
-      e = prepare_dev3_tma(l->tma);
+      e = prepare_dev3_tma();
       if (e != cudaSuccess) return bail(cuda_fail(l, e, "shared-memory size of the staged step"));
       const bool hook = (p->flags & LHE_FLAG_TEST_EXPIRE_WAIT) != 0;
       l->staged[0] = hook || staged_pays(l->tma, false);

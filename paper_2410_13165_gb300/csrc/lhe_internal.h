@@ -269,7 +269,7 @@ cudaError_t launch_df_to_double(const float2 *src, double *dst, int64_t n, cudaS
 cudaError_t launch_scale_fp64(double *p, int64_t n, double factor, cudaStream_t st);
 bool plan_dev3_tma(const Geom &g, int sms, DevTmaPlan &p);
 bool staged_pays(const DevTmaPlan &p, bool adjoint);
-cudaError_t prepare_dev3_tma(const DevTmaPlan &p);
+cudaError_t prepare_dev3_tma();
 cudaError_t launch_step_dev3_tma(bool adjoint, const StepArgs &a, const DevTmaPlan &p, cudaStream_t st);
 bool plan_multi(const Geom &g, bool dev, int sms, MultiPlan &p);
 MultiPlan shorter_multi(const Geom &g, bool dev, const MultiPlan &p, int H);  // the same tiles, 2 <= H <= p.H

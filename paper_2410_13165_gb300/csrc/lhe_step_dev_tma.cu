@@ -373,8 +373,9 @@ bool staged_pays(const DevTmaPlan &p, bool adjoint) {
   return p.R * p.nx == kTileNodes && ((p.nx == 128 && S >= (7 << 18)) || (p.nx == 256 && S >= (1 << 20)));
 }
 
-cudaError_t prepare_dev3_tma(const DevTmaPlan &p) {
-  const int bytes = p.NS * (int)p.stage_bytes;
+// The limit is the kernels', not a plan's: it stays the same for the handles created before and after.
+cudaError_t prepare_dev3_tma() {
+  const int bytes = (int)(LHE_TMA_SMEM_BUDGET);
   cudaError_t e;
 #define LHE_SMEM(kernel) \
   if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes))) return e;
