@@ -1424,6 +1424,9 @@ lhe_status lhe_lbm_adjoint_seed(lhe_lbm *l, const double *seed) {
     }
     LHE_CK(l, cudaMalloc(&l->gR, sizeof(double) * S));
   }
+  // the buffer of dL/d(grad phi0) of a gradient that the library formed, here and not in lhe_lbm_adjoint_grads, which
+  // can be captured into a graph like the steps
+  if (l->grad_was_fd && !l->fdgrad) LHE_CK(l, cudaMalloc(&l->fdgrad, sizeof(double) * S * l->p.d));
   LHE_CK(l, launch_adjoint_seed(l->p.d, dev, l->g, l->omega, seed, l->adj[0], l->adjW[0], l->gR, l->stream));
   l->acur = 0;
   l->adj_ready = true;
