@@ -376,8 +376,11 @@ const void *multi_kernel(int d, bool dev, bool adjoint, bool s2) {
 //   FP64 D2Q9 16^2 1.90 / 1.31, 64^2 2.14 / 1.39, 128^2 2.22 / 1.66, 200^2 3.08 / 2.46, 256^2 3.66 / 3.21, 270 x 260 3.68 / 3.52 with the
 //     adjoint 3.52 / 3.69 (not taken), 500 x 333 5.9 / 7.1 (32 x 8, H = 2; not taken); D1Q3 64 1.92 / 0.74, 30000 2.01 / 1.03,
 //     10^6 16.4 / 18.4 (not taken)
-//   32 bits D2Q9 16^2 1.90 / 0.60, 64^2 1.90 / 0.70, 128^2 1.90 / 0.84, 256^2 2.05 / 1.42, 320^2 2.29 / 2.23, 500 x 333 3.33 / 2.97, 1000^2
-//     11.7 / 12.1 (not taken), 1250^2 23.3 / 19.8, 2048^2 58.7 / 50.5; D1Q3 4096 1.89 / 0.47, 10^5 1.96 / 1.13, 2 10^6 17.1 / 8.3;
+//   32 bits D2Q9 16^2 1.90 / 0.60, 64^2 1.90 / 0.70, 128^2 1.90 / 0.84, 256^2 2.05 / 1.42, 320^2 2.29 / 2.23, 500 x 333 3.33 / 2.97, 430^2 (756
+//     tiles of 32 x 8, one wave is 760) 3.38 / 3.07, 440^2 (770) 3.37 / 3.58, 5000 x 33 (785) 3.38 / 3.66, 560^2 4.53 / 4.82, 700^2 6.05 / 7.01,
+//     1000^2 12.1 / 14.1 (none of these taken), 1250^2 23.3 / 19.8, 2048^2 58.7 / 50.5; with tiles of 32 x 16 that stick out of 2 M to
+//     3 M nodes by 60 % (100000 x 20) 29.9 / 36.3, 33 % (x 24) 35.5 / 38.9, 14 % (x 28) 40.7 / 41.3 (not taken), 7 % (x 30) 43.4 / 41.9;
+//     D1Q3 4096 1.89 / 0.47, 10^5 1.96 / 1.13, 2 10^6 17.1 / 8.3;
 //     D3Q19 8^3 1.93 / 1.14, 16^3 1.95 / 1.44, 24^3 1.94 / 1.75, 28^3 2.18 / 2.13 (not taken); FP64 D3Q19 16^3 2.89 / 2.82, 20^3 2.94 / 3.05 (not taken)
 bool plan_multi(const Geom &g, bool dev, int sms, MultiPlan &best) {
   best = MultiPlan{};
@@ -408,10 +411,12 @@ bool plan_multi(const Geom &g, bool dev, int sms, MultiPlan &best) {
     if (dev && S <= 14000) search(S <= 4200 ? 3 : 2, 1, 24, 24, 24, 2048);
   } else if (share <= (dev ? 480 : 440)) {
     search(dev ? (share <= 160 ? 6 : 4) : (share <= 48 ? 4 : (share <= 160 ? 3 : 2)), 4, 64, 64, 1, kMultiThreads);
-  } else if (dev && S <= 180000 && fits(32, 8, 1, 3)) {
+  } else if (dev && S <= 200000 && fits(32, 8, 1, 3)) {
     best = make_multi(g, dev, 32, 8, 1, 3, 192);
+    if (best.grid > 5 * sms) best = MultiPlan{};  // more than one wave (40 KB of shared memory a CTA)
   } else if (dev && S >= 1500000 && fits(32, 16, 1, 2)) {
     best = make_multi(g, dev, 32, 16, 1, 2, 320);
+    if ((int64_t)best.grid * best.own > S + S / 10) best = MultiPlan{};  // tiles that stick out compute for nothing
   }
   return best.H > 1;
 }
