@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(LHE_STEP_THREADS) k_step_box_dense(const StepA
   const double *__restrict__ src = static_cast<const double *>(a.src);
   double *__restrict__ dst = static_cast<double *>(a.dst);
   const int64_t S = a.g.S;
-  const double Rs = SRC == kSrcConst ? 0.0 : (SRC == kSrcScaled ? a.Rscale * __ldg(a.Rfield + site) : __ldg(a.Rfield + site));
+  const double Rs = SRC == kSrcConst ? 0.0 : (SRC == kSrcField ? __ldg(a.Rfield + site) : (a.Rfield ? a.Rscale * __ldg(a.Rfield + site) : 0.0));
   double f[Q];
   const uint64_t row_out = row_links_out<D>(a.g, x);
   const uint64_t x_out = side1 > 0 ? face_links<D>(0, 1) : (side1 < 0 ? face_links<D>(0, -1) : 0ull);
@@ -295,8 +295,8 @@ __global__ void __launch_bounds__(LHE_STEP_THREADS) k_step_box_dense(const StepA
     f[k] = __ldg(row_unknown ? bdata + k * S + site : (x_unknown ? xrow + jx : src + k * S + o));
   }
   const double sum = fixed_moment_sum<Q, 0>(f);
-  const double psi = MODE == kModeS2 ? fma(2.0, sum, SRC != kSrcConst ? a.dt * Rs : a.dtR)
-                                     : fma(a.sig, sum, SRC != kSrcConst ? a.rho_dt * Rs : a.rho_dtR);
+  const double psi = MODE == kModeS2 ? fma(2.0, sum, SRC != kSrcConst && (SRC == kSrcField || a.Rfield) ? a.dt * Rs : a.dtR)
+                                     : fma(a.sig, sum, SRC != kSrcConst && (SRC == kSrcField || a.Rfield) ? a.rho_dt * Rs : a.rho_dtR);
   pdl_trigger();
 #pragma unroll
   for (int k = 0; k < Q; ++k) {
