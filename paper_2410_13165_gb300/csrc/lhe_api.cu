@@ -894,6 +894,7 @@ static BoundaryArgs boundary_args(const lhe_lbm *l) {
     b.kbar[k] = l->kbar[k];
   }
   b.nrow_ent = l->nrow_ent;
+  b.sms = l->sms;
   b.s = l->s;
   b.oms = 1.0 - l->s;
   b.R = l->R;

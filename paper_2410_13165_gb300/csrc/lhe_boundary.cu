@@ -23,6 +23,7 @@
 // grouped by face signature so that a warp shares one set of unknown populations. The per-node
 // evaluation (lhe_bnode.cuh) is shared with the FP64 interior kernel of Dirichlet boxes, which treats
 // the nodes of the two x_1 faces (whose other coordinates are interior) in the lanes of their rows.
+#include <algorithm>
 #include <type_traits>
 
 #include "lhe_bnode.cuh"
@@ -67,7 +68,7 @@ __global__ void __launch_bounds__(128) k_boundary(const BoundaryArgs a) {
   // EARLY: every load first, so that they are in flight together: a population is read at its pull source, or for an
   // unknown link where the half-way scheme's f*_kbar lies, at the node itself. Else the loads are behind the branch on `inside` and
   // follow one another, Q trips to L2 a node, which is what few nodes wait for; many nodes hide them, and are held back by the
-  // registers and the unknown links' extra loads instead. FP32 deviations, us per step, late / early, full-way and half-way:
+  // registers and the unknown links' extra loads instead (node_launch). FP32 deviations, us per step, late / early, full-way and half-way:
   // D3Q19 16^3 18.9 / 16.4 and 24.6 / 16.0, 48^3 (13,000 nodes) 20.9 / 18.4 and 27.0 / 18.1, D4Q33 16^4 (27,000) 36 / 32 and 47 / 32,
   // 24^4 (97,500) 99 / 107 and 117 / 101, 32^4 (239,000) 241 / 326 and 275 / 312.
   using T = typename std::conditional<DEV, float, double>::type;
@@ -428,21 +429,45 @@ __global__ void __launch_bounds__(128) k_adj_boundary(const BoundaryArgs a) {
   }
 }
 
-constexpr int64_t kEarlyNodes = 40000;  // boundary nodes up to which the kernels issue every load first (k_boundary)
+// FP32 deviations: boundary nodes up to which the kernels issue every load first (EARLY, k_boundary): one wave of CTAs of 64
+// threads, as many an SM as the registers allow (k_boundary 80, 168, 254 and 255 for D = 2 .. 5, k_adj_boundary 72, 87, 142 and 216).
+template <int D>
+static int64_t early_nodes(int sms, bool adjoint) {
+  constexpr int ctas[2][6] = {{0, 32, 12, 6, 4, 4}, {0, 32, 14, 11, 7, 4}};
+  return (int64_t)sms * ctas[adjoint][D] * 64;
+}
 
 // Threads per CTA of the boundary-node kernels: a node is ~150 FP64 operations behind several dependent loads, so few
 // nodes are spread over as many SMs as there are (128 threads: D3Q19 32^3, 5768 nodes, on 46 of 152 SMs).
-static int boundary_threads(int64_t nodes) { return nodes <= 152 * 4 * 32 ? 32 : (nodes <= 152 * 8 * 64 ? 64 : 128); }
+static int boundary_threads(int64_t nodes, int sms) {
+  return nodes <= (int64_t)sms * 4 * 32 ? 32 : (nodes <= (int64_t)sms * 8 * 64 ? 64 : 128);
+}
+
+// How the kernels of one box are launched. FP32 deviations, us per step before there was an early form / early up to 40,000 nodes,
+// more than a wave in D4Q33, and beside the rows' last wave / now (lhe_step_dev.cu), full-way and its adjoint: D4Q33 18^4 (39,440 nodes)
+// 50 / 63 / 45 and 41 / 33 / 30, 19^4 56 / 62 / 49 and 41 / 47 / 32, 22^4 (74,256) 76 / 78 / 73 and 56 / 60 / 52, 24^4 (97,520) 109 / 106 / 106 and 79 / 76 / 76;
+// D3Q19 90^3 (47,528) 55 / 49 / 49 and 45 / 40 / 40.
+struct NodeLaunch {
+  bool early;
+  int threads;
+};
+
+template <int D>
+static NodeLaunch node_launch(bool dev, bool adjoint, const BoundaryArgs &a) {
+  const int threads = boundary_threads(a.nsites, a.sms);
+  if (!dev) return {false, adjoint ? threads : 128};  // (k_boundary)
+  return a.nsites <= early_nodes<D>(a.sms, adjoint) ? NodeLaunch{true, std::min(threads, 64)} : NodeLaunch{false, threads};
+}
 
 template <int D>
 static cudaError_t adj_boundary_d(int kind, bool dev, const BoundaryArgs &a, cudaStream_t st) {
   if (a.nsites <= 0) return cudaSuccess;
-  const int threads = boundary_threads(a.nsites);
-  const unsigned blocks = (unsigned)((a.nsites + threads - 1) / threads);
+  const NodeLaunch n = node_launch<D>(dev, true, a);
+  const unsigned blocks = (unsigned)((a.nsites + n.threads - 1) / n.threads);
   auto kernel = !dev ? (kind == 1 ? k_adj_boundary<D, 1, false, false> : k_adj_boundary<D, 2, false, false>)
-                : a.nsites <= kEarlyNodes ? (kind == 1 ? k_adj_boundary<D, 1, true, true> : k_adj_boundary<D, 2, true, true>)
+                : n.early              ? (kind == 1 ? k_adj_boundary<D, 1, true, true> : k_adj_boundary<D, 2, true, true>)
                                           : (kind == 1 ? k_adj_boundary<D, 1, true, false> : k_adj_boundary<D, 2, true, false>);
-  return launch_kernel(kernel, blocks, threads, 0, st, a.pdl != 0, a);
+  return launch_kernel(kernel, blocks, n.threads, 0, st, a.pdl != 0, a);
 }
 
 cudaError_t launch_adjoint_boundary(int d, int kind, bool dev, const BoundaryArgs &a, cudaStream_t st) {
@@ -459,13 +484,13 @@ cudaError_t launch_adjoint_boundary(int d, int kind, bool dev, const BoundaryArg
 template <int D>
 static cudaError_t boundary_d(int kind, bool dev, const BoundaryArgs &a, cudaStream_t st) {
   if (a.nsites <= 0) return cudaSuccess;
-  const int threads = dev ? boundary_threads(a.nsites) : 128;  // (k_boundary)
-  const unsigned blocks = (unsigned)((a.nsites + threads - 1) / threads);
+  const NodeLaunch n = node_launch<D>(dev, false, a);
+  const unsigned blocks = (unsigned)((a.nsites + n.threads - 1) / n.threads);
   auto kernel = !dev ? (kind == 1 ? k_boundary<D, 1, false, false> : k_boundary<D, 2, false, false>)
-                : a.nsites <= kEarlyNodes ? (kind == 1 ? k_boundary<D, 1, true, true> : k_boundary<D, 2, true, true>)
+                : n.early              ? (kind == 1 ? k_boundary<D, 1, true, true> : k_boundary<D, 2, true, true>)
                                           : (kind == 1 ? k_boundary<D, 1, true, false> : k_boundary<D, 2, true, false>);
   const size_t smem = a.rec || !dev ? 0 : sizeof(double) * 2 * (size_t)(a.nmodes + 1) * Lattice<D>::Q;
-  return launch_kernel(kernel, blocks, threads, smem, st, a.pdl != 0, a);
+  return launch_kernel(kernel, blocks, n.threads, smem, st, a.pdl != 0, a);
 }
 
 cudaError_t launch_boundary(int d, int kind, bool dev, const BoundaryArgs &a, cudaStream_t st) {

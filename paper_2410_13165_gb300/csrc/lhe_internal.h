@@ -173,6 +173,7 @@ struct BoundaryArgs {
   // dense array (k S + x) and half-way partners (kbar S + x) follow from the entry's (k, x)
   int64_t nrow_ent;
   int8_t kbar[kMaxQ];      // the link opposite to k
+  int32_t sms = 0;         // multiprocessors of the device
   int32_t pdl = 0;         // launch with programmatic stream serialization (the kernel calls pdl_wait)
 };
 

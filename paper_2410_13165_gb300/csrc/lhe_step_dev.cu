@@ -32,7 +32,10 @@ namespace lhe {
 template <int D>
 constexpr int dev_min_blocks() { return D == 4 ? 5 : (D == 5 ? 3 : 1); }
 
-template <int D, bool ADJ, bool INTERIOR, bool S2>
+// When the next kernel of the chain may be scheduled (lhe_device.cuh).
+constexpr int kTrigStores = 0, kTrigEnd = 2;
+
+template <int D, bool ADJ, bool INTERIOR, bool S2, int TRIG>
 __global__ void __launch_bounds__(LHE_STEP_THREADS, dev_min_blocks<D>()) k_step_dev(const StepArgs a) {
   constexpr Lattice<D> L{};
   constexpr int Q = Lattice<D>::Q;
@@ -73,7 +76,7 @@ __global__ void __launch_bounds__(LHE_STEP_THREADS, dev_min_blocks<D>()) k_step_
   if (ADJ && a.gR) a.gR[site] = fma(a.dt, df_value(pn), a.gR[site]);
   float dtR = 0.0f;
   if (field) dtR = (float)(a.dt * __ldg(a.Rfield + site));
-  pdl_trigger();
+  if constexpr (TRIG == kTrigStores) pdl_trigger();
 #pragma unroll
   for (int k = 0; k < Q; ++k) {
     const float r = fmaf(a.omega_f[k], dl[k] - Delta, gk[k]);  // pre-collision deviation g_k
@@ -83,13 +86,26 @@ __global__ void __launch_bounds__(LHE_STEP_THREADS, dev_min_blocks<D>()) k_step_
   }
 }
 
+template <int D, bool ADJ, bool INTERIOR, int TRIG>
+static cudaError_t launch_step_dev_trig(const StepArgs &a, cudaStream_t st) {
+  const int threads = LHE_STEP_THREADS;
+  const unsigned blocks = (unsigned)((a.nwork + threads - 1) / threads);
+  if (a.s == 2.0) return launch_kernel(k_step_dev<D, ADJ, INTERIOR, true, TRIG>, blocks, threads, 0, st, a.pdl != 0, a);
+  return launch_kernel(k_step_dev<D, ADJ, INTERIOR, false, TRIG>, blocks, threads, 0, st, a.pdl != 0, a);
+}
+
 template <int D, bool ADJ, bool INTERIOR>
 static cudaError_t launch_step_dev_t(const StepArgs &a, cudaStream_t st) {
   if (a.nwork <= 0) return cudaSuccess;
-  const int threads = LHE_STEP_THREADS;
-  const unsigned blocks = (unsigned)((a.nwork + threads - 1) / threads);
-  if (a.s == 2.0) return launch_kernel(k_step_dev<D, ADJ, INTERIOR, true>, blocks, threads, 0, st, a.pdl != 0, a);
-  return launch_kernel(k_step_dev<D, ADJ, INTERIOR, false>, blocks, threads, 0, st, a.pdl != 0, a);
+  if constexpr (INTERIOR) {
+    // The rows of a box: where its boundary kernel, which comes next, has CTAs of 64 threads and more on every SM, they took places
+    // from the rows' last wave. us per step before the stores / at the end, full-way: D4Q33 14^4 31.6 / 29.4, 19^4 56 / 49, 22^4 78 / 73;
+    // smaller boundaries the other way, adjoint D2Q9 300^2 7.5 / 8.1, D4Q33 12^4 28.7 / 29.3.
+    int64_t inner = 1;
+    for (int i = 0; i < D; ++i) inner *= a.g.n[i] - 2;
+    if (a.g.S - inner > (int64_t)a.sms * 4 * 32) return launch_step_dev_trig<D, ADJ, INTERIOR, kTrigEnd>(a, st);
+  }
+  return launch_step_dev_trig<D, ADJ, INTERIOR, kTrigStores>(a, st);
 }
 
 template <int D>
