@@ -406,7 +406,7 @@ __global__ void __launch_bounds__(128) k_adj_boundary(const BoundaryArgs a) {
     }
   }
   if (DEV) {
-    const double M = fixed_moment_sum<Q, 0>(mu);
+    const double M = fixed_moment_sum<Q, 0, false>(mu);
     const double psi = a.s * M;
     float *edst = static_cast<float *>(a.dst);
 #pragma unroll
@@ -419,11 +419,11 @@ __global__ void __launch_bounds__(128) k_adj_boundary(const BoundaryArgs a) {
   }
   double *__restrict__ dst = static_cast<double *>(a.dst);
   if (a.s == 2.0) {
-    const double psi = fixed_moment_sum<Q, 1>(mu);  // 2 sum_j mu_j
+    const double psi = fixed_moment_sum<Q, 1, false>(mu);  // 2 sum_j mu_j
 #pragma unroll
     for (int k = 0; k < Q; ++k) dst[k * S + site] = fma(a.omega[k], psi, -mu[k]);
   } else {
-    const double psi = a.s * fixed_moment_sum<Q, 0>(mu);
+    const double psi = a.s * fixed_moment_sum<Q, 0, false>(mu);
 #pragma unroll
     for (int k = 0; k < Q; ++k) dst[k * S + site] = fma(a.omega[k], psi, a.oms * mu[k]);
   }

@@ -155,7 +155,9 @@ __device__ __forceinline__ double fixed_value(long long acc, unsigned emf) {
   return __longlong_as_double((long long)(sbit | ((unsigned long long)ex << 52) | (mant & 0xFFFFFFFFFFFFFull)));
 }
 
-template <int Q, int P2, class Get>
+// ZEROS: return at once for a sum of zeros (the latency of small grids' boundary kernels grows by it: adjoint of D2Q9 300^2 boxes
+// in 32 bits 7.6 -> 8.2 us a step, so that k_adj_boundary does without).
+template <int Q, int P2, bool ZEROS = true, class Get>
 __device__ __forceinline__ double fixed_moment_sum_impl(Get f) {
   constexpr int G = 10 - ceil_log2(Q);
   static_assert(G >= 3, "too many terms for a 64-bit accumulator");
@@ -168,10 +170,12 @@ __device__ __forceinline__ double fixed_moment_sum_impl(Get f) {
       // Every term below 2^-954. Zeros take no FP64 operation: summed as the tiny terms are, regions of them were stepped 1.4 to
       // 1.7 times slower than others (D3Q19 256^3: 1.26 ms, now 0.73; 1000^2: 40 us, now 23). Tiny terms in fixed point too,
       // here or in a function apart, made every step of small grids 1 to 3 % slower.
-      unsigned any = 0u;
+      if constexpr (ZEROS) {
+        unsigned any = 0u;
 #pragma unroll
-      for (int k = 0; k < Q; ++k) any |= ((unsigned)__double2hiint(f(k)) & 0x7FFFFFFFu) | (unsigned)__double2loint(f(k));
-      if (any == 0u) return 0.0;
+        for (int k = 0; k < Q; ++k) any |= ((unsigned)__double2hiint(f(k)) & 0x7FFFFFFFu) | (unsigned)__double2loint(f(k));
+        if (any == 0u) return 0.0;
+      }
       double s = 0.0;
 #pragma unroll
       for (int k = 0; k < Q; ++k) s += f(k);
@@ -186,9 +190,9 @@ __device__ __forceinline__ double fixed_moment_sum_impl(Get f) {
   return fixed_value<G, P2>(acc, emf);
 }
 
-template <int Q, int P2>
+template <int Q, int P2, bool ZEROS = true>
 __device__ __forceinline__ double fixed_moment_sum(const double (&f)[Q]) {
-  return fixed_moment_sum_impl<Q, P2>([&](int k) { return f[k]; });
+  return fixed_moment_sum_impl<Q, P2, ZEROS>([&](int k) { return f[k]; });
 }
 
 // Moment sum of the boundary nodes of FP32-deviation boxes in d = 4, 5: the first NFX terms in fixed point, the rest
