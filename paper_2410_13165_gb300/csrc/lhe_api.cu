@@ -1505,9 +1505,12 @@ lhe_status lhe_lbm_stability_map(const lhe_lbm_params *p, const double *sigma, i
   int32_t e[kMaxQ * kMaxD];
   const int Q = lattice_vectors(d, e);
   const int npairs = d * (d - 1) / 2;
-  // one device buffer: the radii (as the bits of doubles, from 0) and the weights
-  std::vector<double> buf((size_t)npoints * (Q + 1), 0.0);
-  double *om = buf.data() + npoints;
+  // one device buffer: the radii (as the bits of doubles, from 0), the number of matrices left to the QR route, the weights,
+  // and the list of those matrices (a few as a rule; of more, all matrices take that route)
+  std::vector<double> buf((size_t)npoints * (Q + 1) + 1, 0.0);
+  double *om = buf.data() + npoints + 1;
+  bool large = false;
+  const int64_t room = std::min<int64_t>(npoints * nper, 1024);
   for (int64_t q = 0; q < npoints; ++q) {
     double sig[kMaxD], m4[10] = {};
     for (int i = 0; i < d; ++i) {
@@ -1518,17 +1521,33 @@ lhe_status lhe_lbm_stability_map(const lhe_lbm_params *p, const double *sigma, i
     weights(d, e, Q, sig, m4, &om[(size_t)q * Q]);
     double mn = om[(size_t)q * Q];
     for (int k = 1; k < Q; ++k) mn = std::fmin(mn, om[(size_t)q * Q + k]);
+    for (int k = 0; k < Q; ++k) large = large || !(std::fabs(om[(size_t)q * Q + k]) <= 1e6);
     omega_min[q] = mn;
   }
   cudaStream_t st = static_cast<cudaStream_t>(p->stream);
   double *dev = nullptr;
-  cudaError_t e1 = cudaMalloc(&dev, sizeof(double) * buf.size());
+  cudaError_t e1 = cudaMalloc(&dev, sizeof(double) * (buf.size() + (size_t)room));
+  auto *rho_bits = reinterpret_cast<unsigned long long *>(dev);
+  StabilityRest rest{rho_bits + npoints, reinterpret_cast<long long *>(dev + buf.size()), room};
+  const double *om_dev = dev + npoints + 1;
+  auto fetch = [&]() {  // the radii and the number of matrices left over
+    cudaError_t e2 = cudaMemcpyAsync(buf.data(), dev, sizeof(double) * ((size_t)npoints + 1), cudaMemcpyDeviceToHost, st);
+    return e2 == cudaSuccess ? cudaStreamSynchronize(st) : e2;
+  };
   if (e1 == cudaSuccess) e1 = cudaMemcpyAsync(dev, buf.data(), sizeof(double) * buf.size(), cudaMemcpyHostToDevice, st);
-  if (e1 == cudaSuccess)
-    e1 = launch_stability(d, dev + npoints, npoints, nxi, 1.0 / p->tau, reinterpret_cast<unsigned long long *>(dev), st);
-  if (e1 == cudaSuccess)
-    e1 = cudaMemcpyAsync(buf.data(), dev, sizeof(double) * (size_t)npoints, cudaMemcpyDeviceToHost, st);
-  if (e1 == cudaSuccess) e1 = cudaStreamSynchronize(st);
+  unsigned long long left = 0;
+  if (large) {  // weights out of the FP32 search's range
+    rest.room = -1;
+    left = 1;
+  } else if (e1 == cudaSuccess) {
+    e1 = launch_stability(d, om_dev, npoints, nxi, 1.0 / p->tau, rho_bits, rest, st);
+    if (e1 == cudaSuccess) e1 = fetch();
+    std::memcpy(&left, &buf[(size_t)npoints], sizeof(left));
+  }
+  if (e1 == cudaSuccess && left) {
+    e1 = launch_stability_rest(d, om_dev, npoints, nxi, 1.0 / p->tau, rho_bits, rest, st);
+    if (e1 == cudaSuccess) e1 = fetch();
+  }
   cudaFree(dev);
   if (e1 != cudaSuccess) return cuda_fail(nullptr, e1, "stability map");
   std::memcpy(rho_max, buf.data(), sizeof(double) * (size_t)npoints);

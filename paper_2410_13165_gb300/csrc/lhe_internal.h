@@ -257,8 +257,16 @@ cudaError_t launch_bdata_step(int kind, bool rec, const BoundaryArgs &b, const l
                               const long long *opp, int64_t nent, const double *data, double *bdata, cudaStream_t st);
 cudaError_t launch_family_sep(int d, int kind, const BoundaryArgs &b, const long long *ent, int64_t nent, double *sep,
                               cudaStream_t st);
+// Matrices of a stability map whose roots were not accepted: their number, and the first `room` of them.
+struct StabilityRest {
+  unsigned long long *count;  // (device, 0 before the launch)
+  long long *list;
+  int64_t room;
+};
 cudaError_t launch_stability(int d, const double *omega_dev, int64_t npoints, int32_t nxi, double s,
-                             unsigned long long *rho_bits_dev, cudaStream_t st);
+                             unsigned long long *rho_bits_dev, const StabilityRest &r, cudaStream_t st);
+cudaError_t launch_stability_rest(int d, const double *omega_dev, int64_t npoints, int32_t nxi, double s,
+                                  unsigned long long *rho_bits_dev, const StabilityRest &r, cudaStream_t st);
 cudaError_t launch_init(int d, bool dev, const InitArgs &a, cudaStream_t st);
 cudaError_t launch_macro_fp64(int d, const StepArgs &a, double *phi_out, cudaStream_t st);
 cudaError_t launch_fd_grad_transpose_add(int d, const Geom &g, double dx, const double *G, double *out,

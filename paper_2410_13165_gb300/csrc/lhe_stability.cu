@@ -101,7 +101,7 @@ __device__ double spectral_radius(cd (&A)[N][N]) {
     if (++iter > 80) {
       // budget spent: a window whose subdiagonal is at rounding level is triangular for our purpose
       for (int i = lo + 1; i <= hi; ++i)
-        if (ab1(A[i][i - 1]) > 1e-10 * (ab1(A[i - 1][i - 1]) + ab1(A[i][i])))
+        if (!(ab1(A[i][i - 1]) <= 1e-10 * (ab1(A[i - 1][i - 1]) + ab1(A[i][i]))))  // (not finite: not converged)
           return __longlong_as_double(0x7FF8000000000000ll);
       for (int i = lo; i <= hi; ++i) rho = fmax(rho, ab(A[i][i]));
       hi = lo - 1;
@@ -185,8 +185,28 @@ struct StabilityArgs {
   int64_t npoints, nper;  // velocities; Fourier variables per velocity that are visited
   int32_t nxi;
   double s;
+  StabilityRest rest;
   int8_t e[33][4];
 };
+
+// Velocity and Fourier indices of matrix t.
+template <int D>
+__device__ __forceinline__ int64_t matrix_of(const StabilityArgs &a, int64_t t, int (&j)[D]) {
+  const int64_t pt = t / a.nper;
+  int64_t r = t - pt * a.nper;
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    j[i] = (int)(i == D - 1 ? r : r % a.nxi);
+    r /= a.nxi;
+  }
+  return pt;
+}
+
+// The bits of non-negative doubles order as integers; most matrices do not raise the maximum.
+__device__ __forceinline__ void raise_radius(unsigned long long *out, double rho) {
+  const unsigned long long bits = (unsigned long long)__double_as_longlong(rho);
+  if (*(volatile unsigned long long *)out < bits) atomicMax(out, bits);
+}
 
 struct cf {
   float re, im;
@@ -223,14 +243,19 @@ __device__ __forceinline__ cd rcp(cd a) {
 // FP32 iterations (the FP32 pipe runs 64 times the FP64 pipe's rate) bring the offsets to ~1e-6; then S and g
 // in FP64, with the denominator still in FP32, until a step is below 2e-9 (the step's relative error
 // is ~1e-6, so the next one would be below rounding): two as a rule. The roots are accepted if their sum and sum
-// of squares match the matrix's traces; else, and without convergence, the matrix takes the QR route.
+// of squares match the matrix's traces, to 1e-10 of its size and of its square (absolute checks, or ones that grow with
+// kappa^2, rejected velocities of order 100 and let anything pass for tau near 1); else, and without convergence, the matrix
+// is left to the QR route (k_stability_qr, a thread per matrix; within this kernel one lane of a group ran it while the others
+// waited: 24 velocities of order 100, D3Q19, 12^3 Fourier variables 134 ms, now 0.84 by the secular equation, 61 by QR).
+// Weights above 1e6 and ones that are not finite go there at once: FP32 cannot hold their products.
 // A group of G lanes holds a matrix, a lane a root (two for the 33rd pole of D = 4); G is the smallest of 8, 16
 // and 32 that holds the poles, of which there are at most nxi (nxi even) or 2 nxi. G(-xi) is the conjugate of G(xi), so half
 // of the last axis is visited. Bound by the FP64 pipe (~70 % busy: S in the last two iterations, the poles' sines). Against roots
-// refined in 80 bits (600 random D3Q19 matrices) the radius is within 6e-15, LAPACK's QR within 3e-14. 24 velocities of D3Q19, 12^3 Fourier variables: 29.2 ms by QR (one thread
-// per matrix, in local memory) -> 0.53 ms.
+// refined in 80 bits (600 random D3Q19 matrices) the radius is within 6e-15, LAPACK's QR within 3e-14. 24 velocities of D3Q19,
+// 12^3 Fourier variables: 29.2 ms by QR (one thread per matrix, in local memory) -> 0.53 ms; the whole call takes 0.04 ms more.
+// (D4Q33 in groups of 8 on at least five CTAs an SM: at 114 registers and four it took a tenth longer. 0 leaves the others alone.)
 template <int D, int G>
-__global__ void __launch_bounds__(128) k_stability(const __grid_constant__ StabilityArgs a) {
+__global__ void __launch_bounds__(128, D == 4 && G == 8 ? 5 : 0) k_stability(const __grid_constant__ StabilityArgs a) {
   constexpr int Q = 2 * D * D + 1;
   constexpr int R = (Q + G - 1) / G;  // roots per lane at most
   constexpr int kGroups = 128 / G;
@@ -246,17 +271,9 @@ __global__ void __launch_bounds__(128) k_stability(const __grid_constant__ Stabi
     const bool idle = t >= total;  // surplus groups repeat the last matrix and write nothing
     if (idle) t = total - 1;
     __syncwarp();  // the last matrix's tables are read out
-    const int64_t pt = t / a.nper;
-    const double *__restrict__ omega = a.omega + pt * Q;
     int j[D];
-    {
-      int64_t r = t - pt * a.nper;
-#pragma unroll
-      for (int i = 0; i < D; ++i) {
-        j[i] = (int)(i == D - 1 ? r : r % nxi);
-        r /= nxi;
-      }
-    }
+    const int64_t pt = matrix_of(a, t, j);
+    const double *__restrict__ omega = a.omega + pt * Q;
     // phases of the links, -e_k . xi = (pi / nxi) (nxi sum_i e_ki - 2 sum_i e_ki j_i)
     for (int k = lane; k < Q; k += G) {
       int v = 0;
@@ -297,7 +314,11 @@ __global__ void __launch_bounds__(128) k_stability(const __grid_constant__ Stabi
       P += __popc(kept);
     }
     __syncwarp();
-    for (int p = 0; p < P; ++p) trace = trace + c64[grp][p];  // kappa sum tau W
+    float size = 0.0f;  // of the matrix over 1 - s, besides its diagonal
+    for (int p = 0; p < P; ++p) {
+      trace = trace + c64[grp][p];  // kappa sum tau W
+      size += fabsf(cfl[grp][p].re) + fabsf(cfl[grp][p].im);
+    }
     if (a.s == 1.0) {  // the matrix has rank one: its only eigenvalue besides 0 is sum tau W
       if (lane == 0 && !idle) atomicMax(a.rho_bits + pt, (unsigned long long)__double_as_longlong(ab(trace)));
       continue;
@@ -434,17 +455,31 @@ __global__ void __launch_bounds__(128) k_stability(const __grid_constant__ Stabi
       top = fmax(top, __shfl_xor_sync(0xffffffffu, top, o));
     }
     s2 = s2 - trace * trace;
-    const double tol = 1e-10 * P * fmax(1.0, kappa * kappa);
-    const bool good = converged && ab1(s1) < tol && ab1(s2) < tol;
+    // (the roots' rounding grows with the matrix: large weights, or s near 1)
+    const double scale = fmax(1.0, (double)size), tol = 1e-10 * P * scale;
+    const bool good = converged && ab1(s1) < tol && ab1(s2) < tol * scale;
     if (lane == 0 && !idle) {
-      double rho = fabs(r1) * sqrt(top);
-      if (deflated) rho = fmax(rho, fabs(r1));
-      if (!good) rho = radius_qr<D>(omega, j, nxi, a.s);
-      // the bits of non-negative doubles order as integers; most matrices do not raise the maximum
-      unsigned long long *out = a.rho_bits + pt;
-      const unsigned long long bits = (unsigned long long)__double_as_longlong(rho);
-      if (*(volatile unsigned long long *)out < bits) atomicMax(out, bits);
+      if (good) {
+        const double rho = fabs(r1) * sqrt(top);
+        raise_radius(a.rho_bits + pt, deflated ? fmax(rho, fabs(r1)) : rho);
+      } else {
+        const unsigned long long q = atomicAdd(a.rest.count, 1ull);
+        if (q < (unsigned long long)a.rest.room) a.rest.list[q] = t;
+      }
     }
+  }
+}
+
+// The matrices that the secular equation left over, one thread each (in local memory): those on the list, or all of
+// them when the list was too short.
+template <int D>
+__global__ void __launch_bounds__(128) k_stability_qr(const __grid_constant__ StabilityArgs a) {
+  const int64_t n = (int64_t)*a.rest.count, total = a.npoints * a.nper;
+  const bool listed = n <= a.rest.room;
+  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < (listed ? n : total); q += (int64_t)gridDim.x * blockDim.x) {
+    int j[D];
+    const int64_t pt = matrix_of(a, listed ? a.rest.list[q] : q, j);
+    raise_radius(a.rho_bits + pt, radius_qr<D>(a.omega + pt * Lattice<D>::Q, j, a.nxi, a.s));
   }
 }
 
@@ -457,7 +492,7 @@ cudaError_t stability_dg(const StabilityArgs &a, cudaStream_t st) {
 }
 
 template <int D>
-cudaError_t stability_d(StabilityArgs &a, cudaStream_t st) {
+cudaError_t stability_d(StabilityArgs &a, bool rest, cudaStream_t st) {
   constexpr Lattice<D> L{};
   constexpr int Q = Lattice<D>::Q;
   for (int k = 0; k < Q; ++k)
@@ -465,6 +500,11 @@ cudaError_t stability_d(StabilityArgs &a, cudaStream_t st) {
   a.nper = a.nxi / 2 + 1;  // G(-xi) = conj G(xi): j_d <= nxi / 2 (and its partner nxi - j_d)
   if (a.nper > a.nxi) a.nper = a.nxi;
   for (int i = 0; i < D - 1; ++i) a.nper *= a.nxi;
+  if (rest) {
+    const int64_t blocks = std::min<int64_t>((a.npoints * a.nper + 127) / 128, 1 << 20);
+    k_stability_qr<D><<<(unsigned)blocks, 128, 0, st>>>(a);
+    return cudaGetLastError();
+  }
   const int poles = std::min(Q, a.nxi % 2 ? 2 * a.nxi : a.nxi);
   if constexpr (Q > 16)
     if (poles > 16) return stability_dg<D, 32>(a, st);
@@ -475,8 +515,8 @@ cudaError_t stability_d(StabilityArgs &a, cudaStream_t st) {
 
 }  // namespace
 
-cudaError_t launch_stability(int d, const double *omega_dev, int64_t npoints, int32_t nxi, double s,
-                             unsigned long long *rho_bits_dev, cudaStream_t st) {
+static cudaError_t stability(int d, const double *omega_dev, int64_t npoints, int32_t nxi, double s,
+                             unsigned long long *rho_bits_dev, const StabilityRest &r, bool rest, cudaStream_t st) {
   if (npoints <= 0) return cudaSuccess;
   StabilityArgs a{};
   a.omega = omega_dev;
@@ -484,13 +524,24 @@ cudaError_t launch_stability(int d, const double *omega_dev, int64_t npoints, in
   a.npoints = npoints;
   a.nxi = nxi;
   a.s = s;
+  a.rest = r;
   switch (d) {
-    case 1: return stability_d<1>(a, st);
-    case 2: return stability_d<2>(a, st);
-    case 3: return stability_d<3>(a, st);
-    case 4: return stability_d<4>(a, st);
+    case 1: return stability_d<1>(a, rest, st);
+    case 2: return stability_d<2>(a, rest, st);
+    case 3: return stability_d<3>(a, rest, st);
+    case 4: return stability_d<4>(a, rest, st);
     default: return cudaErrorInvalidValue;
   }
+}
+
+cudaError_t launch_stability(int d, const double *omega_dev, int64_t npoints, int32_t nxi, double s,
+                             unsigned long long *rho_bits_dev, const StabilityRest &r, cudaStream_t st) {
+  return stability(d, omega_dev, npoints, nxi, s, rho_bits_dev, r, false, st);
+}
+
+cudaError_t launch_stability_rest(int d, const double *omega_dev, int64_t npoints, int32_t nxi, double s,
+                                  unsigned long long *rho_bits_dev, const StabilityRest &r, cudaStream_t st) {
+  return stability(d, omega_dev, npoints, nxi, s, rho_bits_dev, r, true, st);
 }
 
 }  // namespace lhe
