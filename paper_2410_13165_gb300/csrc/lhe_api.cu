@@ -1019,9 +1019,7 @@ static std::vector<double> jet_weights(const lhe_lbm *l, const int16_t *jidx) {
   return out;
 }
 
-// The tables of the unknown populations (device) and the record buffer, on first use.
-static lhe_status ensure_jet_buffers(lhe_lbm *l) {
-  if (l->brec) return LHE_OK;
+static lhe_status make_jet_buffers(lhe_lbm *l) {
   const int d = l->p.d;
   std::vector<int2> links;
   links.reserve((size_t)l->nrec);
@@ -1053,6 +1051,16 @@ static lhe_status ensure_jet_buffers(lhe_lbm *l) {
 }
 
 extern "C" {
+
+// The tables of the unknown populations (device) and the record buffer, on first use.
+static lhe_status ensure_jet_buffers(lhe_lbm *l) {
+  if (l->brec) return LHE_OK;
+  try {
+    return make_jet_buffers(l);
+  } catch (const std::bad_alloc &) {
+    return fail(l, LHE_ERR_OOM, "host allocation failed");
+  }
+}
 
 lhe_status lhe_lbm_set_boundary_jet(lhe_lbm *l, const double *jet_dev) {
   if (lhe_status s = check_handle(l)) return s;
@@ -1488,8 +1496,8 @@ lhe_status lhe_lbm_adjoint_step(lhe_lbm *l, int64_t n) {
   return LHE_OK;
 }
 
-lhe_status lhe_lbm_stability_map(const lhe_lbm_params *p, const double *sigma, int64_t npoints, int32_t nxi,
-                                 double *rho_max, double *omega_min) {
+static lhe_status stability_map(const lhe_lbm_params *p, const double *sigma, int64_t npoints, int32_t nxi, double *rho_max,
+                                double *omega_min) {
   if (!p || (npoints > 0 && (!sigma || !rho_max || !omega_min))) return fail(nullptr, LHE_ERR_ARG, "NULL argument");
   const int d = p->d;
   if (d < 1 || d > 4) return fail(nullptr, LHE_ERR_ARG, "stability maps take d = 1..4");
@@ -1552,6 +1560,15 @@ lhe_status lhe_lbm_stability_map(const lhe_lbm_params *p, const double *sigma, i
   if (e1 != cudaSuccess) return cuda_fail(nullptr, e1, "stability map");
   std::memcpy(rho_max, buf.data(), sizeof(double) * (size_t)npoints);
   return LHE_OK;
+}
+
+lhe_status lhe_lbm_stability_map(const lhe_lbm_params *p, const double *sigma, int64_t npoints, int32_t nxi,
+                                 double *rho_max, double *omega_min) {
+  try {
+    return stability_map(p, sigma, npoints, nxi, rho_max, omega_min);
+  } catch (const std::bad_alloc &) {
+    return fail(nullptr, LHE_ERR_OOM, "host allocation failed");
+  }
 }
 
 lhe_status lhe_lbm_adjoint_grads(lhe_lbm *l, double *gphi0, double *ggrad, double *gR) {
