@@ -185,7 +185,10 @@ class LBM:
     def step_jets(self, jets):
         """One step per block of jets (jets: (T, P, jet_len(d)), contiguous): set_boundary_jet(jets[i]) and step(1) for
         every i in one call."""
-        T, P = int(jets.shape[0]), _abi.lhe_lbm_boundary_count(self.h)
+        T = int(jets.shape[0])
+        if T == 0:
+            return
+        P = _abi.lhe_lbm_boundary_count(self.h)
         self._stream()
         _abi.lhe_lbm_step_jets(self.h, self._ptr(jets, T * P * jet_len(self.d), "jets"), T)
 
@@ -249,7 +252,10 @@ class LBM:
     def adjoint_step_jets(self, out):
         """The reverse of step_jets: adjoint_jet_grad(out[i]) and adjoint_step(1) for i = T - 1 .. 0 in one call (out:
         (T, P, jet_len(d)), contiguous)."""
-        T, P = int(out.shape[0]), _abi.lhe_lbm_boundary_count(self.h)
+        T = int(out.shape[0])
+        if T == 0:
+            return out
+        P = _abi.lhe_lbm_boundary_count(self.h)
         self._stream()
         _abi.lhe_lbm_adjoint_step_jets(self.h, self._ptr(out, T * P * jet_len(self.d), "out"), T)
         return out
