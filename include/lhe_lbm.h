@@ -76,7 +76,7 @@ typedef enum { LHE_M4_RULE = 0, LHE_M4_EXPLICIT = 1 } lhe_m4_mode;
  * with the register-pull kernel instead of the one that stages the pulled rows in shared memory
  * by bulk asynchronous copies (both compute the same bits; the staged one is the default where
  * its layout conditions hold, n_1 a multiple of 4 and at most 512, and it is the faster one: large
- * grids whose rows fill its tiles). */
+ * grids whose rows fill its tiles; LHE_FLAG_STAGING: wherever they hold). */
 #define LHE_FLAG_NO_STAGING 1
 /* LHE_FLAG_NO_PDL: launch every step kernel with plain stream ordering. By default the second and
  * later step kernels of one lhe_lbm_step / lhe_lbm_adjoint_step call are launched with programmatic
@@ -104,6 +104,9 @@ typedef enum { LHE_M4_RULE = 0, LHE_M4_EXPLICIT = 1 } lhe_m4_mode;
  * solution, to rounding with the exact-solution family (whose data the dense form evaluates from
  * coefficients separated in time). */
 #define LHE_FLAG_NODE_BOUNDARY 8
+/* LHE_FLAG_STAGING: the staged FP32-deviation step on every periodic D3Q19 grid that its layout conditions admit, also where
+ * another kernel is faster, one step per launch (16 is not assigned). No effect with LHE_FLAG_NO_STAGING. */
+#define LHE_FLAG_STAGING 32
 
 typedef struct {
   int32_t d;              /* spatial dimension, 1..5 */

@@ -25,6 +25,7 @@ FLAG_NO_STAGING = 1
 FLAG_NO_PDL = 2
 FLAG_TEST_EXPIRE_WAIT = 4  # test hook: the first staged launch of a handle takes its wait-timeout path
 FLAG_NODE_BOUNDARY = 8
+FLAG_STAGING = 32
 
 # every entry point declared in include/lhe_lbm.h
 EXPORTS = [

@@ -117,7 +117,8 @@ lhe_status build_model(const lhe_lbm_params *p, Model &m, lhe_lbm *err_to) {
     return fail(err_to, LHE_ERR_ARG, "half-way bc_order must be 1..4");
   if (!(p->c > 0.0) || !std::isfinite(p->c)) return fail(err_to, LHE_ERR_ARG, "c must be positive");
   if (!(p->tau > 0.0) || !std::isfinite(p->tau)) return fail(err_to, LHE_ERR_ARG, "tau must be positive");
-  if (p->flags & ~(LHE_FLAG_NO_STAGING | LHE_FLAG_NO_PDL | LHE_FLAG_TEST_EXPIRE_WAIT | LHE_FLAG_NODE_BOUNDARY))
+  if (p->flags & ~(LHE_FLAG_NO_STAGING | LHE_FLAG_NO_PDL | LHE_FLAG_TEST_EXPIRE_WAIT | LHE_FLAG_NODE_BOUNDARY |
+                   LHE_FLAG_STAGING))
     return fail(err_to, LHE_ERR_ARG, "unknown bits in flags");
   if (p->m4_mode != LHE_M4_RULE && p->m4_mode != LHE_M4_EXPLICIT) return fail(err_to, LHE_ERR_ARG, "unknown m4_mode");
   if (p->m4_mode == LHE_M4_RULE && !(p->g >= 0.0 && p->g <= 1.0)) return fail(err_to, LHE_ERR_ARG, "g must be in [0, 1]");
@@ -591,26 +592,26 @@ lhe_status lhe_lbm_create(const lhe_lbm_params *p, lhe_lbm **out) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&l->sms, cudaDevAttrMultiProcessorCount, dev);
   }
-  if (p->bc == LHE_BC_PERIODIC && plan_multi(l->g, p->precision == LHE_FP32_DEV, l->sms, l->multi)) {
+  const bool stage = p->d == 3 && p->bc == LHE_BC_PERIODIC && p->precision == LHE_FP32_DEV && !(p->flags & LHE_FLAG_NO_STAGING) &&
+                     l->sms > 0 && plan_dev3_tma(l->g, l->sms, l->tma);
+  const bool force = stage && (p->flags & (LHE_FLAG_TEST_EXPIRE_WAIT | LHE_FLAG_STAGING));
+  if (p->bc == LHE_BC_PERIODIC && !force && plan_multi(l->g, p->precision == LHE_FP32_DEV, l->sms, l->multi)) {
     e = prepare_multi(p->d, p->precision == LHE_FP32_DEV, l->multi);
     if (e != cudaSuccess) return bail(cuda_fail(l, e, "shared-memory size of the multi-step kernel"));
   }
-  if (p->d == 3 && p->bc == LHE_BC_PERIODIC && p->precision == LHE_FP32_DEV && !(p->flags & LHE_FLAG_NO_STAGING)) {
-    const int sms = l->sms;
-    if (sms > 0 && plan_dev3_tma(l->g, sms, l->tma) &&
-        ((p->flags & LHE_FLAG_TEST_EXPIRE_WAIT) || staged_pays(l->tma, false) || staged_pays(l->tma, true))) {
-      e = cudaHostAlloc((void **)&l->tma_err_host, sizeof(int32_t), cudaHostAllocMapped);
-      if (e != cudaSuccess) return bail(cuda_fail(l, e, "cudaHostAlloc(pipeline flag)"));
-      *l->tma_err_host = 0;
-      e = cudaHostGetDevicePointer((void **)&l->tma.err, l->tma_err_host, 0);
-      if (e != cudaSuccess) return bail(cuda_fail(l, e, "cudaHostGetDevicePointer(pipeline flag)"));
-      e = prepare_dev3_tma();
-      if (e != cudaSuccess) return bail(cuda_fail(l, e, "shared-memory size of the staged step"));
-      const bool hook = (p->flags & LHE_FLAG_TEST_EXPIRE_WAIT) != 0;
-      l->staged[0] = hook || staged_pays(l->tma, false);
-      l->staged[1] = hook || staged_pays(l->tma, true);
-      l->tma_expire_armed = (p->flags & LHE_FLAG_TEST_EXPIRE_WAIT) != 0;
-    }
+  if (stage) {
+    l->staged[0] = force || staged_pays(l->tma, false);
+    l->staged[1] = force || staged_pays(l->tma, true);
+  }
+  if (l->staged[0] || l->staged[1]) {
+    e = cudaHostAlloc((void **)&l->tma_err_host, sizeof(int32_t), cudaHostAllocMapped);
+    if (e != cudaSuccess) return bail(cuda_fail(l, e, "cudaHostAlloc(pipeline flag)"));
+    *l->tma_err_host = 0;
+    e = cudaHostGetDevicePointer((void **)&l->tma.err, l->tma_err_host, 0);
+    if (e != cudaSuccess) return bail(cuda_fail(l, e, "cudaHostGetDevicePointer(pipeline flag)"));
+    e = prepare_dev3_tma();
+    if (e != cudaSuccess) return bail(cuda_fail(l, e, "shared-memory size of the staged step"));
+    l->tma_expire_armed = (p->flags & LHE_FLAG_TEST_EXPIRE_WAIT) != 0;
   }
   *out = l;
   return LHE_OK;
