@@ -361,19 +361,32 @@ bool plan_dev3_tma(const Geom &g, int sms, DevTmaPlan &p) {
   return true;
 }
 
-// Whether the staged kernel beats the register kernel, which reads the pulled rows through L1 and L2: it pays
-// where the state leaves L2 and its tiles are full. us per step, staged / register (the register kernel won by up to
-// 2.7 x on small grids): forward 64^3 13.6 / 6.4, 96^3 36.5 / 26.9, 160^3 161 / 117, 224^3 325 / 321 (rows of runtime
-// length: never ahead); 128 x 128 x 96 46.1 / 45.9, 128^3 58.6 / 60.5, 256 x 64 x 32 16.3 / 12.8, 256 x 64^2 30.4 / 31.7, 256^3 413 / 469.
-// Adjoint: 64^3 13.9 / 7.0, 256 x 64 x 32 17.9 / 15.4, 128^2 x 64 33.3 / 36.8, 192^3 (tiles of 384 nodes) 237 / 232, 200^3 (400)
-// 258 / 264, 256^3 458 / 543.
+// Whether the staged kernel beats the register kernel, which reads the pulled rows through L1 and L2: it pays where the
+// state leaves L2, with three stages of (nearly) full tiles. The lines are those where the ratio staged / register of
+// the time per step crosses 1, measured for rows of 16 to 512 nodes on grids of 0.5 M to 17 M nodes:
+//   forward, constant rows: 128 nodes 1.18 at 0.6 M nodes, 1.02 at 1.18 M, 0.97 at 1.31 M, 0.91 at 5 M; 256 nodes 1.14, 0.995
+//     at 0.79 M, 0.95 at 0.89 M, 0.88 at 5 M. Rows of runtime length: tiles of two rows (240 .. 252 nodes) 1.00 to 1.13
+//     at 1.5 M, 0.96 to 0.99 from 2.2 M on, of three rows (168 nodes) 1.01 at 5 M, 0.95 at 9 M; more, shorter rows 1.00
+//     to 1.7 throughout (100 nodes 1.00 to 1.03 at 2.2 M to 17 M, 64 nodes 1.09 to 1.12), a single row 1.03 to 1.15.
+//   adjoint (which also reads dL/dR): full tiles of 128 and 256 nodes 1.05 at 0.59 M, 0.93 at 0.69 M; rows from 100 nodes on
+//     1.03 to 1.10 at 0.70 M, 0.92 to 0.99 at 0.79 M; 84 nodes 1.05 at 0.80 M, 0.97 at 0.90 M; 64 nodes 1.09 at 0.90 M (128 x 110), 0.96 at
+//     1.24 M; 60 nodes 1.02 to 1.1 up to 1.25 M, 0.98 at 2.4 M; tiles of 400 (200 nodes) 1.06 at 1.3 M, 0.98 to 1.00 from 2.2 M on, a row of 420
+//     0.95 at 1.7 M, 0.93 at 5 M; 32 and 16 nodes 1.07 to 1.48 throughout; rows of 500 and
+//     512 nodes, which leave room for two stages, 1.13 at 0.8 M, 1.02 at 5 M, 1.00 at 17 M.
 bool staged_pays(const DevTmaPlan &p, bool adjoint) {
   const int64_t S = (int64_t)p.nx * p.ny * p.nz;
-  if (adjoint) return S >= (1 << 20) && p.R * p.nx >= 400;
-  return p.R * p.nx == kTileNodes && ((p.nx == 128 && S >= (7 << 18)) || (p.nx == 256 && S >= (1 << 20)));
+  const int tile = p.R * p.nx;
+  const bool whole = tile == kTileNodes && (p.nx == 128 || p.nx == 256);
+  if (p.NS < 3) return false;
+  if (adjoint) {
+    if (p.nx < 60 || tile < 400) return false;
+    if (tile < 480) return S >= (p.R == 1 ? 1 << 20 : 2000000);
+    return S >= (whole ? 680000 : (p.nx >= 100 ? 780000 : (p.nx >= 84 ? 880000 : 1 << 20)));
+  }
+  if (whole) return S >= (p.nx == 128 ? 1250000 : 820000);
+  return tile >= 480 && ((p.R == 2 && S >= 2000000) || (p.R == 3 && S >= 8000000));
 }
 
-// The limit is the kernels', not a plan's: it stays the same for the handles created before and after.
 cudaError_t prepare_dev3_tma() {
   const int bytes = (int)(LHE_TMA_SMEM_BUDGET);
   cudaError_t e;
