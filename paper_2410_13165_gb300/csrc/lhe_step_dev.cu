@@ -33,12 +33,13 @@ template <int D>
 constexpr int dev_min_blocks() { return D == 4 ? 5 : (D == 5 ? 3 : 1); }
 
 // When the next kernel of the chain may be scheduled (lhe_device.cuh).
-constexpr int kTrigStores = 0, kTrigEnd = 2;
+constexpr int kTrigStores = 0, kTrigEntry = 1, kTrigEnd = 2;
 
 template <int D, bool ADJ, bool INTERIOR, bool S2, int TRIG>
 __global__ void __launch_bounds__(LHE_STEP_THREADS, dev_min_blocks<D>()) k_step_dev(const StepArgs a) {
   constexpr Lattice<D> L{};
   constexpr int Q = Lattice<D>::Q;
+  if constexpr (TRIG == kTrigEntry) pdl_trigger();
   pdl_wait();
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= a.nwork) return;
@@ -104,6 +105,11 @@ static cudaError_t launch_step_dev_t(const StepArgs &a, cudaStream_t st) {
     int64_t inner = 1;
     for (int i = 0; i < D; ++i) inner *= a.g.n[i] - 2;
     if (a.g.S - inner > (int64_t)a.sms * 4 * 32) return launch_step_dev_trig<D, ADJ, INTERIOR, kTrigEnd>(a, st);
+  } else if constexpr (D >= 4) {
+    // D4Q33 and D5Q51 in many waves, before the stores / on entry: 24^4 15.1 / 14.7, 32^4 50.7 / 50.1, 48^4 249.7 / 247.5, adjoint 269.8 /
+    // 267.7; 24^5 597.0 / 595.8, adjoint 624 / 620. Smaller grids the other way: 16^4 4.2 / 4.9, 8^5 3.8 / 4.5, 12^5 adjoint 20.1 / 20.3; and 2D and 3D,
+    // 1150^2 18.8 / 19.2.
+    if (a.nwork >= (D == 4 ? 250000 : 500000)) return launch_step_dev_trig<D, ADJ, INTERIOR, kTrigEntry>(a, st);
   }
   return launch_step_dev_trig<D, ADJ, INTERIOR, kTrigStores>(a, st);
 }
