@@ -371,7 +371,7 @@ bool plan_dev3_tma(const Geom &g, int sms, DevTmaPlan &p) {
 //   adjoint (which also reads dL/dR): full tiles of 128 and 256 nodes 1.05 at 0.59 M, 0.93 at 0.69 M; rows from 100 nodes on
 //     1.03 to 1.10 at 0.70 M, 0.92 to 0.99 at 0.79 M; 84 nodes 1.05 at 0.80 M, 0.97 at 0.90 M; 64 nodes 1.09 at 0.90 M (128 x 110), 0.96 at
 //     1.24 M; 60 nodes 1.02 to 1.1 up to 1.25 M, 0.98 at 2.4 M; tiles of 400 (200 nodes) 1.06 at 1.3 M, 0.98 to 1.00 from 2.2 M on, a row of 420
-//     0.95 at 1.7 M, 0.93 at 5 M; 32 and 16 nodes 1.07 to 1.48 throughout; rows of 500 and
+//     0.95 at 1.7 M, 0.93 at 5 M, of 384 1.00 at 5 M, 0.98 from 6.3 M on; 32 and 16 nodes 1.07 to 1.48 throughout; rows of 500 and
 //     512 nodes, which leave room for two stages, 1.13 at 0.8 M, 1.02 at 5 M, 1.00 at 17 M.
 bool staged_pays(const DevTmaPlan &p, bool adjoint) {
   const int64_t S = (int64_t)p.nx * p.ny * p.nz;
@@ -379,6 +379,7 @@ bool staged_pays(const DevTmaPlan &p, bool adjoint) {
   const bool whole = tile == kTileNodes && (p.nx == 128 || p.nx == 256);
   if (p.NS < 3) return false;
   if (adjoint) {
+    if (p.R == 1 && p.nx >= 384 && p.nx < 400) return S >= 6000000;
     if (p.nx < 60 || tile < 400) return false;
     if (tile < 480) return S >= (p.R == 1 ? 1 << 20 : 2000000);
     return S >= (whole ? 680000 : (p.nx >= 100 ? 780000 : (p.nx >= 84 ? 880000 : 1 << 20)));

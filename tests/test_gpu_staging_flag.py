@@ -53,6 +53,20 @@ def test_staged_everywhere_is_bitwise_the_other_kernels(n, tau, source):
             assert torch.equal(a, b)
 
 
+# nodes on either side of the lines of the default choice: forward 0.82 M (rows of 256), 1.25 M (128), 2 M (two rows a tile); adjoint
+# 0.68 M (256), 0.78 M (100), 0.88 M (84), 1.05 M (60), 2 M (tiles of 400), and two stages only (512)
+@pytest.mark.parametrize("n", [(256, 64, 50), (256, 64, 51), (128, 96, 101), (128, 96, 102), (240, 90, 92), (240, 90, 94), (256, 52, 51), (256, 52, 52),
+                               (100, 80, 97), (100, 80, 98), (84, 96, 109), (84, 96, 110), (60, 128, 136), (60, 128, 137), (200, 100, 99),
+                               (200, 100, 101), (512, 50, 42), (384, 30, 28)])
+def test_the_default_choice_does_not_show(n):
+    import torch
+
+    rng = np.random.default_rng(sum(n))
+    data = [torch.from_numpy(rng.standard_normal(int(np.prod(n)))).cuda() for _ in range(3)]
+    for a, b in zip(_run(n, 0.8, data, [2]), _run(n, 0.8, data, [2], staged=False)):
+        assert torch.equal(a, b)
+
+
 def test_staged_small_grid_matches_the_oracle():
     import torch
 
