@@ -443,10 +443,10 @@ static int boundary_threads(int64_t nodes, int sms) {
   return nodes <= (int64_t)sms * 4 * 32 ? 32 : (nodes <= (int64_t)sms * 8 * 64 ? 64 : 128);
 }
 
-// How the kernels of one box are launched. FP32 deviations, us per step before there was an early form / early up to 40,000 nodes,
-// more than a wave in D4Q33, and beside the rows' last wave / now (lhe_step_dev.cu), full-way and its adjoint: D4Q33 18^4 (39,440 nodes)
-// 50 / 63 / 45 and 41 / 33 / 30, 19^4 56 / 62 / 49 and 41 / 47 / 32, 22^4 (74,256) 76 / 78 / 73 and 56 / 60 / 52, 24^4 (97,520) 109 / 106 / 106 and 79 / 76 / 76;
-// D3Q19 90^3 (47,528) 55 / 49 / 49 and 45 / 40 / 40.
+// How the kernels of one box are launched. FP32 deviations, us per step before there was an early form / early up to 40,000
+// nodes, more than a wave in D4Q33, and beside the rows' last wave / now (lhe_step_dev.cu), full-way and its adjoint:
+// D4Q33 18^4 (39,440 nodes) 50 / 63 / 45 and 41 / 33 / 30, 19^4 56 / 62 / 50 and 41 / 47 / 32, 22^4 (74,256) 76 / 78 / 73 and
+// 56 / 60 / 52, 24^4 (97,520) 109 / 106 / 106 and 79 / 76 / 76; D3Q19 90^3 (47,528) 55 / 49 / 49 and 45 / 40 / 40.
 struct NodeLaunch {
   bool early;
   int threads;

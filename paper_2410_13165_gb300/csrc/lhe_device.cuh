@@ -301,7 +301,7 @@ __device__ __forceinline__ void st_stream(float *p, float v) { *p = v; }
 // before the stores / at the end: FP64 D2Q9 256^2 5.93 / 3.93 / 3.66, 500 x 333 (8.6 CTAs per SM) 7.16 / 6.76 / 6.01,
 // 1000^2 (51) 23.7 / 23.4 / 25.3, D3Q19 32^3 8.94 / 4.86 / 4.03, 45 x 37 x 51 9.52 / 8.12 / 6.87, 64^3 (13.5) 13.5 / 13.5 / 14.0;
 // 128^3 and larger the same (the adjoint, which also updates dL/dR, is faster with the trigger at the end at every size:
-// 64^3 13.7 / 13.3, 128^3 100.4 / 99.2); FP32 deviations the same before the stores and at the end. (A run-time choice in
+// 64^3 13.7 / 13.3, 128^3 100.4 / 99.2); FP32 deviations: lhe_step_dev.cu. (A run-time choice in
 // one kernel measured like the trigger at the end everywhere, so the two are separate instantiations.)
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

@@ -250,9 +250,9 @@ __device__ __forceinline__ cd rcp(cd a) {
 // Weights above 1e6 and ones that are not finite go there at once: FP32 cannot hold their products.
 // A group of G lanes holds a matrix, a lane a root (two for the 33rd pole of D = 4); G is the smallest of 8, 16
 // and 32 that holds the poles, of which there are at most nxi (nxi even) or 2 nxi. G(-xi) is the conjugate of G(xi), so half
-// of the last axis is visited. Bound by the FP64 pipe (~70 % busy: S in the last two iterations, the poles' sines). Against roots
+// of the last axis is visited. Bound by the FP64 pipe (85 % busy: S in the last two iterations, the poles' sines). Against roots
 // refined in 80 bits (600 random D3Q19 matrices) the radius is within 6e-15, LAPACK's QR within 3e-14. 24 velocities of D3Q19,
-// 12^3 Fourier variables: 29.2 ms by QR (one thread per matrix, in local memory) -> 0.53 ms; the whole call takes 0.04 ms more.
+// 12^3 Fourier variables: 29.2 ms by QR (one thread per matrix, in local memory) -> 0.50 ms; the whole call takes 0.55.
 // (D4Q33 in groups of 8 on at least five CTAs an SM: at 114 registers and four it took a tenth longer. 0 leaves the others alone.)
 template <int D, int G>
 __global__ void __launch_bounds__(128, D == 4 && G == 8 ? 5 : 0) k_stability(const __grid_constant__ StabilityArgs a) {
