@@ -67,6 +67,21 @@ def test_weights_beyond_the_stable_range(d, nxi, tau, size):
             assert abs(rho[p] - want) <= 64 * 2.0 ** -53 * norm * cond, (S[p], rho[p], want, cond)
 
 
+@pytest.mark.parametrize("copies", [1, 300, 1100])
+def test_leftover_matrices_one_by_one_and_in_numbers(copies):
+    """One matrix of these velocities' is left to the QR route: on the list of such matrices, on a longer one, and among more of
+    them than the list holds (when all matrices take the route)."""
+    rng = np.random.default_rng(42)
+    S = rng.uniform(-0.6, 0.6, (6, 2))
+    S[0], S[1], S[2], S[3] = 0.0, 0.5, 0.1, 0.5 - 1e-7
+    S[1, 1:] = 0.0
+    rho, _ = stability_map(2, np.tile(S, (copies, 1)), 9)
+    for p in range(len(S)):
+        want, cond, norm = _reference(2, S[p], 9, 0.5)
+        tol = min(64 * 2.0 ** -53 * norm * cond, 8 * 2.0 ** -26.5 * max(1.0, want))
+        assert np.all(np.abs(rho[p::6] - want) <= tol), (S[p], rho[p], want, cond)
+
+
 @pytest.mark.parametrize("m4", [float("nan"), float("inf")])
 @pytest.mark.parametrize("tau", [0.5, 1.0])
 def test_weights_that_are_not_finite_are_not_stable(tau, m4):
